@@ -87,11 +87,22 @@ __device__ __forceinline__ uint4 edge2_reduce(unsigned long long reduce_sum_mask
   return make_uint4(res[0], res[1], res[2], res[3]);
 }
 
+// 16-byte chunks a lane has in flight while it moves rows of run-time widths: as many loads as a warp of the tuned
+// variants keeps (16 + 4).  592-byte rows, 37 x 17,003 candidates: one chunk at a time with a division per chunk
+// 198 us, 8 / 12 / 16 / 20 / 24 in flight 142 / 137 / 133 / 123 / 132 us; batches of equal length (13 + 12 + 12 chunks
+// of 37 instead of 20 + 17) 138 us.  Second-degree joins and
+// the cosine section keep more beside the loads and have the registers for 8.
+constexpr int kGenericUnroll = 20;
+constexpr int kGenericUnrollSecond = 8;
+
 // Section widths of a launch, in 16-byte chunks and bytes (compile-time where the variant fixes them).
 template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, bool COS = false>
 struct RowShape {
   int doc_ch, edge_ch, req_ch, doc_b, edge_b, req_b;
   long long out_b;
+  // run-time widths: chunks of a row that are loaded as they are, the (row, chunk) of this lane's first one in a group
+  // and the step to the one 32 chunks further
+  int src_ch, lane_row, lane_piece, step_row, step_piece;
   __device__ __forceinline__ explicit RowShape(const JoinArgs& a) {
     doc_ch = DOC_CH ? DOC_CH : a.doc_ch;
     edge_ch = EDGE_CH ? EDGE_CH : a.edge_ch;
@@ -100,6 +111,12 @@ struct RowShape {
     edge_b = edge_ch * 16;
     req_b = req_ch * 16;
     out_b = doc_b + edge_b * (SECOND ? 2 : 1) + req_b + (COS ? kCosSectionBytes : 0);
+    src_ch = doc_ch + edge_ch + req_ch;
+    const int lane = threadIdx.x & 31;
+    lane_row = lane / src_ch;
+    lane_piece = lane - lane_row * src_ch;
+    step_row = 32 / src_ch;
+    step_piece = 32 - step_row * src_ch;
   }
 };
 
@@ -288,23 +305,50 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
       if (row < cnt) st128_stream(out + row * out_b + DOC_CH * 16 + piece * 16, ev[i]);
     }
   } else {
-    for (int i = 0; i < sh.doc_ch; ++i) {
-      const int c = i * 32 + lane, row = c / sh.doc_ch, piece = c - row * sh.doc_ch;
-      const int ridx = row < cnt ? s_idx[row] : -1;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (ridx >= 0) v = ldg128_once(a.doc_feats + static_cast<long long>(ridx) * sh.doc_b + piece * 16);
-      if (row < cnt) st128_stream(out + row * out_b + piece * 16, v);
-      if constexpr (kCos) {
-        const int q = piece - p0;
-        if (q >= 0 && q < np) stage[row * sstride + q] = v;
+    // Run-time widths.  The loaded chunks of the rows (document, edge and request sections taken as one run of
+    // sh.src_ch chunks per row) are walked U x 32 at a time, every load of a batch in front of its first store; a lane
+    // steps by additions (32 chunks further = sh.step_row rows and sh.step_piece chunks, with a carry).  All sections
+    // share one load instruction: a second one under the opposite predicate (document rows past L1) writes the same
+    // registers and so waits for the first to return, which serialised the batch (321 us where this takes 123 us).
+    constexpr int U = (SECOND || kCos) ? kGenericUnrollSecond : kGenericUnroll;
+    constexpr bool kLinear = !SECOND && !kCos;  // the chunks leave in the order they are walked: consecutive lanes, consecutive chunks
+    const int edge_end = sh.doc_ch + sh.edge_ch, n_chunks = cnt * sh.src_ch;
+    int row = sh.lane_row, piece = sh.lane_piece;
+    for (int i0 = 0; i0 < sh.src_ch; i0 += U) {
+      uint4 v[U];
+      [[maybe_unused]] int at[U];           // where the chunk goes in the group's output
+      [[maybe_unused]] int at_stage[U];     // ... in the embedding staging block; < 0 = not part of the embedding
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (!kLinear) at[u] = 0;
+        if constexpr (kCos) at_stage[u] = -1;
+        if ((i0 + u) * 32 + lane < n_chunks) {
+          const bool is_doc = piece < sh.doc_ch, is_edge = !is_doc && piece < edge_end;
+          const int src_row = is_doc ? s_idx[row] : (is_edge ? s_pos[row] : 0);
+          const uint8_t* base = is_doc ? a.doc_feats : (is_edge ? edge_base : req_src);
+          const int width = is_doc ? sh.doc_b : sh.edge_b, first = is_doc ? 0 : (is_edge ? sh.doc_ch : edge_end);
+          if (src_row >= 0) v[u] = ldg128(base + static_cast<long long>(src_row) * width + (piece - first) * 16);
+          if constexpr (!kLinear) at[u] = row * static_cast<int>(out_b) + (piece + (SECOND && piece >= edge_end ? sh.edge_ch : 0)) * 16;
+          if constexpr (kCos) {
+            if (is_doc && piece >= p0 && piece < p0 + np) at_stage[u] = row * sstride + (piece - p0);
+          }
+        }
+        row += sh.step_row;
+        piece += sh.step_piece;
+        if (piece >= sh.src_ch) {
+          piece -= sh.src_ch;
+          ++row;
+        }
       }
-    }
-    for (int i = 0; i < sh.edge_ch; ++i) {
-      const int c = i * 32 + lane, row = c / sh.edge_ch, piece = c - row * sh.edge_ch;
-      const int rpos = row < cnt ? s_pos[row] : -1;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (rpos >= 0) v = ldg128(edge_base + static_cast<long long>(rpos) * sh.edge_b + piece * 16);
-      if (row < cnt) st128_stream(out + row * out_b + sh.doc_b + piece * 16, v);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int c = (i0 + u) * 32 + lane;
+        if (c < n_chunks) st128_stream(out + (kLinear ? c * 16 : at[u]), v[u]);
+        if constexpr (kCos) {
+          if (at_stage[u] >= 0) stage[at_stage[u]] = v[u];
+        }
+      }
     }
   }
   // edge2 section: the matched rows of the found engager slots, reduced per dim in slot order
@@ -329,8 +373,8 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
       if (row < cnt) st128_stream(out + row * out_b + sh.doc_b + sh.edge_b + piece * 16, v);
     }
   }
-  // request section: one source row for the whole request (L1/L2 hits)
-  if (sh.req_ch) {
+  // request section: one source row for the whole request (L1/L2 hits); run-time widths have stored it above
+  if constexpr (DOC_CH > 0 && EDGE_CH > 0 && REQ_CH > 0) {
     const int off = sh.doc_b + sh.edge_b * (SECOND ? 2 : 1);
     for (int i = 0; i < sh.req_ch; ++i) {
       const int c = i * 32 + lane, row = c / sh.req_ch, piece = c - row * sh.req_ch;
