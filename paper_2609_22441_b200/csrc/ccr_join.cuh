@@ -172,12 +172,12 @@ __device__ __forceinline__ int block_lower_bound(const int64_t* g, int K, int64_
 // Shared-memory layout of join_kernel, shared by host (sizing) and device (carving).
 struct TileLayout {
   int off_idx, off_pos, off_apos, off_auth, off_keys, bytes;
-  __host__ __device__ TileLayout(int tile, bool second, bool merge, int search_area) {
+  __host__ __device__ TileLayout(int tile, bool second, bool merge, int search_area) {  // (author ids: merge mode and the stash of the first sub-tile)
     off_idx = kSmemHeader;
     off_pos = off_idx + tile * 4;
     off_apos = off_pos + tile * 4;
     off_auth = off_apos + (second ? tile * 16 : 0);
-    off_keys = off_auth + (merge ? tile * 8 : 0);
+    off_keys = off_auth + tile * 8;
     off_keys = (off_keys + 15) & ~15;
     bytes = off_keys + search_area;
   }
@@ -424,14 +424,42 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
   }
   __syncthreads();
   uint32_t phase = 0;
+  pdl_trigger();  // a join launched behind this one may move in as blocks leave; it stores nothing before this one is done
 
   // this block's contiguous slice of the flat candidate range, in whole groups of 32
   const long long groups = (a.total + 31) >> 5;
   const long long per = (groups + gridDim.x - 1) / gridDim.x;
   const long long j0 = min(a.total, static_cast<long long>(blockIdx.x) * per * 32);
   const long long j1 = min(a.total, j0 + per * 32);
-  if (j0 >= j1) return;
-  int r = request_of(a.cand_offsets, a.n_req, j0);
+  if (j0 >= j1) {
+    pdl_wait();  // (a launch never completes before the one in front of it)
+    return;
+  }
+  // The positions and author ids of the first sub-tile do not depend on the request they belong to: they are fetched
+  // here, beside the offsets and the staging of the keys, and kept in the thread's own slots of the resolved arrays.
+  if (!MERGE) {
+    // (padded output: a.total may be an upper bound, the list ends where the last request does)
+    const long long j_lim = PADDED ? min(j1, static_cast<long long>(gload(a.cand_offsets + a.n_req))) : j1;
+    const int n0 = static_cast<int>(min(static_cast<long long>(a.tile), max(j_lim - j0, 0LL)));
+    for (int base = 0; base < n0; base += kThreads * kUnroll) {
+      int idx[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const int i = base + u * kThreads + tid;
+        idx[u] = i < n0 ? gload(a.cand_idx + j0 + i) : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const int i = base + u * kThreads + tid;
+        if (i < n0) {
+          if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
+          s_idx[i] = idx[u];
+          s_auth[i] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
+        }
+      }
+    }
+  }
+  int r = a.n_req == 1 ? 0 : request_of(a.cand_offsets, a.n_req, j0);
 
   long long seg = j0;
   while (seg < j1 && r < a.n_req) {
@@ -467,15 +495,24 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
         for (int base = 0; base < n; base += kThreads * kUnroll) {
           int idx[kUnroll];
           int64_t auth[kUnroll];
+          if (sub == j0) {  // fetched above
 #pragma unroll
-          for (int u = 0; u < kUnroll; ++u) {
-            const int i = base + u * kThreads + tid;
-            idx[u] = i < n ? gload(a.cand_idx + sub + i) : -1;
-          }
+            for (int u = 0; u < kUnroll; ++u) {
+              const int i = base + u * kThreads + tid;
+              idx[u] = i < n ? s_idx[i] : -1;
+              auth[u] = i < n ? s_auth[i] : -1;
+            }
+          } else {
 #pragma unroll
-          for (int u = 0; u < kUnroll; ++u) {
-            if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
-            auth[u] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
+            for (int u = 0; u < kUnroll; ++u) {
+              const int i = base + u * kThreads + tid;
+              idx[u] = i < n ? gload(a.cand_idx + sub + i) : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+              if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
+              auth[u] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
+            }
           }
           bool found[kUnroll];
           int pos[kUnroll];
@@ -492,6 +529,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
               pos[h + q] = p4[q];
             }
           }
+          pdl_wait();  // the first store is about to be made
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u) {
             const int i = base + u * kThreads + tid;
@@ -526,6 +564,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
           }
         }
       } else {
+        pdl_wait();
         // 1. author ids of the sub-tile
         int bad = 0;
         for (int base = 0; base < n; base += kThreads * kUnroll) {
@@ -612,6 +651,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
     seg = seg_end;
     ++r;
   }
+  pdl_wait();  // also of a block that had nothing to store: a launch never completes before the one in front of it
 }
 
 }  // namespace ccr

@@ -172,7 +172,10 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   const long long per = (groups + gridDim.x - 1) / gridDim.x;
   const long long slice0 = min(a.total, static_cast<long long>(blockIdx.x) * per * 32);
   const long long slice1 = min(a.total, slice0 + per * 32);
-  if (a.sched == nullptr && slice0 >= slice1) return;  // block-uniform, before any named barrier
+  if (a.sched == nullptr && slice0 >= slice1) {  // block-uniform, before any named barrier
+    pdl_wait();  // (a launch never completes before the one in front of it)
+    return;
+  }
 
   const int n_res = (n_threads >> 5) - n_streamers;
   const int role_rank = (n_threads >> 5) - 1 - warp;  // resolvers are the last n_res warps
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0 + 8 * s);
     }
+    pdl_wait();  // also of a block that had nothing to store: a launch never completes before the one in front of it
     return;
   }
 

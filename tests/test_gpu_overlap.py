@@ -1,0 +1,51 @@
+"""Joins launched back to back on one stream may overlap on the device; whatever they leave must be what one after the
+other would leave.  Batches of different sizes are joined alternately into the SAME output buffers, with a padded join
+that has nothing to store in between, and the last state is compared byte for byte with the CPU oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2609_22441_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("second", [False, True])
+@pytest.mark.parametrize("n_req,big,small", [(1, 60_000, 40), (3, 20_000, 500), (8, 30_000, 33)])  # the last: one of each kernel
+def test_alternating_batches_into_one_buffer(n_req, big, small, second):
+    from paper_2609_22441_b200 import binding as B
+
+    wls = [W.config1(seed=5 + i, n_docs=200_000, n_req=n_req, n_cand=n, second_degree=second, edge_lo=40, edge_hi=3_000) for i, n in enumerate((big, small))]
+    wls[1].store = wls[0].store
+    wants = [oracle.join_workload(wl, n_threads=4) for wl in wls]
+    store = B.store_from_workload(wls[0])
+    dbs = [B.DeviceBatch(wl.batch) for wl in wls]
+    out_b = store.out_row_bytes(0)
+    rows = torch.zeros((dbs[0].total_cands, out_b), dtype=torch.uint8, device="cuda")
+    mask = torch.zeros(dbs[0].total_cands, dtype=torch.uint8, device="cuda")
+    # compacted offsets that keep nothing: the padded join over them stores no row of its own
+    none_kept = torch.zeros(n_req + 1, dtype=torch.int64, device="cuda")
+    T, M = (torch.zeros(s, dtype=torch.uint8, device="cuda") for s in ((n_req, 1, out_b), (n_req, 1)))
+
+    def join(db):
+        B.ccr_join_batch(store, db.n_req, db.total_cands, db.max_edge_len, db.edge_keys, db.edge_feats, db.edge_offsets, db.cand_idx,
+                         db.cand_offsets, db.req_feats, rows, mask)
+
+    def nothing(db):
+        B.ccr_join_batch_padded(store, db.n_req, db.total_cands, db.max_edge_len, 1, db.edge_keys, db.edge_feats, db.edge_offsets, db.cand_idx,
+                                none_kept, db.req_feats, T, M)
+
+    torch.cuda.synchronize()
+    for _ in range(30):
+        join(dbs[0])
+        nothing(dbs[1])
+        join(dbs[1])
+        join(dbs[0])
+        join(dbs[1])
+    torch.cuda.synchronize()
+    got_rows, got_mask, n = rows.cpu().numpy(), mask.cpu().numpy(), dbs[1].total_cands
+    assert np.array_equal(got_mask[:n], wants[1][1]) and np.array_equal(got_rows[:n], wants[1][0])
+    assert np.array_equal(got_mask[n:], wants[0][1][n:]) and np.array_equal(got_rows[n:], wants[0][0][n:])
+    assert not T.any() and store.device_status() == B.CCR_OK
+    store.free()
