@@ -1,16 +1,14 @@
 // Algorithm 1 step 1 of the paper on the device: per request, sort the viewer's affinity records by author
 // id (a_sorted, idx = sort(a); F_sorted = gather(F, idx)) so that unsorted request payloads can be joined.
 //
-// The order is on (key, index of the record in its list), which makes the result the stable sort.  Keys that leave
-// room for the index in the same 64-bit word (the usual case) are sorted as single words, key << bits | index.
-// With a permutation output the lists are cut into chunks of 4,096 records, one block sorts a chunk in shared
-// memory (a merge sort: four words per thread in registers, then runs doubled per pass along merge paths), the
-// sorted chunks are merged pairwise by grid-wide launches (merge path again, one output tile per block), and the
-// rows follow their keys in one grid-wide gather.  Without a permutation output, or for keys that do not leave
-// room for the index, one 1024-thread block sorts a whole list in shared memory (merge sort up to 16,384 packed
-// words, a bitonic network written for arbitrary n beyond that and for the 12-byte (key, index) records of
-// unpackable keys; lists that do not fit shared memory are sorted by the network on the output arrays in L2) and
-// moves its rows itself.
+// The order is on (key, index of the record in its list), which makes the result the stable sort.  Lists of up to
+// kListMax records (every batch whose length bound says so) are radix sorted in shared memory, one cluster of blocks per
+// list, and the rows follow in a launch of their own (short lists: in the same one); see sort_lists_kernel.  Batches with
+// longer lists are cut into chunks of 4,096 records: one block sorts a chunk as packed words, key << bits | index (a
+// merge sort: four words per thread in registers, then runs doubled per pass along merge paths), the sorted chunks
+// are merged pairwise by grid-wide launches (merge path again, one output tile per block), and the rows follow their keys
+// in one grid-wide gather.  A batch with a key that leaves no room for the index is then sorted list by list by one
+// 1024-thread block each.
 #pragma once
 
 #include "ccr_device.cuh"
@@ -309,7 +307,8 @@ __device__ __forceinline__ void gather_rows(const uint4* src, uint4* dst, long l
 }
 
 struct SortArgs {
-  int* call_flag;          // multi: device word, zero between calls; set when a key of the batch cannot share a word with its index
+  int* call_flag;          // chunked path: device word, zero between calls; set when a key of the batch cannot share a word with its index
+  int rows_here;             // sort_lists_kernel moves the rows itself
   int more_follow;           // another kernel of the same ccr_sort_edges call is launched behind this one
   int n_req;
   const int64_t* keys_in;
@@ -318,12 +317,10 @@ struct SortArgs {
   int row_ch;            // 16-byte chunks per feature row
   int64_t* keys_out;
   uint8_t* feats_out;
-  int* perm_out;         // may be null when every list fits shared memory
+  int* perm_out;         // may be null on the whole-list path
   int smem_keys;         // (key, index) records the dynamic shared memory can hold: 12 bytes each
   int smem_words;        // packed key|index words it can hold: 8 bytes each
   int max_len;           // the host's bound on the list length: longer lists are cut there (their tail is left alone)
-  int multi;             // 1: the chunked kernels sort every list (sort_edges_kernel only when a key of the batch cannot be
-                         //    packed), and the rows of every list are moved by gather_all_kernel (perm_out is then required)
 };
 
 #ifndef CCR_SORT_CHUNK_LOG
@@ -370,12 +367,9 @@ __global__ void __launch_bounds__(kSortThreads, 1) sort_edges_kernel(const SortA
   // keys that leave room for the record index in one 64-bit word (non-negative, below 2^(63 - index bits)) are
   // sorted as single words: key << shift | index orders like (key, index), needs 8 bytes per record and no
   // index array at all (the word's low bits are the index)
-  if (a.multi && gload(a.call_flag) == 0) return;  // the chunked kernels have sorted every list
+  if (gload(a.call_flag) == 0) return;  // the chunked kernels have sorted every list
   const int idx_bits = sort_index_bits(K);
   const bool packable = list_is_packable(a.keys_in + e0, K, idx_bits);
-  const long long chunks = a.multi ? 0 : static_cast<long long>(K) * a.row_ch;  // multi: rows move in gather_all_kernel
-  const uint4* src = reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch;
-  uint4* dst = reinterpret_cast<uint4*>(a.feats_out) + e0 * a.row_ch;
 
   if (packable && K <= a.smem_words) {
     unsigned long long* w = reinterpret_cast<unsigned long long*>(smem_sort);
@@ -391,14 +385,12 @@ __global__ void __launch_bounds__(kSortThreads, 1) sort_edges_kernel(const SortA
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
       const unsigned long long v = w[i];
       gstore(a.keys_out + e0 + i, v >> idx_bits);
-      if (a.perm_out) gstore(a.perm_out + e0 + i, v & low);
+      gstore(a.perm_out + e0 + i, v & low);
     }
-    gather_rows(src, dst, chunks, a.row_ch, [&](int row) { return static_cast<long long>(w[row] & low); });
     return;
   }
 
   const bool in_smem = K <= a.smem_keys;
-  if (!in_smem && a.perm_out == nullptr) return;  // refused on the host; never reached
   long long* keys = in_smem ? reinterpret_cast<long long*>(smem_sort) : reinterpret_cast<long long*>(a.keys_out + e0);
   int* idx = in_smem ? reinterpret_cast<int*>(smem_sort + static_cast<size_t>(a.smem_keys) * 8) : a.perm_out + e0;
   if (packable) {  // only reached by lists too long for shared memory: the words live in the key output array
@@ -425,10 +417,9 @@ __global__ void __launch_bounds__(kSortThreads, 1) sort_edges_kernel(const SortA
   if (in_smem) {
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
       gstore(a.keys_out + e0 + i, keys[i]);
-      if (a.perm_out) gstore(a.perm_out + e0 + i, idx[i]);
+      gstore(a.perm_out + e0 + i, idx[i]);
     }
   }
-  gather_rows(src, dst, chunks, a.row_ch, [&](int row) { return static_cast<long long>(idx[row]); });
 }
 
 
@@ -646,6 +637,293 @@ __global__ void __launch_bounds__(kSortGatherThreads) gather_all_kernel(const So
   for (int u = 0; u < kSortGatherUnroll; ++u) {
     const long long c = first + static_cast<long long>(u) * kSortGatherThreads + threadIdx.x;
     if (c < chunks) st128_stream(dst + c, v[u]);  // written once, read by a later kernel at the earliest
+  }
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Whole lists by radix sort, one cluster of blocks each: lists of up to kListBlockMax records per block of the cluster.
+// A record's word is what its key has behind the list's common prefix, above the record's index in the list.  The words
+// are sorted by the bits that differ anywhere in the list, seven a pass and lowest first (stable, so equal keys keep
+// their order); a digit that is the same throughout costs nothing.  Between the passes the words are in registers: a
+// warp owns 32 * R consecutive ones (R = words per thread this list needs), counts its digits, a scan over (digit, block,
+// warp) turns the counts into places, and the warp hands its words out in order — into the shared memory of the block
+// that owns the place — the lanes that share a digit found with one ballot per digit bit.  Keys whose differing bits
+// leave no room for the index (the far outlier of a clustered list is enough) are sorted in two rounds: by their low 32
+// bits, then by the rest.
+// A pass is bound by instruction issue (about 50 instructions a word and pass; over 20,000 words on one SM 11 us), hence
+// the cluster: a list takes as many blocks as hold it, the others of its cluster leave at once.  Blocks of up to 4,096
+// records each, 3 resident per SM at 80 registers: with 1,024 / 2,048 / 3,072 wanted per block the 256-list batch below
+// takes 104 / 100 / 97 us instead of 94 (cluster barriers and blocks that leave at once), a single list of 20,000 31
+// instead of 34; __match_any_sync for the ballots 99; 64 registers, 4 resident 96.
+// Lists of up to kListNetwork records have too few words for the passes to pay: sorted by sort_words_merge128 instead (256
+// lists of 900-1,000 records, 2^40 keys: 37 -> 29 us; one list of 200 records 12.9 -> 9.7 us).
+// 256 lists <= 20,000 (700,000 records of 128-byte rows): 141 us as chunks and merges, 90 us this way; 4 such lists
+// 38.7 -> 29 us; 64 lists <= 5,000 in the request flow 37 -> 27 us; 4 lists <= 9,214 with a far outlier each 145 -> 82 us.
+constexpr int kListRadixBits = 7, kListDigits = 1 << kListRadixBits;
+constexpr int kListStride = kListDigits + 1;  // counters of a warp; odd, so that the scan's column reads spread over the banks
+constexpr int kListThreads = 256, kListPer = 16, kListWarps = kListThreads / 32;
+constexpr int kListBlockMax = kListThreads * kListPer;  // 4,096 words of a block: 32 registers of a thread
+constexpr int kListNetwork = 1024;  // lists up to this length are sorted as one block's merge sort behind a register network
+constexpr int kListRowsHere = 512;  // batches of lists up to this length move their rows in the sorting kernel
+static_assert(kListNetwork <= 4 * kListThreads, "sort_words_merge128 takes four words a thread");
+constexpr int kListMaxCluster = 8;                      // the portable size
+constexpr int kListMax = kListBlockMax * kListMaxCluster;
+static_assert(kListDigits * kListWarps == 4 * kListThreads, "in the scan a thread has four warps' counters of one digit");
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Barrier over the blocks of the cluster that are still running, with their shared-memory writes made visible.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t smem, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_ld32(uint32_t addr) {
+  unsigned v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_st64(uint32_t addr, unsigned long long v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortArgs a) {
+  chain_enter(a.more_follow != 0);
+  __shared__ unsigned long long w[kListBlockMax];
+  __shared__ unsigned cnt[kListWarps * kListStride];       // [warp][digit]
+  __shared__ unsigned block_count[kListDigits];            // this block's words with each digit, read by the whole cluster
+  __shared__ unsigned digit_base[kListDigits];             // place of this block's first word with each digit
+  __shared__ unsigned warp_total[kListWarps], or_bits[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int cs = static_cast<int>(cluster_size()), rank = static_cast<int>(cluster_rank());
+  const int list = blockIdx.x / cs;
+  const long long e0 = gload(a.edge_offsets + list);
+  const long long Kl = min(static_cast<long long>(gload(a.edge_offsets + list + 1) - e0), static_cast<long long>(a.max_len));
+  if (Kl <= 0) return;
+  const int K = static_cast<int>(Kl);
+  const int blocks = min(cs, (K + kListBlockMax - 1) / kListBlockMax);
+  const int R = (K + blocks * kListThreads - 1) / (blocks * kListThreads), per = R * kListThreads;  // words per thread, per block
+  const int n = min(per, K - rank * per);  // words of this block
+  if (rank >= blocks || n <= 0) return;    // (nobody reads the shared memory of a block without words)
+  const int used_blocks = (K + per - 1) / per;
+  auto sync_all = [&]() {
+    if (used_blocks > 1) cluster_sync();
+    else __syncthreads();
+  };
+  const int first = warp * 32 * R + lane;  // word r of this thread: first + 32 * r of the block's
+  const int64_t* keys = a.keys_in + e0;
+  const unsigned per_inv = 0xffffffffu / static_cast<unsigned>(per) + 1u;  // place / per for places below 2^16: exact
+
+  constexpr unsigned long long kSign = 0x8000000000000000ull;  // signed keys as unsigned words of the same order
+  const unsigned long long key0 = static_cast<unsigned long long>(gload(keys)) ^ kSign;
+  unsigned long long v[kListPer];
+  unsigned lo = 0, hi = 0;
+  if (threadIdx.x < 2) or_bits[threadIdx.x] = 0u;
+#pragma unroll
+  for (int r = 0; r < kListPer; ++r) {
+    v[r] = key0;
+    if (r < R && first + 32 * r < n) v[r] = static_cast<unsigned long long>(gload(keys + rank * per + first + 32 * r)) ^ kSign;
+    lo |= static_cast<unsigned>(v[r] ^ key0);
+    hi |= static_cast<unsigned>((v[r] ^ key0) >> 32);
+  }
+  lo = __reduce_or_sync(kFull, lo);
+  hi = __reduce_or_sync(kFull, hi);
+  __syncthreads();
+  if (lane == 0) {
+    atomicOr(or_bits, lo);
+    atomicOr(or_bits + 1, hi);
+  }
+  sync_all();
+  lo = hi = 0;
+  if (used_blocks > 1) {
+    if (lane < used_blocks) {
+      const uint32_t at = cluster_addr(smem_u32(or_bits), static_cast<uint32_t>(lane));
+      lo = cluster_ld32(at);
+      hi = cluster_ld32(at + 4);
+    }
+    lo = __reduce_or_sync(kFull, lo);
+    hi = __reduce_or_sync(kFull, hi);
+  } else {
+    lo = or_bits[0];
+    hi = or_bits[1];
+  }
+  const unsigned long long used = (static_cast<unsigned long long>(hi) << 32) | lo;  // bits that differ within the list
+  const unsigned long long suffix = used == 0 ? 0 : ~0ull >> __clzll(static_cast<long long>(used));
+  const int idx_bits = sort_index_bits(K);
+  const unsigned low = (1u << idx_bits) - 1u;
+  const bool two = (suffix >> (63 - idx_bits)) != 0;
+#pragma unroll
+  for (int r = 0; r < kListPer; ++r)
+    v[r] = ((v[r] & (two ? 0xffffffffull : suffix)) << idx_bits) | static_cast<unsigned>(rank * per + first + 32 * r);
+
+  const bool network = K <= kListNetwork && used_blocks == 1 && !two;
+  if (network) {
+#pragma unroll
+    for (int r = 0; r < kListPer; ++r)
+      if (r < R && first + 32 * r < n) w[first + 32 * r] = v[r];
+    __syncthreads();
+    sort_words_merge128(w, n);
+#pragma unroll
+    for (int r = 0; r < kListPer; ++r)
+      if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
+  }
+  for (int round = 0; round < (network ? 0 : (two ? 2 : 1)); ++round) {
+    if (round == 1) {
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r) {
+        if (r < R && first + 32 * r < n) {
+          const unsigned i = static_cast<unsigned>(v[r]) & low;
+          v[r] = (((static_cast<unsigned long long>(gload(keys + i)) ^ kSign) >> 32) << idx_bits) | i;
+        }
+      }
+    }
+    const unsigned long long bits = !two ? used : (round == 0 ? used & 0xffffffffull : used >> 32);
+    for (int bit = 0; bit < 64 && (bits >> bit) != 0; bit += kListRadixBits) {
+      if (((bits >> bit) & (kListDigits - 1)) == 0) continue;
+      const int shift = idx_bits + bit;
+      for (int t = threadIdx.x; t < kListWarps * kListStride; t += kListThreads) cnt[t] = 0u;
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) atomicAdd(cnt + warp * kListStride + (static_cast<unsigned>(v[r] >> shift) & (kListDigits - 1)), 1u);
+      __syncthreads();
+      // counts -> places: a thread has four warps' counters of digit d; two neighbouring threads share a digit
+      const int d = threadIdx.x >> 1, w0 = (threadIdx.x & 1) * 4;
+      unsigned c[4], sum = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        c[j] = cnt[(w0 + j) * kListStride + d];
+        sum += c[j];
+      }
+      const unsigned other = __shfl_xor_sync(kFull, sum, 1);
+      if (w0 == 0) block_count[d] = sum + other;
+      sync_all();
+      unsigned total = sum + other, before_me = 0;  // words with digit d in the list, in the blocks before this one
+      if (used_blocks > 1) {
+        total = 0;
+        const uint32_t mine = smem_u32(block_count + d);
+#pragma unroll
+        for (int q = 0; q < kListMaxCluster; ++q) {
+          if (q < used_blocks) {
+            const unsigned x = cluster_ld32(cluster_addr(mine, static_cast<uint32_t>(q)));
+            total += x;
+            before_me += q < rank ? x : 0u;
+          }
+        }
+      }
+      unsigned incl = w0 == 0 ? total : 0u;  // one of the two threads of a digit carries it
+      const unsigned own = incl;
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const unsigned t = __shfl_up_sync(kFull, incl, s);
+        if (lane >= s) incl += t;
+      }
+      if (lane == 31) warp_total[warp] = incl;
+      __syncthreads();
+      const unsigned warps_before = __reduce_add_sync(kFull, lane < warp ? warp_total[lane & (kListWarps - 1)] : 0u);
+      if (w0 == 0) digit_base[d] = warps_before + incl - own + before_me;
+      __syncwarp();
+      unsigned at = digit_base[d] + (w0 == 0 ? 0u : other);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        cnt[(w0 + j) * kListStride + d] = at;
+        at += c[j];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r) {
+        if (r < R && first - lane + 32 * r < n) {  // warp-uniform
+          const bool live = first + 32 * r < n;
+          const unsigned dg = static_cast<unsigned>(v[r] >> shift) & (kListDigits - 1);
+          unsigned same = __ballot_sync(kFull, live);
+#pragma unroll
+          for (int b = 0; b < kListRadixBits; ++b) {
+            const unsigned vote = __ballot_sync(kFull, (dg >> b) & 1u);
+            same &= ((dg >> b) & 1u) ? vote : ~vote;
+          }
+          const unsigned before = __popc(same & lt);
+          unsigned* c2 = cnt + warp * kListStride + dg;
+          const unsigned start = *c2;
+          __syncwarp();
+          if (live && before == 0) *c2 = start + __popc(same);
+          __syncwarp();
+          if (live) {
+            const unsigned p = start + before;
+            if (used_blocks > 1) {
+              const unsigned q = __umulhi(p, per_inv);
+              cluster_st64(cluster_addr(smem_u32(w + (p - q * per)), q), v[r]);
+            } else {
+              w[p] = v[r];
+            }
+          }
+        }
+      }
+      sync_all();
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
+      // (the next pass writes any block's w only behind a barrier that every block reaches after these loads)
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kListPer; ++r) {
+    const int e = first + 32 * r;
+    if (r < R && e < n) {
+      const unsigned i = static_cast<unsigned>(v[r]) & low;
+      const long long k = two ? gload(keys + i) : static_cast<long long>(((key0 & ~suffix) | (v[r] >> idx_bits)) ^ kSign);
+      gstore(a.keys_out + e0 + rank * per + e, k);
+      if (a.perm_out) gstore(a.perm_out + e0 + rank * per + e, static_cast<int>(i));
+      if (a.rows_here) w[e] = v[r];
+    }
+  }
+  if (a.rows_here) {
+    __syncthreads();
+    gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + (e0 + rank * per) * a.row_ch,
+                static_cast<long long>(n) * a.row_ch, a.row_ch, [&](int row) { return static_cast<long long>(static_cast<unsigned>(w[row]) & low); });
+  }
+}
+
+// Rows of sorted lists follow the permutation.  Work is dealt out in units of kSortRowsTile records of the flat record
+// range: list r owns the items [start(r), start(r + 1)), start(r) = e_r / unit - e_0 / unit + r, at least as many as its
+// units, so no block is launched for a length that a list does not have; a warp finds an item's list by a 32-way search.
+constexpr int kSortRowsTileLog = 8, kSortRowsTile = 1 << kSortRowsTileLog;
+__global__ void __launch_bounds__(kSortRowsTile) sort_rows_kernel(const SortArgs a) {
+  chain_enter(false);
+  __shared__ int s_src[kSortRowsTile];
+  const int lane = threadIdx.x & 31;
+  const long long base = gload(a.edge_offsets) >> kSortRowsTileLog;
+  const long long n_items = (gload(a.edge_offsets + a.n_req) >> kSortRowsTileLog) - base + a.n_req;
+  for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
+    int r = 0, m = a.n_req;
+    while (m > 1) {
+      const int step = (m + 31) >> 5, p = r + lane * step;
+      const bool holds = lane * step < m && (gload(a.edge_offsets + p) >> kSortRowsTileLog) - base + p <= item;
+      const int c = max(1, __popc(__ballot_sync(kFull, holds)));  // starts ascend: the first c probes hold
+      r += (c - 1) * step;
+      m = min(step, m - (c - 1) * step);
+    }
+    const long long e0 = gload(a.edge_offsets + r);
+    const long long K = min(static_cast<long long>(gload(a.edge_offsets + r + 1) - e0), static_cast<long long>(a.max_len));
+    const long long first = (item - ((e0 >> kSortRowsTileLog) - base + r)) << kSortRowsTileLog;
+    if (first < 0 || first >= K) continue;  // block-uniform
+    const int n = static_cast<int>(min(static_cast<long long>(kSortRowsTile), K - first));
+    if (static_cast<int>(threadIdx.x) < n) s_src[threadIdx.x] = gload(a.perm_out + e0 + first + threadIdx.x);
+    __syncthreads();
+    gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + (e0 + first) * a.row_ch,
+                static_cast<long long>(n) * a.row_ch, a.row_ch, [&](int row) { return static_cast<long long>(s_src[row]); });
+    __syncthreads();  // s_src is rewritten by the next item
   }
 }
 

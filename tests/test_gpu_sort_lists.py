@@ -1,0 +1,74 @@
+"""GPU parity of the whole-list radix sort (ccr_sort_edges, lists of up to 32,768 records) against the CPU oracle: list
+lengths around a block's and a cluster's share, key ranges around every rule of the kernel (no differing bit, one digit,
+just room and no room for the index, full 64 bits), with and without the permutation output."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2609_22441_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+IMIN, IMAX = np.iinfo(np.int64).min, np.iinfo(np.int64).max
+LENS = ([1, 0, 2, 127, 128, 129, 511, 512], [513, 1023, 1024, 1025, 300], [4095, 4096, 4097, 1, 8191], [8193, 12_288, 12_289, 1000, 255], [32_768, 32_767, 20_000, 5, 28_673])
+KEYS = {
+    "equal": lambda rng, n: np.full(n, 7_000_000_019, np.int64),
+    "few": lambda rng, n: rng.integers(0, 3, size=n),
+    "26_bits": lambda rng, n: rng.integers(0, 50_000_000, size=n),
+    "48_bits": lambda rng, n: rng.integers(0, 1 << 48, size=n),  # with 15 index bits: just room
+    "49_bits": lambda rng, n: rng.integers(0, 1 << 49, size=n),
+    "high_half": lambda rng, n: rng.integers(0, 5, size=n) << 61,  # only the upper word differs
+    "outlier": lambda rng, n: np.where(np.arange(n) == n // 2, IMAX - 3, 123_456_789 + rng.permutation(n)),
+    "any": lambda rng, n: rng.integers(IMIN, IMAX, size=n, endpoint=True),
+    "ends": lambda rng, n: np.array([IMIN, -1, 0, IMAX])[rng.integers(0, 4, size=n)],
+}
+
+
+@pytest.mark.parametrize("with_perm", [True, False])
+@pytest.mark.parametrize("kind", list(KEYS))
+@pytest.mark.parametrize("lens", LENS, ids=lambda l: str(max(l)))
+def test_whole_lists_match_the_oracle(lens, kind, with_perm):
+    from paper_2609_22441_b200 import binding as B
+
+    if not with_perm and max(lens) > 19_000:
+        pytest.skip("refused without a permutation output")
+    rng = np.random.default_rng(len(kind) + sum(lens))
+    keys = np.concatenate([KEYS[kind](rng, n) for n in lens]).astype(np.int64)
+    feats = rng.integers(0, 1 << 16, size=(len(keys), 24), dtype=np.uint16).view(np.float16)  # 48-byte rows
+    eo = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    want_k, want_f, want_p = oracle.sort_edges(keys, feats, eo)
+    store = B.Docstore(16, 8, "float16", 24, "float16")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    k_out = torch.full((len(keys) + 2,), -7, dtype=torch.int64, device="cuda")
+    f_out = torch.full((len(keys) + 2, 24), 7.0, dtype=torch.float16, device="cuda")
+    p_out = torch.full((len(keys) + 2,), -7, dtype=torch.int32, device="cuda")
+    n = len(keys)
+    B.ccr_sort_edges(store, len(lens), max(lens), dev(keys), dev(feats.view(np.int16)), dev(eo), k_out[1:-1], f_out, p_out[1:-1] if with_perm else None)
+    torch.cuda.synchronize()
+    assert np.array_equal(k_out.cpu().numpy()[1:-1], want_k) and int(k_out[0]) == -7 and int(k_out[-1]) == -7
+    assert np.array_equal(f_out.cpu().numpy()[:n].view(np.uint16), want_f.view(np.uint16)) and bool((f_out[n:] == 7).all())
+    if with_perm:
+        assert np.array_equal(p_out.cpu().numpy()[1:-1], want_p) and int(p_out[0]) == -7 and int(p_out[-1]) == -7
+    store.free()
+
+
+def test_a_longer_batch_with_keys_that_cannot_be_packed():
+    """A list beyond the clusters' reach sends the batch to the chunked path; negative and far keys take its fallback."""
+    from paper_2609_22441_b200 import binding as B
+
+    rng = np.random.default_rng(3)
+    lens = [40_000, 9_000, 100, 0, 33_000]
+    keys = np.concatenate([KEYS[k](rng, n) for k, n in zip(("any", "26_bits", "few", "equal", "ends"), lens)]).astype(np.int64)
+    feats = rng.integers(0, 1 << 16, size=(len(keys), 24), dtype=np.uint16).view(np.float16)
+    eo = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    want_k, want_f, want_p = oracle.sort_edges(keys, feats, eo)
+    store = B.Docstore(16, 8, "float16", 24, "float16")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    k_out, p_out = torch.empty(len(keys), dtype=torch.int64, device="cuda"), torch.empty(len(keys), dtype=torch.int32, device="cuda")
+    f_out = torch.empty((len(keys), 24), dtype=torch.float16, device="cuda")
+    B.ccr_sort_edges(store, len(lens), max(lens), dev(keys), dev(feats.view(np.int16)), dev(eo), k_out, f_out, p_out)
+    torch.cuda.synchronize()
+    assert np.array_equal(k_out.cpu().numpy(), want_k) and np.array_equal(p_out.cpu().numpy(), want_p)
+    assert np.array_equal(f_out.cpu().numpy().view(np.uint16), want_f.view(np.uint16))
+    store.free()
