@@ -87,6 +87,36 @@ __device__ __forceinline__ uint4 edge2_reduce(unsigned long long reduce_sum_mask
   return make_uint4(res[0], res[1], res[2], res[3]);
 }
 
+// The same for a candidate with one found slot: a maximum keeps the row's bits; a sum is +0 plus the value, which changes
+// a negative zero to +0 and any NaN to 0x7fff and leaves every other value as it is (fp16 -> fp32 -> fp16 is exact).
+__device__ __forceinline__ uint4 edge2_single(unsigned long long reduce_sum_mask, int piece, const uint4& q) {
+  const unsigned sum8 = static_cast<unsigned>(reduce_sum_mask >> ((piece * 8) & 63)) & 0xffu;
+  const unsigned v[4] = {q.x, q.y, q.z, q.w};
+  unsigned res[4];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const unsigned lo = v[w] & 0xffffu, hi = v[w] >> 16;
+    const unsigned slo = lo == 0x8000u ? 0u : ((lo & 0x7fffu) > 0x7c00u ? 0x7fffu : lo);
+    const unsigned shi = hi == 0x8000u ? 0u : ((hi & 0x7fffu) > 0x7c00u ? 0x7fffu : hi);
+    res[w] = (((sum8 >> (2 * w)) & 1u) ? slo : lo) | ((((sum8 >> (2 * w + 1)) & 1u) ? shi : hi) << 16);
+  }
+  return make_uint4(res[0], res[1], res[2], res[3]);
+}
+
+// Position of the n-th set bit (from 0) of m; anything below 32 when m has no such bit.
+__device__ __forceinline__ int nth_set_bit(unsigned m, int n) {
+  int at = 0;
+#pragma unroll
+  for (int w = 16; w >= 1; w >>= 1) {
+    const int below = __popc((m >> at) & ((1u << w) - 1u));
+    if (n >= below) {
+      n -= below;
+      at += w;
+    }
+  }
+  return at & 31;
+}
+
 // 16-byte chunks a lane has in flight while it moves rows of run-time widths: as many loads as a warp of the tuned
 // variants keeps (16 + 4).  592-byte rows, 37 x 17,003 candidates: one chunk at a time with a division per chunk
 // 198 us, 8 / 12 / 16 / 20 / 24 in flight 142 / 137 / 133 / 123 / 132 us; batches of equal length (13 + 12 + 12 chunks
@@ -94,6 +124,7 @@ __device__ __forceinline__ uint4 edge2_reduce(unsigned long long reduce_sum_mask
 // the cosine section keep more beside the loads and have the registers for 8.
 constexpr int kGenericUnroll = 20;
 constexpr int kGenericUnrollSecond = 8;
+constexpr int kGenericUnrollSecondTwoPhase = 12;  // the two-phase kernel's 128 registers hold more (16 was no faster)
 
 // Section widths of a launch, in 16-byte chunks and bytes (compile-time where the variant fixes them).
 template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, bool COS = false>
@@ -243,7 +274,7 @@ __device__ __forceinline__ uint4 cosine_section(const JoinArgs& a, const uint4* 
   return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), 0u, 0u);
 }
 
-template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0>
+template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0, int GU = kGenericUnrollSecond>
 __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC_CH, EDGE_CH, REQ_CH, SECOND, CNP != 0>& sh,
                                            const int* s_idx, const int* s_pos, const int4* s_apos,
                                            const uint8_t* edge_base, const uint8_t* req_src, uint8_t* out, int cnt,
@@ -310,7 +341,7 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
     // steps by additions (32 chunks further = sh.step_row rows and sh.step_piece chunks, with a carry).  All sections
     // share one load instruction: a second one under the opposite predicate (document rows past L1) writes the same
     // registers and so waits for the first to return, which serialised the batch (321 us where this takes 123 us).
-    constexpr int U = (SECOND || kCos) ? kGenericUnrollSecond : kGenericUnroll;
+    constexpr int U = (SECOND || kCos) ? GU : kGenericUnroll;
     constexpr bool kLinear = !SECOND && !kCos;  // the chunks leave in the order they are walked: consecutive lanes, consecutive chunks
     const int edge_end = sh.doc_ch + sh.edge_ch, n_chunks = cnt * sh.src_ch;
     int row = sh.lane_row, piece = sh.lane_piece;
@@ -351,26 +382,46 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
       }
     }
   }
-  // edge2 section: the matched rows of the found engager slots, reduced per dim in slot order
+  // edge2 section: the matched rows of the found engager slots, reduced per dim in slot order.  Most candidates have no
+  // found slot and most others one: the rows without get their zeros in a pass of stores only, the rows with are
+  // counted off and share the lanes among themselves, and where none of a pass has a second slot the reduction is skipped.
+  // What a pass costs is its chain of dependent instructions, not its bytes (keeping the loads of several passes in flight
+  // made every case slower, 309 -> 392 us at the worst): 64 x 50,000 candidates with 128-byte edge rows 698 -> 664 us,
+  // single requests of 50,000 20.0 -> 18.5 us, 64-byte edge rows (30,000 x 64) no change at 309 us.
   if constexpr (SECOND) {
-    auto slots_of = [&](int row, int (&rp)[4]) {
-      rp[0] = rp[1] = rp[2] = rp[3] = -1;
-      if (row < cnt) {
+    const int4 ap = lane < cnt ? s_apos[lane] : make_int4(-1, -1, -1, -1);
+    // (rows of one chunk: a pass covers all 32 rows as it is, counting them off would only add to it)
+    const unsigned with = __ballot_sync(kFull, sh.edge_ch > 1 ? (ap.x & ap.y & ap.z & ap.w) >= 0 : lane < cnt);  // indices are >= 0, -1 = not found
+    uint8_t* out2 = out + sh.doc_b + sh.edge_b;
+    for (int i = 0; i < sh.edge_ch; ++i) {
+      const int c = i * 32 + lane, row = c / sh.edge_ch, piece = c - row * sh.edge_ch;
+      if (row < cnt && !((with >> row) & 1u)) st128_stream(out2 + row * out_b + piece * 16, make_uint4(0u, 0u, 0u, 0u));
+    }
+    const int n_chunks = __popc(with) * sh.edge_ch;
+#pragma unroll 1
+    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+      const int c = c0 + lane, nth = c / sh.edge_ch, piece = c - nth * sh.edge_ch;
+      const int row = nth_set_bit(with, nth);
+      int rp[4] = {-1, -1, -1, -1};
+      if (c < n_chunks) {
         const int4 p = s_apos[row];
         rp[0] = p.x;
         rp[1] = p.y;
         rp[2] = p.z;
         rp[3] = p.w;
       }
-    };
-    for (int i = 0; i < sh.edge_ch; ++i) {
-      const int c = i * 32 + lane, row = c / sh.edge_ch, piece = c - row * sh.edge_ch;
-      int rp[4];
-      slots_of(row, rp);
-      uint4 q[4];
-      edge2_load(edge_base, sh.edge_b, piece, rp, q);
-      const uint4 v = edge2_reduce(a.reduce_sum_mask, piece, rp, q);
-      if (row < cnt) st128_stream(out + row * out_b + sh.doc_b + sh.edge_b + piece * 16, v);
+      const int found = (rp[0] >= 0) + (rp[1] >= 0) + (rp[2] >= 0) + (rp[3] >= 0);
+      uint4 v;
+      if (!__any_sync(kFull, found > 1)) {
+        const int only = max(max(rp[0], rp[1]), max(rp[2], rp[3]));
+        v = make_uint4(0u, 0u, 0u, 0u);
+        if (only >= 0) v = edge2_single(a.reduce_sum_mask, piece, ldg128(edge_base + static_cast<long long>(only) * sh.edge_b + piece * 16));
+      } else {
+        uint4 q[4];
+        edge2_load(edge_base, sh.edge_b, piece, rp, q);
+        v = edge2_reduce(a.reduce_sum_mask, piece, rp, q);
+      }
+      if (c < n_chunks) st128_stream(out2 + row * out_b + piece * 16, v);
     }
   }
   // request section: one source row for the whole request (L1/L2 hits); run-time widths have stored it above
@@ -643,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
 
       // ================= phase B: stream the rows =================
       for (int g = warp * 32; g < n; g += kWarps * 32) {
-        emit_group<DOC_CH, EDGE_CH, REQ_CH, SECOND>(a, sh, s_idx + g, s_pos + g, s_apos + g, edge_base, req_src,
+        emit_group<DOC_CH, EDGE_CH, REQ_CH, SECOND, 0, kGenericUnrollSecondTwoPhase>(a, sh, s_idx + g, s_pos + g, s_apos + g, edge_base, req_src,
                                                                        a.out_rows + (out0 + g) * sh.out_b, min(32, n - g), lane);
       }
       __syncthreads();  // phase A of the next sub-tile overwrites the resolved arrays (and, in merge mode, the keys)
