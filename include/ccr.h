@@ -344,7 +344,8 @@ ccr_status ccr_workspace_outputs(const ccr_workspace* ws, void** rows, uint8_t**
 
 /* The same join with HOST buffers (the request payload of Section 6.1.3 arrives in host memory):
  * copies the inputs to the workspace, runs ccr_join_batch, copies rows and mask back — all enqueued
- * on `stream`, nothing synchronised.  Pinned host memory makes the copies asynchronous.
+ * on `stream`, nothing synchronised.  Pinned host memory makes the copies asynchronous; a payload whose arrays
+ * are all pinned and 16-byte aligned is fetched by one kernel instead of one copy per array.
  * total_edges = edge_offsets[n_req].  Sizes beyond the workspace give CCR_ERR_INVALID_ARG.
  * A batch of at least three requests and 786,432 candidates is pipelined: the requests are cut into three
  * groups of about equal candidate counts, and a group's payload crosses PCIe on a stream the workspace owns while

@@ -2,6 +2,7 @@
 // No CPU fallback exists: when CUDA is unavailable every compute entry fails with CCR_ERR_CUDA.
 #include "../../include/ccr.h"
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -14,6 +15,7 @@
 #include <new>
 #include <unordered_set>
 
+#include "ccr_copy.cuh"
 #include "ccr_join.cuh"
 #include "ccr_pad.cuh"
 #include "ccr_resolve.cuh"
@@ -43,6 +45,9 @@ constexpr size_t kStageBytes = 16u << 20;  // staging block of second-degree sto
 #ifndef CCR_HOST_GROUP_CANDS
 #define CCR_HOST_GROUP_CANDS (2 * kSmallLaunchCands)
 #endif
+// Host payloads up to this size are fetched by one kernel (ccr_copy.cuh), larger ones by the copy engine: the kernel is ahead by the
+// gaps between the copies (3 MB 249 -> 221 us a call), from about 16 MB on the two are level (387 against 398 us, alone 387 / 414).
+constexpr size_t kKernelCopyBytes = 16u << 20;
 constexpr int kHostGroups = CCR_HOST_GROUPS;         // most request groups of a pipelined host-buffer join
 constexpr int kSchedRegions = 64;                    // launches of one store that may be in flight at once
 constexpr int kStatusHead = 4;                       // [0] wait expiry, [1] validation code; then the scheduling words:
@@ -360,6 +365,55 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   return launch_chained_cluster(fn, grid, block, smem, st, 1, args...);
 }
+
+// May a kernel access the host range [p, p + bytes) as it stands?  Only if one page-locked allocation holds all of it under
+// this very address (pageable memory, ranges that reach beyond their registration and managed memory are left to
+// cudaMemcpyAsync).  Asked anew for every call: an address says nothing about what is behind it the next time.
+bool device_reads_host(const void* p, size_t bytes) {
+  using GetAttributes = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static const GetAttributes get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<GetAttributes>(f);
+  }();
+  if (get == nullptr || p == nullptr || !aligned16(p)) return false;
+  unsigned int type = 0;
+  int managed = 0;
+  CUdeviceptr device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* into[5] = {&type, &managed, &device, &start, &size};
+  const CUdeviceptr q = reinterpret_cast<CUdeviceptr>(p);
+  if (get(5, what, into, q) != CUDA_SUCCESS) return false;
+  return type == CU_MEMORYTYPE_HOST && !managed && device == q && start != 0 && start <= q && bytes <= size && q - start <= size - bytes;
+}
+
+// Copies collected into one launch of copy_segments_kernel.
+struct SegmentCopy {
+  ccr::CopyArgs a = {};
+  bool ok = true;  // every segment may be copied by a kernel, and together they are small enough for it to pay
+  size_t total = 0;
+  explicit SegmentCopy(size_t bytes) : ok(bytes <= kKernelCopyBytes) {}
+  void add(void* dst, const void* src, size_t bytes, const void* host_side) {
+    if (bytes == 0 || !ok) return;
+    ok = a.n < ccr::kCopySegments && aligned16(dst) && (host_side == nullptr || device_reads_host(host_side, bytes));
+    if (!ok) return;
+    a.src[a.n] = static_cast<const uint8_t*>(src);
+    a.dst[a.n] = static_cast<uint8_t*>(dst);
+    a.bytes[a.n++] = static_cast<long long>(bytes);
+    total += bytes;
+  }
+  dim3 grid() const {
+    const size_t per_block = static_cast<size_t>(ccr::kCopyThreads) * ccr::kCopyUnroll * 16;
+    return dim3(static_cast<unsigned>(std::min<size_t>((total + per_block - 1) / per_block + a.n, 256)));
+  }
+};
 
 size_t out_row_bytes(const ccr_docstore* s, uint32_t flags) {
   const bool second = s->desc.max_actors > 0 && !(flags & CCR_FLAG_FIRST_DEGREE_ONLY);
@@ -1459,16 +1513,33 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
     if (n_groups > n_req) n_groups = n_req;
     if (n_groups < kHostGroups) n_groups = 1;
   }
+  bool by_kernel = false;
   if (n_groups == 1) {
-    if (total_edges > 0) {
-      ok = ok && cudaMemcpyAsync(w->edge_keys, edge_keys, total_edges * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-      ok = ok && cudaMemcpyAsync(w->edge_feats, edge_feats, total_edges * w->edge_b, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    const size_t sz_keys = static_cast<size_t>(total_edges) * 8, sz_feats = static_cast<size_t>(total_edges) * w->edge_b;
+    const size_t sz_off = (static_cast<size_t>(n_req) + 1) * 8, sz_idx = static_cast<size_t>(total_cands) * 4;
+    const size_t sz_req = static_cast<size_t>(n_req) * s->req_b;
+    SegmentCopy in(sz_keys + sz_feats + 2 * sz_off + sz_idx + sz_req);
+    in.add(w->edge_keys, edge_keys, sz_keys, edge_keys);
+    in.add(w->edge_feats, edge_feats, sz_feats, edge_feats);
+    in.add(w->edge_offsets, edge_offsets, sz_off, edge_offsets);
+    in.add(w->cand_idx, cand_idx, sz_idx, cand_idx);
+    in.add(w->cand_offsets, cand_offsets, sz_off, cand_offsets);
+    in.add(w->req_feats, req_feats, sz_req, req_feats);
+    by_kernel = in.ok;
+    if (by_kernel) {
+      // (an ordinary launch: it writes what the join in front of it may still be reading)
+      ccr::copy_segments_kernel<<<in.grid(), ccr::kCopyThreads, 0, st>>>(in.a);
+      ok = cudaGetLastError() == cudaSuccess;
+    } else {
+      if (total_edges > 0) {
+        ok = ok && cudaMemcpyAsync(w->edge_keys, edge_keys, sz_keys, cudaMemcpyHostToDevice, st) == cudaSuccess;
+        ok = ok && cudaMemcpyAsync(w->edge_feats, edge_feats, sz_feats, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      }
+      ok = ok && cudaMemcpyAsync(w->edge_offsets, edge_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      ok = ok && cudaMemcpyAsync(w->cand_idx, cand_idx, sz_idx, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      ok = ok && cudaMemcpyAsync(w->cand_offsets, cand_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      if (s->req_b > 0) ok = ok && cudaMemcpyAsync(w->req_feats, req_feats, sz_req, cudaMemcpyHostToDevice, st) == cudaSuccess;
     }
-    ok = ok && cudaMemcpyAsync(w->edge_offsets, edge_offsets, (n_req + 1) * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(w->cand_idx, cand_idx, total_cands * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(w->cand_offsets, cand_offsets, (n_req + 1) * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    if (s->req_b > 0)
-      ok = ok && cudaMemcpyAsync(w->req_feats, req_feats, static_cast<size_t>(n_req) * w->req_b, cudaMemcpyHostToDevice, st) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
       return CCR_ERR_CUDA;
@@ -1540,7 +1611,12 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
   }
   if (out_rows != nullptr)  // NULL: the rows stay in the workspace for a consumer on the device (ccr_workspace_outputs)
     ok = ok && cudaMemcpyAsync(out_rows, w->out_rows, total_cands * out_b, cudaMemcpyDeviceToHost, st) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(out_mask, w->out_mask, total_cands, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+  SegmentCopy back(by_kernel ? static_cast<size_t>(total_cands) : SIZE_MAX);
+  back.add(out_mask, w->out_mask, static_cast<size_t>(total_cands), out_mask);
+  if (back.ok)
+    ok = ok && launch_chained(ccr::copy_segments_kernel, back.grid(), dim3(ccr::kCopyThreads), 0, st, back.a) == cudaSuccess;
+  else
+    ok = ok && cudaMemcpyAsync(out_mask, w->out_mask, total_cands, cudaMemcpyDeviceToHost, st) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     return CCR_ERR_CUDA;
@@ -1622,15 +1698,29 @@ ccr_status ccr_join_payload_static(const ccr_docstore* s, int32_t n_req, int64_t
   const ccr_status rs = static_scratch(s->desc.device, &base);
   if (rs != CCR_OK) return rs;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  bool ok = cudaMemsetAsync(base, 0, kStaticControlBytes, st) == cudaSuccess;  // the words must start at zero
-  if (total_edges > 0) {
-    ok = ok && cudaMemcpyAsync(base + o_keys, edge_keys, sz_keys, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(base + o_feats, edge_feats, sz_feats, cudaMemcpyHostToDevice, st) == cudaSuccess;
+  bool ok = true;
+  SegmentCopy in(sz_keys + sz_feats + 2 * sz_off + sz_idx + sz_req);
+  in.add(base, nullptr, kStaticControlBytes, nullptr);  // the scheduling words must start at zero
+  in.add(base + o_keys, edge_keys, sz_keys, edge_keys);
+  in.add(base + o_feats, edge_feats, sz_feats, edge_feats);
+  in.add(base + o_eo, edge_offsets, sz_off, edge_offsets);
+  in.add(base + o_idx, cand_idx, sz_idx, cand_idx);
+  in.add(base + o_co, cand_offsets, sz_off, cand_offsets);
+  in.add(base + o_req, req_feats, sz_req, req_feats);
+  if (in.ok) {
+    ccr::copy_segments_kernel<<<in.grid(), ccr::kCopyThreads, 0, st>>>(in.a);
+    ok = cudaGetLastError() == cudaSuccess;
+  } else {
+    ok = cudaMemsetAsync(base, 0, kStaticControlBytes, st) == cudaSuccess;
+    if (total_edges > 0) {
+      ok = ok && cudaMemcpyAsync(base + o_keys, edge_keys, sz_keys, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      ok = ok && cudaMemcpyAsync(base + o_feats, edge_feats, sz_feats, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    }
+    ok = ok && cudaMemcpyAsync(base + o_eo, edge_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(base + o_idx, cand_idx, sz_idx, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(base + o_co, cand_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    if (sz_req > 0) ok = ok && cudaMemcpyAsync(base + o_req, req_feats, sz_req, cudaMemcpyHostToDevice, st) == cudaSuccess;
   }
-  ok = ok && cudaMemcpyAsync(base + o_eo, edge_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(base + o_idx, cand_idx, sz_idx, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(base + o_co, cand_offsets, sz_off, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  if (sz_req > 0) ok = ok && cudaMemcpyAsync(base + o_req, req_feats, sz_req, cudaMemcpyHostToDevice, st) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     return CCR_ERR_CUDA;
