@@ -785,7 +785,7 @@ ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sort
   ok = ok && cudaFuncSetAttribute(ccr::resolve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   ccr::kResolveTopMax * 8 + 256) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(ccr::resolve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  ccr::kResolveTopMax * 8 + 256) == cudaSuccess;
+                                  ((ccr::kResolveTopMax + 1) << ccr::kResolveFanLog2) * 8 + 256) == cudaSuccess;
   ix->magic = kIxMagic;
   handle_add(ix);
   if (!ok) {
@@ -836,11 +836,12 @@ ccr_status ccr_resolve_ids(const ccr_idindex* cix, int64_t n_queries, const int6
   long long blocks = (n_queries * lanes + per_block - 1) / per_block;
   const long long cap = static_cast<long long>(ix->n_sms) * ccr::kResolveBlocksPerSm;  // the top level is re-read by every block
   if (blocks > cap) blocks = cap;
-  const size_t smem = static_cast<size_t>(ix->count[ix->n_levels - 1]) * 8 + 16;
-  if (n_queries >= ccr::kResolveWarpMin)
-    ccr::resolve_kernel<true><<<static_cast<unsigned>(blocks), ccr::kResolveThreads, smem, static_cast<cudaStream_t>(stream)>>>(a);
-  else
-    ccr::resolve_kernel<false><<<static_cast<unsigned>(blocks), ccr::kResolveThreads, smem, static_cast<cudaStream_t>(stream)>>>(a);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const bool wide = n_queries >= (ix->n_ids * 8 <= kIdsInL2Bytes ? ccr::kResolveWarpMinInL2 : ccr::kResolveWarpMin);
+  if (wide && a.n_levels > 2) --a.n_levels;  // the level below the top is staged (the leaf level never is)
+  const size_t smem = static_cast<size_t>(a.count[a.n_levels - 1]) * 8 + 16;
+  if (wide) ccr::resolve_kernel<true><<<static_cast<unsigned>(ix->n_sms), ccr::kResolveWideThreads, smem, st>>>(a);
+  else ccr::resolve_kernel<false><<<static_cast<unsigned>(blocks), ccr::kResolveThreads, smem, st>>>(a);
   ix->launches++;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
 #ifdef CCR_DEBUG_BOUNDS

@@ -11,11 +11,10 @@
 // keys below the id and add the counts up with two shuffles; the leaf round also says whether the id is
 // present.  The small levels stay in L2, the large ones come from HBM 64 bytes at a time.  A query over 300M ids
 // makes 6 dependent rounds instead of 29 dependent probes across the whole array.  Two queries per group of
-// lanes in flight, up to 2,048 threads per SM.  A batch of a million queries or more is bound by instruction
-// issue rather than by the chain of rounds; there a warp takes 32 queries at a time, searches the top level a lane
-// per query (the same instructions serve 32 queries instead of 8) and hands the queries to the lane groups by
-// shuffles, four per group in flight (1.92M queries over 1M ids: 75 -> 62 us; on 240,000 queries over 300M ids
-// that form was 13-20 % slower, hence the size rule).  Measured and slower: wider windows (128 bytes with eight lanes
+// lanes in flight, up to 2,048 threads per SM.  Large batches are bound
+// by the windows' traffic and by instruction issue rather than by the chain of rounds; there a warp takes 32 queries at
+// a time, searches the staged level a lane per query (the same instructions serve 32 queries instead of 8) and hands the
+// queries to the lane groups by shuffles, four per group in flight; see kResolveWarpMin.  Measured and slower: wider windows (128 bytes with eight lanes
 // per query; 256 bytes in two rounds), a lane per query with 1-8 queries in flight, and a larger staged top
 // level (it takes shared memory from the L1 and start-up time from every block).
 #pragma once
@@ -28,10 +27,17 @@ constexpr int kResolveFanLog2 = 3;                 // 8 keys = one 64-byte windo
 constexpr int kResolveMaxLevels = 8;               // 2,048 x 8^7 ids: more than int32 positions can name
 constexpr int kResolveTopMax = 2048;               // keys of the top level (16 KB of shared memory)
 constexpr int kResolveThreads = 256;
+constexpr int kResolveWideThreads = 1024;         // one block per SM for large batches, around the level below the top
 constexpr int kResolveBlocksPerSm = 8;             // grid cap: the top level is staged by every block
 constexpr int kResolveUnroll = 2;                  // queries a group of lanes keeps in flight
 constexpr int kResolveWarpUnroll = 4;              // ... when a warp takes 32 queries at a time (all of them at once)
-constexpr long long kResolveWarpMin = 1 << 20;     // batches from this size on search the top level a lane per query
+// Large batches: a lane per query in the top search, and one block of 1,024 threads per SM that stages the level BELOW the
+// top (up to 16,391 keys, 131 KB): 148 copies of it cost 2-3 us and save every query a 64-byte window, which is what bounds a large
+// batch (L2 to SM).  1.92M queries over 1M ids 62 -> 50 us, 1.45M over 5.8M 54.9 -> 49.2 us, 1M over 300M 83.5 -> 77.4 us, 300,000
+// over 5M 17.2 -> 15.4 us; where the chain of rounds counts, half the threads are too few: 240,000 over 300M 24.4 -> 26.6 us, 674,000
+// over 139M 69.6 -> 73.5 us.
+constexpr long long kResolveWarpMin = 1 << 20;        // batches from this size on
+constexpr long long kResolveWarpMinInL2 = 1 << 18;    // ... over an index that stays in L2
 constexpr long long kResolveInf = 0x7fffffffffffffffLL;  // stands for the keys beyond the end of a level
 
 struct ResolveArgs {
@@ -76,12 +82,17 @@ __global__ void pad_level_kernel(int64_t* level, long long n) {
 // WARP_TOP: the top level searched a lane per query (large batches, bound by instruction issue); otherwise by the
 // group of lanes that descends with the query (small batches, bound by the chain of dependent rounds).
 template <bool WARP_TOP>
-__global__ void __launch_bounds__(kResolveThreads) resolve_kernel(const ResolveArgs a) {
+__global__ void __launch_bounds__(WARP_TOP ? kResolveWideThreads : kResolveThreads) resolve_kernel(const ResolveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_res[];
   int64_t* top = reinterpret_cast<int64_t*>(smem_res);
   const int top_l = a.n_levels - 1;
   const int n_top = static_cast<int>(a.count[top_l]);
-  for (int i = threadIdx.x; i < n_top; i += blockDim.x) top[i] = gload(a.level[top_l] + i);
+  if constexpr (WARP_TOP) {
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n_top; i += kResolveWideThreads) top[i] = gload(a.level[top_l] + i);
+  } else {
+    for (int i = threadIdx.x; i < n_top; i += blockDim.x) top[i] = gload(a.level[top_l] + i);
+  }
   __syncthreads();
   constexpr int G = 1 << (kResolveFanLog2 - 1);  // lanes that share a query: one 16-byte load each per window
   if constexpr (WARP_TOP) {
