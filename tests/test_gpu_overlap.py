@@ -49,3 +49,18 @@ def test_alternating_batches_into_one_buffer(n_req, big, small, second):
     assert np.array_equal(got_mask[n:], wants[0][1][n:]) and np.array_equal(got_rows[n:], wants[0][0][n:])
     assert not T.any() and store.device_status() == B.CCR_OK
     store.free()
+
+
+@pytest.mark.parametrize("k", [28_400, 28_540, 28_700, 28_790])
+def test_forced_staging_of_the_longest_lists(k):
+    """Lists that just fit the two-phase kernel's shared memory are staged whole, with and without room for anything beside them."""
+    from paper_2609_22441_b200 import binding as B
+
+    wl = W.config1(seed=77, n_docs=60_000, n_req=1, n_cand=3_001, edge_lo=k, edge_hi=k)
+    assert wl.batch.max_edge_len == k
+    want_rows, want_mask = oracle.join_workload(wl, n_threads=4)
+    store, db = B.store_from_workload(wl), B.DeviceBatch(wl.batch)
+    rows, mask = B.join_batch(store, db, B.CCR_FLAG_FORCE_SMEM)
+    torch.cuda.synchronize()
+    assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
+    store.free()
