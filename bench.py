@@ -806,8 +806,8 @@ def sort_bench(args, B, device: int):
                    "peak_kind": "of " + peak_kind},
         "roofline": {"bound": "hbm", "achieved": head["algorithmic_gbs"], "peak": peak, "unit": "GB/s",
                      "frac": head["frac_of_hbm_peak"], "traffic": None,
-                     "note": "seven dependent kernels per call, each starting on flushed caches, and the shared-memory merge "
-                             "sort of the chunks: latency- and instruction-bound, not by HBM"},
+                     "note": "two dependent kernels per call, each starting on flushed caches; the radix sort of the lists is "
+                             "bound by instruction issue, not by HBM"},
         "payloads": results, "gpu_launches": head["gpu_launches"],
     }))
 
