@@ -658,7 +658,8 @@ __global__ void __launch_bounds__(kSortGatherThreads) gather_all_kernel(const So
 // Lists of up to kListNetwork records have too few words for the passes to pay: sorted by sort_words_merge128 instead (256
 // lists of 900-1,000 records, 2^40 keys: 37 -> 29 us; one list of 200 records 12.9 -> 9.7 us).
 // 256 lists <= 20,000 (700,000 records of 128-byte rows): 141 us as chunks and merges, 90 us this way; 4 such lists
-// 38.7 -> 29 us; 64 lists <= 5,000 in the request flow 37 -> 27 us; 4 lists <= 9,214 with a far outlier each 145 -> 82 us.
+// 38.7 -> 29 us; 64 lists <= 5,000 (61,823 records) 44 -> 28 us; a request flow with 4 lists <= 9,214 that hold a far outlier
+// each 164 -> 92 us.
 constexpr int kListRadixBits = 7, kListDigits = 1 << kListRadixBits;
 constexpr int kListStride = kListDigits + 1;  // counters of a warp; odd, so that the scan's column reads spread over the banks
 constexpr int kListThreads = 256, kListPer = 16, kListWarps = kListThreads / 32;
