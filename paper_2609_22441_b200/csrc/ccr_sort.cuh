@@ -761,6 +761,9 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
     hi = or_bits[1];
   }
   const unsigned long long used = (static_cast<unsigned long long>(hi) << 32) | lo;  // bits that differ within the list
+  // No block may leave while another can still read its shared memory.  The passes end in a barrier of the whole cluster
+  // behind their last remote access; a list of equal keys (`used` is the same in every block) makes no pass and needs one here.
+  if (used_blocks > 1 && used == 0) cluster_sync();
   const unsigned long long suffix = used == 0 ? 0 : ~0ull >> __clzll(static_cast<long long>(used));
   const int idx_bits = sort_index_bits(K);
   const unsigned low = (1u << idx_bits) - 1u;

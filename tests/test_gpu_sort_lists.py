@@ -72,3 +72,31 @@ def test_a_longer_batch_with_keys_that_cannot_be_packed():
     assert np.array_equal(k_out.cpu().numpy(), want_k) and np.array_equal(p_out.cpu().numpy(), want_p)
     assert np.array_equal(f_out.cpu().numpy().view(np.uint16), want_f.view(np.uint16))
     store.free()
+
+
+def test_many_long_lists_of_equal_keys():
+    """Lists of several blocks without a differing bit are sorted without a single pass: the blocks of a cluster only exchange what
+    differs and then leave at different times (a last block of one record beside full ones).  One list of each length has a
+    differing bit in its last record."""
+    from paper_2609_22441_b200 import binding as B
+
+    rng = np.random.default_rng(11)
+    lens = [n for n in (4097, 8191, 8193, 12_289, 16_385, 28_673, 32_768) for _ in range(24)]
+    keys = [np.full(n, 3 * i - 200, np.int64) for i, n in enumerate(lens)]
+    for i in range(0, len(lens), 24):
+        keys[i][-1] -= 1
+    keys = np.concatenate(keys)
+    feats = rng.integers(0, 1 << 16, size=(len(keys), 8), dtype=np.uint16).view(np.float16)
+    eo = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    want_k, want_f, want_p = oracle.sort_edges(keys, feats, eo)
+    store = B.Docstore(16, 8, "float16", 8, "float16")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    k_in, f_in, o = dev(keys), dev(feats.view(np.int16)), dev(eo)
+    for _ in range(5):
+        k_out, p_out = torch.full_like(k_in, -7), torch.full((len(keys),), -7, dtype=torch.int32, device="cuda")
+        f_out = torch.empty((len(keys), 8), dtype=torch.float16, device="cuda")
+        B.ccr_sort_edges(store, len(lens), max(lens), k_in, f_in, o, k_out, f_out, p_out)
+        torch.cuda.synchronize()
+        assert np.array_equal(k_out.cpu().numpy(), want_k) and np.array_equal(p_out.cpu().numpy(), want_p)
+        assert np.array_equal(f_out.cpu().numpy().view(np.uint16), want_f.view(np.uint16))
+    store.free()
