@@ -1235,8 +1235,8 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     long long blocks = static_cast<long long>(s->n_sms) * per_sm;
     const long long most = (groups + 1) / 2;
     if (blocks > most) blocks = most;
-    // (programmatic stream serialization as above: a request resolves its candidates while the one in front of it
-    // drains; a stream of single requests of 50,000 candidates 16.7 -> 10.6 us each, 38,000 of 752-byte rows 25.7 -> 17.2 us)
+    // (programmatic stream serialization: the launch is set up while the work in front of it drains, and waits for its end
+    // before it reads anything; figures at the wait in join_kernel)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(blocks));
     cfg.blockDim = dim3(ccr::kThreads);

@@ -140,11 +140,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   return false;
 }
 
-// Programmatic dependent launch.  A join launched right behind another join on the same stream may become resident
-// while the earlier one drains (as its blocks leave their SMs) and run everything that only reads its own inputs;
+// Programmatic dependent launch.  A launch of the warp-specialised join right behind another one on the same stream may become
+// resident while the earlier one drains (as its blocks leave their SMs) and run everything that only reads its own inputs;
 // pdl_wait() returns once the earlier grid has completed and its writes are visible, and comes before the first
-// global store.  pdl_trigger() tells the runtime that this block no longer needs to hold back a dependent launch.
-// Both are no-ops for a launch without the attribute or without a predecessor that triggers.
+// global store.  The two-phase join waits before it reads anything.  pdl_trigger() tells the runtime that this block no longer
+// needs to hold back a dependent launch.  Both are no-ops for a launch without the attribute or without a predecessor that triggers.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -51,6 +51,51 @@ def test_alternating_batches_into_one_buffer(n_req, big, small, second):
     store.free()
 
 
+@pytest.mark.parametrize("second", [False, True])
+@pytest.mark.parametrize("front_ws", [False, True])
+def test_small_join_reads_what_the_join_in_front_wrote(second, front_ws):
+    """A small join is in stream order with everything in front of it, its inputs included: its candidate positions are the rows
+    of the join launched directly before it.  Two such joins write the buffer in turn, so an early read would find the other's."""
+    from paper_2609_22441_b200 import binding as B
+
+    rng = np.random.default_rng(17)
+    back = W.config1(seed=31, n_docs=50_000, n_req=1, n_cand=64, second_degree=second, edge_lo=900, edge_hi=900)
+    fronts = []
+    for i in range(2):  # rows of 64 bytes of positions and a 16-byte edge section
+        st = W.make_store(rng, 5_000, 25_000, 16, np.float32)
+        st.doc_feats = rng.integers(0, back.store.n_docs, size=(st.n_docs, 16)).astype(np.int32).view(np.float32)
+        keys, _ = W.make_viewer(rng, 25_000, 1_000, 8, np.float16)
+        feats = rng.integers(0, 40, size=(1_000, 8)).astype(np.uint16).view(np.float16)
+        cands = rng.integers(0, st.n_docs, size=6_000).astype(np.int32)
+        fronts.append(W.Workload("front", i, st, W.assemble_batch([keys], [feats], [cands], None, 8, np.float16, 0, np.float32)))
+    wants = []
+    for wl in fronts:
+        idx = np.ascontiguousarray(oracle.join_workload(wl, n_threads=4)[0]).view(np.int32).reshape(-1)
+        b = back.batch
+        b2 = W.assemble_batch([b.edge_keys], [b.edge_feats], [idx], b.req_feats, b.edge_dim, b.edge_dtype, b.req_dim, b.req_dtype)
+        wants.append(oracle.join_workload(W.Workload("back", 0, back.store, b2), n_threads=4))
+    n = fronts[0].batch.total_cands * 20
+    front_stores, dbs = [B.store_from_workload(wl) for wl in fronts], [B.DeviceBatch(wl.batch) for wl in fronts]
+    store, db = B.store_from_workload(back), B.DeviceBatch(back.batch)
+    idx_buf = torch.zeros(n, dtype=torch.int32, device="cuda")
+    front_mask = torch.zeros(n // 20, dtype=torch.uint8, device="cuda")
+    co = torch.tensor([0, n], dtype=torch.int64, device="cuda")
+    outs = [(torch.zeros((n, store.out_row_bytes(0)), dtype=torch.uint8, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda")) for _ in range(2)]
+    flags = B.CCR_FLAG_WARP_SPECIALISED if front_ws else 0
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for st, d, (rows, mask) in zip(front_stores, dbs, outs):
+            B.ccr_join_batch(st, 1, d.total_cands, d.max_edge_len, d.edge_keys, d.edge_feats, d.edge_offsets, d.cand_idx, d.cand_offsets, None, idx_buf,
+                             front_mask, flags)
+            B.ccr_join_batch(store, 1, n, db.max_edge_len, db.edge_keys, db.edge_feats, db.edge_offsets, idx_buf, co, db.req_feats, rows, mask)
+    torch.cuda.synchronize()
+    for (rows, mask), (want_rows, want_mask) in zip(outs, wants):
+        assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
+    for st in front_stores + [store]:
+        assert st.device_status() == B.CCR_OK
+        st.free()
+
+
 @pytest.mark.parametrize("k", [28_400, 28_540, 28_700, 28_790])
 def test_forced_staging_of_the_longest_lists(k):
     """Lists that just fit the two-phase kernel's shared memory are staged whole, with and without room for anything beside them."""
