@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
       const int s = it % kSlots;
       if (!mbar_wait_bounded(full0 + 8 * s, (it / kSlots) & 1u)) {
         if (lane == 0) atomicExch(a.status, kDevWaitExpired);
-        return;
+        break;
       }
       const WsSlot d = slots[s];
       if (d.n == 0) break;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0 + 8 * s);
     }
-    pdl_wait();  // also of a block that had nothing to store: a launch never completes before the one in front of it
+    pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
     return;
   }
 

@@ -1,0 +1,33 @@
+"""Every block of the join kernels waits for the launch in front of it before it leaves, whichever way it leaves: a launch that
+completed before its predecessor would let the work behind it start too early.  No wait can be made to run out in a sound launch,
+so the exits are checked in the source."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_22441_b200", "csrc")
+
+
+def _kernel_body(file, name):
+    src = open(os.path.join(CSRC, file)).read()
+    at = src.index("{", re.search(r"\b%s\(const JoinArgs a" % name, src).start())
+    depth, i = 1, at + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(src[i], 0)
+        i += 1
+    return re.sub(r"//[^\n]*", "", src[at:i])
+
+
+@pytest.mark.parametrize("file,name", [("ccr_join.cuh", "join_kernel"), ("ccr_ws.cuh", "join_ws_kernel")])
+def test_no_exit_of_a_join_kernel_without_the_wait(file, name):
+    body = _kernel_body(file, name)
+    wait = "pdl_wait();"
+    if name == "join_kernel":  # the whole block waits in front of its first read
+        first = body.index(wait)
+        assert not re.search(r"\breturn\b|\bgload\b|\bstage_keys\b", body[:first])
+        return
+    exits = [m.start() for m in re.finditer(r"\breturn;", body)]
+    assert len(exits) == 2  # a block without work, and the streamers
+    for e in exits:
+        assert body[:e].rstrip().endswith(wait)
