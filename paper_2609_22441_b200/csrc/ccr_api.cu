@@ -1044,12 +1044,11 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   const int cos_bytes = cos ? ccr::ws_cos_bytes(n_str, cos_stage) : 0;
   // Shared memory of a block: the kernel's own arrays for a sub-tile of t candidates plus `area` bytes for the search
   // (staged keys, hash tables, sampled keys; ccr_search.cuh).
-  bool stash = true;  // the two-phase kernel's author ids of the first sub-tile
   auto smem_for = [&](int t, int area) -> size_t {
     return use_ws ? static_cast<size_t>(ccr::WsLayout(t, second, area, n_req <= ccr::kWsMaxCachedReq ? n_req : 0, cos_bytes, n_res,
                                                       rebal ? ccr::kRebalSlots : ccr::kWsSlots,
                                                       rebal ? ccr::kRebalInFlight * 128 : ccr::kWsWorkItems).bytes)
-                  : static_cast<size_t>(ccr::TileLayout(t, second, merge || stash, area).bytes);
+                  : static_cast<size_t>(ccr::TileLayout(t, second, merge, area).bytes);
   };
   // bytes that hold a list of K keys in its best form: staged next to its table (the merge path builds no table)
   auto best_area = [&](long long K) -> long long {
@@ -1085,7 +1084,6 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   const bool explicit_cap = (flags & CCR_FLAG_FORCE_SMEM) || s->key_cap > 0;
   const int must_fit = explicit_cap ? ccr::search_keys_bytes(key_cap) : 0;
   while (tile > 256 && static_cast<long long>(smem_for(tile, must_fit)) > kMaxSmemBytes) tile -= 256;
-  if (static_cast<long long>(smem_for(tile, must_fit)) > kMaxSmemBytes) stash = false;  // the promised keys come first
   const long long fixed = static_cast<long long>(smem_for(tile, 0));
   long long area = best_area(key_cap);
   if (fixed + area > budget) area = budget - fixed;
@@ -1134,7 +1132,6 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   a.key_cap = key_cap;
   a.search_area = static_cast<int>(area);
   a.min_stride_log2 = (flags & CCR_FLAG_FORCE_SAMPLED) ? 2 : 0;
-  a.stash = stash ? 1 : 0;
   a.warp_search = ((flags & CCR_FLAG_WARP_SEARCH) && use_ws) ? 1 : 0;  // its callers there are converged warps
   a.status = s->status;
   a.sched = nullptr;

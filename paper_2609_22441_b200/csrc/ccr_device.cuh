@@ -70,7 +70,6 @@ struct JoinArgs {
   int key_cap;                // longest list a block may stage in full per request; 0 = search global memory
   int search_area;            // bytes of shared memory the search may use for keys, tables or sampled keys
   int min_stride_log2;        // >0 forces sampling with at least this stride (testing aid)
-  int stash;                  // two-phase kernel: the first sub-tile's author ids are fetched ahead (0: no room beside the keys)
   int warp_search;            // searches that run in global memory use the warp-cooperative 32-ary search (comparison aid)
   int* status;                // device status words
   int* sched;                 // two scheduling words (next tile, finished blocks), zero between launches; or null

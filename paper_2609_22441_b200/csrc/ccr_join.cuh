@@ -203,13 +203,12 @@ __device__ __forceinline__ int block_lower_bound(const int64_t* g, int K, int64_
 // Shared-memory layout of join_kernel, shared by host (sizing) and device (carving).
 struct TileLayout {
   int off_idx, off_pos, off_apos, off_auth, off_keys, bytes;
-  // author_ids: a slot for every candidate's author id (merge mode; JoinArgs::stash)
-  __host__ __device__ TileLayout(int tile, bool second, bool author_ids, int search_area) {
+  __host__ __device__ TileLayout(int tile, bool second, bool merge, int search_area) {
     off_idx = kSmemHeader;
     off_pos = off_idx + tile * 4;
     off_apos = off_pos + tile * 4;
     off_auth = off_apos + (second ? tile * 16 : 0);
-    off_keys = off_auth + (author_ids ? tile * 8 : 0);
+    off_keys = off_auth + (merge ? tile * 8 : 0);
     off_keys = (off_keys + 15) & ~15;
     bytes = off_keys + search_area;
   }
@@ -456,7 +455,7 @@ constexpr int kJoinMinBlocks = CCR_JOIN_MIN_BLOCKS;  // resident blocks per SM t
 template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, bool MERGE, bool PADDED = false>
 __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const JoinArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const TileLayout lay(a.tile, SECOND, MERGE || a.stash, a.search_area);
+  const TileLayout lay(a.tile, SECOND, MERGE, a.search_area);
   int* s_idx = reinterpret_cast<int*>(smem + lay.off_idx);
   int* s_pos = reinterpret_cast<int*>(smem + lay.off_pos);
   int4* s_apos = reinterpret_cast<int4*>(smem + lay.off_apos);
@@ -488,30 +487,6 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
   const long long j0 = min(a.total, static_cast<long long>(blockIdx.x) * per * 32);
   const long long j1 = min(a.total, j0 + per * 32);
   if (j0 >= j1) return;
-  // The positions and author ids of the first sub-tile do not depend on the request they belong to: they are fetched
-  // here, beside the offsets and the staging of the keys, and kept in the thread's own slots of the resolved arrays.
-  if (!MERGE && a.stash) {
-    // (padded output: a.total may be an upper bound, the list ends where the last request does)
-    const long long j_lim = PADDED ? min(j1, static_cast<long long>(gload(a.cand_offsets + a.n_req))) : j1;
-    const int n0 = static_cast<int>(min(static_cast<long long>(a.tile), max(j_lim - j0, 0LL)));
-    for (int base = 0; base < n0; base += kThreads * kUnroll) {
-      int idx[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int i = base + u * kThreads + tid;
-        idx[u] = i < n0 ? gload(a.cand_idx + j0 + i) : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int i = base + u * kThreads + tid;
-        if (i < n0) {
-          if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
-          s_idx[i] = idx[u];
-          s_auth[i] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
-        }
-      }
-    }
-  }
   int r = a.n_req == 1 ? 0 : request_of(a.cand_offsets, a.n_req, j0);
 
   long long seg = j0;
@@ -548,24 +523,15 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
         for (int base = 0; base < n; base += kThreads * kUnroll) {
           int idx[kUnroll];
           int64_t auth[kUnroll];
-          if (sub == j0 && a.stash) {  // fetched above
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-              const int i = base + u * kThreads + tid;
-              idx[u] = i < n ? s_idx[i] : -1;
-              auth[u] = i < n ? s_auth[i] : -1;
-            }
-          } else {
+          for (int u = 0; u < kUnroll; ++u) {
+            const int i = base + u * kThreads + tid;
+            idx[u] = i < n ? gload(a.cand_idx + sub + i) : -1;
+          }
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-              const int i = base + u * kThreads + tid;
-              idx[u] = i < n ? gload(a.cand_idx + sub + i) : -1;
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-              if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
-              auth[u] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
-            }
+          for (int u = 0; u < kUnroll; ++u) {
+            if (idx[u] < 0 || idx[u] >= a.n_docs) idx[u] = -1;  // unresolved / out-of-range position
+            auth[u] = idx[u] >= 0 ? load_author(a, idx[u]) : -1;
           }
           bool found[kUnroll];
           int pos[kUnroll];
