@@ -349,7 +349,8 @@ ccr_status ccr_workspace_outputs(const ccr_workspace* ws, void** rows, uint8_t**
  * copies the inputs to the workspace, runs ccr_join_batch, copies rows and mask back — all enqueued
  * on `stream`, nothing synchronised.  Pinned host memory makes the copies asynchronous; a payload whose arrays
  * are all pinned and 16-byte aligned is fetched by one kernel instead of one copy per array.
- * total_edges = edge_offsets[n_req].  Sizes beyond the workspace give CCR_ERR_INVALID_ARG.
+ * total_edges = edge_offsets[n_req].  Sizes beyond the workspace give CCR_ERR_INVALID_ARG; with a store other than the one the
+ * workspace was created for (same device), its edge, request and output rows must fit the workspace's buffers in bytes.
  * A batch of at least three requests and 786,432 candidates is pipelined: the requests are cut into three
  * groups of about equal candidate counts, and a group's payload crosses PCIe on a stream the workspace owns while
  * the groups already on the device are joined on `stream` (events order the two; results are those of one

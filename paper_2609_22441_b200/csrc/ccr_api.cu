@@ -1503,6 +1503,11 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
   if (!scope.ok) return CCR_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t out_b = out_row_bytes(s, flags);
+  // the workspace may have been sized for a store with other widths: what counts is the bytes
+  if (static_cast<size_t>(total_edges) * s->edge_b > static_cast<size_t>(w->max_edges) * w->edge_b ||
+      static_cast<size_t>(n_req) * s->req_b > static_cast<size_t>(w->max_req) * w->req_b ||
+      static_cast<size_t>(total_cands) * out_b > static_cast<size_t>(w->max_cands) * w->out_b_max)
+    return CCR_ERR_INVALID_ARG;
   bool ok = true;
   // A batch of several large requests is pipelined: its requests are cut into up to kHostGroups groups of about
   // equal candidate counts; group g + 1 crosses PCIe on the workspace's copy stream while group g is joined on the
@@ -1516,7 +1521,7 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
   }
   bool by_kernel = false;
   if (n_groups == 1) {
-    const size_t sz_keys = static_cast<size_t>(total_edges) * 8, sz_feats = static_cast<size_t>(total_edges) * w->edge_b;
+    const size_t sz_keys = static_cast<size_t>(total_edges) * 8, sz_feats = static_cast<size_t>(total_edges) * s->edge_b;
     const size_t sz_off = (static_cast<size_t>(n_req) + 1) * 8, sz_idx = static_cast<size_t>(total_cands) * 4;
     const size_t sz_req = static_cast<size_t>(n_req) * s->req_b;
     SegmentCopy in(sz_keys + sz_feats + 2 * sz_off + sz_idx + sz_req);
@@ -1585,22 +1590,22 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
       const int64_t c0 = cand_offsets[r0], c1 = cand_offsets[r1], e0 = edge_offsets[r0], e1 = edge_offsets[r1];
       if (e1 > e0) {
         ok = ok && cudaMemcpyAsync(w->edge_keys + e0, edge_keys + e0, (e1 - e0) * 8, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
-        ok = ok && cudaMemcpyAsync(w->edge_feats + e0 * w->edge_b, static_cast<const uint8_t*>(edge_feats) + e0 * w->edge_b,
-                                   (e1 - e0) * w->edge_b, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
+        ok = ok && cudaMemcpyAsync(w->edge_feats + e0 * s->edge_b, static_cast<const uint8_t*>(edge_feats) + e0 * s->edge_b,
+                                   (e1 - e0) * s->edge_b, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
       }
       if (c1 > c0)
         ok = ok && cudaMemcpyAsync(w->cand_idx + c0, cand_idx + c0, (c1 - c0) * 4, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
       if (s->req_b > 0)
-        ok = ok && cudaMemcpyAsync(w->req_feats + static_cast<size_t>(r0) * w->req_b,
-                                   static_cast<const uint8_t*>(req_feats) + static_cast<size_t>(r0) * w->req_b,
-                                   static_cast<size_t>(r1 - r0) * w->req_b, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
+        ok = ok && cudaMemcpyAsync(w->req_feats + static_cast<size_t>(r0) * s->req_b,
+                                   static_cast<const uint8_t*>(req_feats) + static_cast<size_t>(r0) * s->req_b,
+                                   static_cast<size_t>(r1 - r0) * s->req_b, cudaMemcpyHostToDevice, w->copy_stream) == cudaSuccess;
       ok = ok && cudaEventRecord(w->ev_group[g], w->copy_stream) == cudaSuccess;
       ok = ok && cudaStreamWaitEvent(st, w->ev_group[g], 0) == cudaSuccess;
       if (!ok) break;
       if (c1 > c0) {
         const ccr_status js = ccr_join_batch(s, r1 - r0, c1 - c0, max_edge_len, w->edge_keys, w->edge_feats, w->edge_offsets + r0,
                                              w->cand_idx + c0, w->cand_offsets + group_off[g],
-                                             s->req_b ? w->req_feats + static_cast<size_t>(r0) * w->req_b : nullptr,
+                                             s->req_b ? w->req_feats + static_cast<size_t>(r0) * s->req_b : nullptr,
                                              w->out_rows + static_cast<size_t>(c0) * out_b, w->out_mask + c0, flags, stream);
         if (js != CCR_OK) return js;
       }

@@ -63,3 +63,46 @@ def test_payload_in_any_host_memory(n_req, n_cand, second, how, lead, entry):
     assert store.device_status() == B.CCR_OK
     ws.free()
     store.free()
+
+
+@pytest.mark.parametrize("n_req,n_cand", [(2, 900), (3, 262_200)])  # one group of requests, three pipelined ones
+def test_a_workspace_of_another_store(n_req, n_cand):
+    """A workspace serves any store whose rows fit its buffers; rows that do not are refused before anything is enqueued."""
+    from paper_2609_22441_b200 import binding as B
+
+    def workload(seed, edge_dim, req_dim):
+        rng = np.random.default_rng(seed)
+        st = W.make_store(rng, 40_000, 120_000, 8, np.float32)
+        lists = [W.make_viewer(rng, 120_000, int(k), edge_dim, np.float16) for k in rng.integers(50, 700, size=n_req)]
+        cands = [rng.integers(0, st.n_docs, size=n_cand).astype(np.int32) for _ in range(n_req)]
+        req = rng.standard_normal((n_req, req_dim)).astype(np.float32)
+        return W.Workload("w", seed, st, W.assemble_batch([k for k, _ in lists], [f for _, f in lists], cands, req, edge_dim, np.float16, req_dim, np.float32))
+
+    def call(store, ws, wl, mask, rows):
+        b = wl.batch
+        B.ccr_join_batch_host(store, ws, b.n_req, b.total_cands, b.max_edge_len, int(b.edge_offsets[-1]), b.edge_keys, b.edge_feats.view(np.uint8), b.edge_offsets,
+                              b.cand_idx, b.cand_offsets, b.req_feats, rows, mask)
+        torch.cuda.synchronize()
+
+    narrow, wide_req, wide_edge = workload(1, 8, 4), workload(2, 8, 24), workload(3, 64, 4)
+    stores = {id(w): B.store_from_workload(w) for w in (narrow, wide_req, wide_edge)}
+    mask = np.zeros(n_req * n_cand, np.uint8)
+    big = B.Workspace(stores[id(wide_edge)], n_req, n_req * n_cand, max(int(w.batch.edge_offsets[-1]) for w in (narrow, wide_edge)))
+    for wl in (narrow, wide_edge):
+        rows = np.zeros((n_req * n_cand, stores[id(wl)].out_row_bytes(0)), np.uint8)
+        call(stores[id(wl)], big, wl, mask, rows)
+        want_rows, want_mask = oracle.join_workload(wl, n_threads=4)
+        assert np.array_equal(mask, want_mask) and np.array_equal(rows, want_rows)
+    # request rows of 96 bytes where 16 were sized for (the output rows fit), edge rows of 128 where 16 were
+    small = B.Workspace(stores[id(narrow)], n_req, 64 * n_req * n_cand, 700 * n_req) if n_cand < 1000 else None
+    for ws, wl in ((big, wide_req), (small, wide_edge)):
+        if ws is None:
+            continue
+        rows = np.full((n_req * n_cand, stores[id(wl)].out_row_bytes(0)), 7, np.uint8)
+        with pytest.raises(B.CcrError) as e:
+            call(stores[id(wl)], ws, wl, mask, rows)
+        assert e.value.status == B.CCR_ERR_INVALID_ARG and (rows == 7).all()
+        ws.free()
+    for st in stores.values():
+        assert st.device_status() == B.CCR_OK
+        st.free()
