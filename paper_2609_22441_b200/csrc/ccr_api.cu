@@ -981,11 +981,14 @@ ccr_status ccr_docstore_selftest_wait(ccr_docstore* s, void* stream) {
 namespace {
 // ccr_join_batch (n_max == 0, ragged output) and ccr_join_batch_padded (n_max > 0) share everything but the
 // output addressing.
+// read_ahead false: the launch directly in front is a kernel that writes the inputs.  Its end is no point at which its writes are
+// promised to be visible to a launch that has not executed griddepcontrol.wait, so the warp-specialised kernel, which reads its
+// inputs before it waits, is then launched in plain stream order.
 ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands, int64_t max_edge_len,
                      const int64_t* edge_keys, const void* edge_feats, const int64_t* edge_offsets,
                      const int32_t* cand_idx, const int64_t* cand_offsets, const void* req_feats,
                      void* out_rows, uint8_t* out_mask, uint32_t flags, void* stream, int64_t n_max,
-                     const void* member_emb, int* sched_override = nullptr) {
+                     const void* member_emb, int* sched_override = nullptr, bool read_ahead = true) {
   if (!good(cs)) return CCR_ERR_BAD_HANDLE;
   ccr_docstore* s = const_cast<ccr_docstore*>(cs);  // only the launch counter and status words change
   if (n_req < 0 || total_cands < 0 || max_edge_len < 0) return CCR_ERR_INVALID_ARG;
@@ -1214,7 +1217,7 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = (flags & CCR_FLAG_NO_OVERLAP) ? 0 : 1;
+    cfg.numAttrs = ((flags & CCR_FLAG_NO_OVERLAP) || !read_ahead) ? 0 : 1;
     if (cudaLaunchKernelEx(&cfg, fn, a, n_str) != cudaSuccess) {
       cudaGetLastError();
       return CCR_ERR_CUDA;
@@ -1550,9 +1553,10 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
       cudaGetLastError();
       return CCR_ERR_CUDA;
     }
-    const ccr_status js = ccr_join_batch(s, n_req, total_cands, max_edge_len, w->edge_keys, w->edge_feats, w->edge_offsets,
-                                         w->cand_idx, w->cand_offsets, s->req_b ? w->req_feats : nullptr, w->out_rows,
-                                         w->out_mask, flags, stream);
+    if (flags & CCR_FLAG_COSINE) return CCR_ERR_INVALID_ARG;  // the member embeddings come through ccr_join_batch_ex
+    const ccr_status js = join_impl(s, n_req, total_cands, max_edge_len, w->edge_keys, w->edge_feats, w->edge_offsets, w->cand_idx,
+                                    w->cand_offsets, s->req_b ? w->req_feats : nullptr, w->out_rows, w->out_mask, flags, stream, 0,
+                                    nullptr, nullptr, !by_kernel);
     if (js != CCR_OK) return js;
   } else {
     // group boundaries: request ranges [first[g], first[g + 1]) with about total_cands / n_groups candidates each
@@ -1738,7 +1742,7 @@ ccr_status ccr_join_payload_static(const ccr_docstore* s, int32_t n_req, int64_t
                                   base + o_feats, reinterpret_cast<const int64_t*>(base + o_eo),
                                   reinterpret_cast<const int32_t*>(base + o_idx),
                                   reinterpret_cast<const int64_t*>(base + o_co), s->req_b > 0 ? base + o_req : nullptr,
-                                  out_rows, out_mask, flags, stream, 0, nullptr, reinterpret_cast<int*>(base));
+                                  out_rows, out_mask, flags, stream, 0, nullptr, reinterpret_cast<int*>(base), !in.ok);
   return js;
 }
 
