@@ -419,7 +419,7 @@ ccr_status ccr_join_payload_static(const ccr_docstore* store,
  * last call (the affected rows of that launch were not written).  Clears the word.
  * The bounds-checked build of the library (compiled with -DCCR_DEBUG_BOUNDS; `python -m paper_2609_22441_b200.build
  * --debug-bounds` writes it next to the release build) checks every global address the join, sort, resolve,
- * compaction and upsert kernels compute against the extents of the launch's buffers and leaves out an access that
+ * compaction, upsert and host-payload kernels compute against the extents of the launch's buffers and leaves out an access that
  * falls outside (never a trap).  A join reports CCR_ERR_BOUNDS here; the other calls wait for their kernels and
  * return it as their own status.  The build synchronises in every call and is meant for tests, not for serving.   */
 ccr_status ccr_docstore_device_status(ccr_docstore* store, void* stream);

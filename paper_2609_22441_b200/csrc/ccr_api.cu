@@ -409,6 +409,18 @@ struct SegmentCopy {
     a.bytes[a.n++] = static_cast<long long>(bytes);
     total += bytes;
   }
+#ifdef CCR_DEBUG_BOUNDS
+  // the extents of the segments, the last `shrink` bytes of the last destination left out; waits for what is still checked on `st`
+  bool dbg_register(int* word, cudaStream_t st, int64_t shrink) const {
+    if (cudaStreamSynchronize(st) != cudaSuccess) return false;
+    DbgRegistrar reg;
+    for (int i = 0; i < a.n; ++i) {
+      reg.add(a.src[i], static_cast<size_t>(a.bytes[i]));
+      reg.add(a.dst[i], static_cast<size_t>(i == a.n - 1 ? std::max<int64_t>(a.bytes[i] - shrink, 0) : a.bytes[i]));
+    }
+    return reg.commit(word);
+  }
+#endif
   dim3 grid() const {
     const size_t per_block = static_cast<size_t>(ccr::kCopyThreads) * ccr::kCopyUnroll * 16;
     return dim3(static_cast<unsigned>(std::min<size_t>((total + per_block - 1) / per_block + a.n, 256)));
@@ -1536,6 +1548,9 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
     in.add(w->req_feats, req_feats, sz_req, req_feats);
     by_kernel = in.ok;
     if (by_kernel) {
+#ifdef CCR_DEBUG_BOUNDS
+      if (!in.dbg_register(s->status + 2, st, 0)) return CCR_ERR_CUDA;
+#endif
       // (an ordinary launch: it writes what the join in front of it may still be reading)
       ccr::copy_segments_kernel<<<in.grid(), ccr::kCopyThreads, 0, st>>>(in.a);
       ok = cudaGetLastError() == cudaSuccess;
@@ -1623,10 +1638,17 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
     ok = ok && cudaMemcpyAsync(out_rows, w->out_rows, total_cands * out_b, cudaMemcpyDeviceToHost, st) == cudaSuccess;
   SegmentCopy back(by_kernel ? static_cast<size_t>(total_cands) : SIZE_MAX);
   back.add(out_mask, w->out_mask, static_cast<size_t>(total_cands), out_mask);
-  if (back.ok)
+  if (back.ok) {
+#ifdef CCR_DEBUG_BOUNDS
+    ok = ok && back.dbg_register(s->status + 2, st, s->dbg_shrink_rows);
+#endif
     ok = ok && launch_chained(ccr::copy_segments_kernel, back.grid(), dim3(ccr::kCopyThreads), 0, st, back.a) == cudaSuccess;
-  else
+#ifdef CCR_DEBUG_BOUNDS
+    ok = ok && cudaStreamSynchronize(st) == cudaSuccess;  // the table is one per process: no overlap
+#endif
+  } else {
     ok = ok && cudaMemcpyAsync(out_mask, w->out_mask, total_cands, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+  }
   if (!ok) {
     cudaGetLastError();
     return CCR_ERR_CUDA;
@@ -1718,6 +1740,9 @@ ccr_status ccr_join_payload_static(const ccr_docstore* s, int32_t n_req, int64_t
   in.add(base + o_co, cand_offsets, sz_off, cand_offsets);
   in.add(base + o_req, req_feats, sz_req, req_feats);
   if (in.ok) {
+#ifdef CCR_DEBUG_BOUNDS
+    if (!in.dbg_register(s->status + 2, st, 0)) return CCR_ERR_CUDA;
+#endif
     ccr::copy_segments_kernel<<<in.grid(), ccr::kCopyThreads, 0, st>>>(in.a);
     ok = cudaGetLastError() == cudaSuccess;
   } else {

@@ -46,15 +46,16 @@ __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const CopyA
       len[u] = left < 16 ? static_cast<int>(left) : 16;
       to[u] = a.dst[s] + c * 16;
       from[u] = a.src[s] != nullptr ? a.src[s] + c * 16 : nullptr;
-      if (len[u] == 16 && from[u] != nullptr) {
-        v[u] = __ldcg(reinterpret_cast<const uint4*>(from[u]));
-      }
+      if (len[u] == 16 && from[u] != nullptr && CCR_CHK(from[u], 16)) v[u] = __ldcg(reinterpret_cast<const uint4*>(from[u]));
     }
 #pragma unroll
     for (int u = 0; u < kCopyUnroll; ++u) {
-      if (len[u] == 16) *reinterpret_cast<uint4*>(to[u]) = v[u];
-      else
-        for (int i = 0; i < len[u]; ++i) to[u][i] = from[u] != nullptr ? *reinterpret_cast<const volatile uint8_t*>(from[u] + i) : 0;
+      if (len[u] == 16) {
+        gstore(reinterpret_cast<uint4*>(to[u]), v[u]);
+      } else {
+        for (int i = 0; i < len[u]; ++i)
+          gstore(to[u] + i, from[u] != nullptr && CCR_CHK(from[u] + i, 1) ? *reinterpret_cast<const volatile uint8_t*>(from[u] + i) : 0);
+      }
     }
   }
 }

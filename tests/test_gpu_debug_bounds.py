@@ -126,6 +126,50 @@ print("ok")
     assert out.returncode == 0 and "ok" in out.stdout, out.stdout[-2000:] + out.stderr[-3000:]
 
 
+@pytest.mark.parametrize("files,select", [
+    ("tests/test_gpu_sort_lists.py", "not many_long and (8191 or 12289 or 32768 or longer) and (equal or 48_bits or 49_bits or outlier or any)"),
+    ("tests/test_gpu_resolve_wide.py", "262144 and not 9000000"),
+    ("tests/test_gpu_widths.py", "24-16-0 or 60-32-4 or 104-48-4 or 768"),
+    ("tests/test_gpu_host_payload.py", "any_host_memory and (pinned-0 or mixed)"),
+], ids=lambda x: x.split("/")[-1].split(" ")[0])
+def test_sizes_around_the_kernels_rules_run_clean_under_the_bounds_checked_build(debug_lib, files, select):
+    env = dict(os.environ, CCR_LIB_OVERRIDE=debug_lib)
+    out = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", files, "-k", select], cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)
+    assert out.returncode == 0, out.stdout[-3000:] + out.stderr[-2000:]
+    assert " passed" in out.stdout
+
+
+def test_a_returned_mask_whose_host_buffer_ends_early_is_reported_and_not_overrun(debug_lib):
+    code = r"""
+import numpy as np, torch
+from paper_2609_22441_b200 import binding as B, workloads as W
+assert B.lib().ccr_debug_bounds_enabled() == 1
+wl = W.config1(n_docs=20_000, n_req=2, n_cand=701)
+store, b = B.store_from_workload(wl), wl.batch
+pin = lambda a: torch.from_numpy(np.ascontiguousarray(a).view(np.uint8).reshape(-1)).pin_memory()
+args = [pin(x) for x in (b.edge_keys, b.edge_feats, b.edge_offsets, b.cand_idx, b.cand_offsets, b.req_feats)]
+ws = B.Workspace(store, b.n_req, b.total_cands, len(b.edge_keys))
+def call():
+    mask = torch.full((b.total_cands,), 0xA5, dtype=torch.uint8).pin_memory()
+    B.ccr_join_batch_host(store, ws, b.n_req, b.total_cands, b.max_edge_len, len(b.edge_keys), *args, None, mask)
+    return store.device_status(), mask
+st, want = call()
+assert st == B.CCR_OK and want[-1] != 0xA5
+B.lib().ccr_debug_shrink_outputs(store.handle, 1)
+st, mask = call()
+assert st == B.CCR_ERR_BOUNDS and torch.equal(mask[:-1], want[:-1]) and mask[-1] == 0xA5
+B.lib().ccr_debug_shrink_outputs(store.handle, 0)
+st, mask = call()
+assert st == B.CCR_OK and torch.equal(mask, want)
+ws.free()
+store.free()
+print("ok")
+"""
+    env = dict(os.environ, CCR_LIB_OVERRIDE=debug_lib)
+    out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0 and "ok" in out.stdout, out.stdout[-2000:] + out.stderr[-3000:]
+
+
 def test_release_build_has_no_checks():
     from paper_2609_22441_b200 import binding as B
 
