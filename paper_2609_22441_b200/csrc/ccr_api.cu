@@ -16,6 +16,7 @@
 #include <unordered_set>
 
 #include "ccr_copy.cuh"
+#include "ccr_hostrange.h"
 #include "ccr_join.cuh"
 #include "ccr_pad.cuh"
 #include "ccr_resolve.cuh"
@@ -391,7 +392,7 @@ bool device_reads_host(const void* p, size_t bytes) {
   void* into[5] = {&type, &managed, &device, &start, &size};
   const CUdeviceptr q = reinterpret_cast<CUdeviceptr>(p);
   if (get(5, what, into, q) != CUDA_SUCCESS) return false;
-  return type == CU_MEMORYTYPE_HOST && !managed && device == q && start != 0 && start <= q && bytes <= size && q - start <= size - bytes;
+  return ccr::pinned_range_holds(type == CU_MEMORYTYPE_HOST, managed != 0, device, start, size, q, bytes);
 }
 
 // Copies collected into one launch of copy_segments_kernel.

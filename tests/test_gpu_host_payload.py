@@ -65,6 +65,59 @@ def test_payload_in_any_host_memory(n_req, n_cand, second, how, lead, entry):
     store.free()
 
 
+SWEEP = 256 * 256 * 4 * 16  # bytes of one round of the transfer kernel's grid
+LIMIT = 16 << 20            # larger payloads go by copies
+
+
+def _payload_bytes(n_req, n_cand, k):
+    return n_req * k * 72 + 2 * 8 * (n_req + 1) + n_req * n_cand * 4 + n_req * 64
+
+
+@pytest.mark.parametrize("entry", ["workspace", "static"])
+@pytest.mark.parametrize("n_req,n_cand,k", [(2, 90_000, 300), (3, 500, 19_400), (3, 700, 24_800), (12, 16, 19_416), (12, 17, 19_416), (12, 18, 19_416)])
+def test_payloads_around_the_sizes_of_the_transfer_kernel(n_req, n_cand, k, entry):
+    """Pinned payloads of one and several rounds of the transfer kernel's grid, segments that lie across two rounds, up to and beyond its
+    size limit, and a batch whose join is the warp-specialised one."""
+    from paper_2609_22441_b200 import binding as B
+
+    n_bytes = _payload_bytes(n_req, n_cand, k)
+    assert {19_400: SWEEP < n_bytes < 1.1 * SWEEP, 24_800: SWEEP < n_bytes < 1.4 * SWEEP, 300: n_bytes < SWEEP}.get(k, True)
+    assert k != 19_416 or {16: n_bytes < LIMIT, 17: n_bytes == LIMIT, 18: n_bytes > LIMIT}[n_cand]
+    wls = [W.config1(seed=60 + i, n_docs=40_000 if k > 1000 else 200_000, n_req=n_req, n_cand=n_cand, edge_lo=k, edge_hi=k) for i in range(2)]
+    wls[1].store = wls[0].store
+    store = B.store_from_workload(wls[0])
+    b, out_b = wls[0].batch, store.out_row_bytes(0)
+    assert b.total_cands == n_req * n_cand and len(b.edge_keys) == n_req * k and b.edge_feats.nbytes == n_req * k * 64 and b.req_feats.nbytes == n_req * 64
+    ws = B.Workspace(store, n_req, b.total_cands, len(b.edge_keys))
+    names = ("edge_keys", "edge_feats", "edge_offsets", "cand_idx", "cand_offsets", "req_feats")
+    bufs = [torch.zeros(getattr(b, n).nbytes, dtype=torch.uint8, pin_memory=True) for n in names]
+    mask = torch.zeros(b.total_cands, dtype=torch.uint8, pin_memory=True)
+    rows = torch.zeros((b.total_cands, out_b), dtype=torch.uint8)
+    d_rows, d_mask = torch.zeros((b.total_cands, out_b), dtype=torch.uint8, device="cuda"), torch.zeros(b.total_cands, dtype=torch.uint8, device="cuda")
+    for wl in wls:
+        for n, buf in zip(names, bufs):
+            buf.copy_(torch.from_numpy(np.ascontiguousarray(getattr(wl.batch, n)).reshape(-1).view(np.uint8)))
+        args = (n_req, b.total_cands, k, n_req * k) + tuple(bufs)
+        want_rows, want_mask = oracle.join_workload(wl, n_threads=4)
+        if entry == "workspace":
+            B.ccr_join_batch_host(store, ws, *args, rows, mask)
+            torch.cuda.synchronize()
+            got_rows, got_mask = rows.numpy(), mask.numpy()
+        elif n_bytes > 16_770_000:  # with its roundings it does not fit the fixed block
+            with pytest.raises(B.CcrError) as e:
+                B.ccr_join_payload_static(store, *args, d_rows, d_mask)
+            assert e.value.status == B.CCR_ERR_UNSUPPORTED
+            continue
+        else:
+            B.ccr_join_payload_static(store, *args, d_rows, d_mask)
+            torch.cuda.synchronize()
+            got_rows, got_mask = d_rows.cpu().numpy(), d_mask.cpu().numpy()
+        assert np.array_equal(got_mask, want_mask) and np.array_equal(got_rows, want_rows)
+    assert store.device_status() == B.CCR_OK
+    ws.free()
+    store.free()
+
+
 @pytest.mark.parametrize("n_req,n_cand", [(2, 900), (3, 262_200)])  # one group of requests, three pipelined ones
 def test_a_workspace_of_another_store(n_req, n_cand):
     """A workspace serves any store whose rows fit its buffers; rows that do not are refused before anything is enqueued."""
