@@ -300,19 +300,20 @@ ccr_status ccr_join_batch_ex(const ccr_docstore* store, const ccr_join_io* io, u
  * records [edge_offsets[r], edge_offsets[r+1]) — key int64 + feature row of the store's edge width — are put
  * in ascending key order (records with equal keys keep their input order) into keys_out / feats_out, which
  * use the same offsets and must not alias the inputs.  perm_out (optional, int32[E]) receives for every
- * output record the index of its source record inside the request.  Without perm_out every list is sorted by
- * one 1024-thread block in shared memory (one kernel); lists of more than 19,000 records then have no place to
- * be sorted in and the call returns CCR_ERR_INVALID_ARG.  With perm_out, and max_edge_len above 4,096, lists
- * whose keys leave room for the record index in one 64-bit word (non-negative, below 2^(63 - index bits): every
- * realistic id) are sorted in chunks of 4,096 records by one block each and the sorted chunks merged pairwise,
- * one grid-wide launch per doubling of the run length (the merged words alternate between keys_out and the
- * list's own part of feats_out, which therefore holds scratch data until the end of the call), so that a long
- * list is spread over many SMs instead of one, and the rows of all lists are moved by one grid-wide gather:
- * 3 + ceil(log2(max_edge_len / 4096)) small kernels on `stream` (CCR_ERR_UNSUPPORTED if n_req x the tiles of
- * max_edge_len records exceed the 2^31 - 1 blocks of a grid).
- * A batch in which some key does not leave that room is sorted list by list by the one-block kernel inside the same
- * call (a device-side flag word of the store, taken in turn from 64 such words: at most 64 calls with perm_out may be
- * in flight on one store at once, on any streams).
+ * output record the index of its source record inside the request.  Any key values are sorted.  Two forms, chosen by max_edge_len:
+ *   up to 32,768: every list is radix sorted by a thread-block cluster in shared memory: one kernel, or two when perm_out is given
+ *     and max_edge_len exceeds 512 (the rows then follow the permutation in a launch of their own).  No scratch memory; any
+ *     number of calls may be in flight.
+ *   beyond: perm_out is required.  Lists whose keys leave room for the record index in one 64-bit word (non-negative, below
+ *     2^(63 - index bits): every realistic id) are sorted in chunks of 4,096 records by one block each and the sorted chunks
+ *     merged pairwise, one grid-wide launch per doubling of the run length (the merged words alternate between keys_out and
+ *     the list's own part of feats_out, which therefore holds scratch data until the end of the call); the rows of all lists
+ *     are moved by one grid-wide gather: 3 + ceil(log2(max_edge_len / 4096)) kernels on `stream` (CCR_ERR_UNSUPPORTED if
+ *     n_req x the tiles of max_edge_len records exceed the 2^31 - 1 blocks of a grid).  A batch in which some key does not
+ *     leave that room is sorted list by list by one block each inside the same call (a device-side flag word of the store,
+ *     taken in turn from 64 such words: at most 64 calls of this form may be in flight on one store at once, on any streams).
+ * Without perm_out, max_edge_len beyond 19,000 is refused with CCR_ERR_INVALID_ARG: the limit of the interface since its first form,
+ * kept so that it does not depend on which kernel serves a length.
  * max_edge_len (HOST) must be at least the longest list; a longer list is cut there (its first max_edge_len
  * records are sorted among themselves, the rest of its output is left unwritten) and no access leaves the arrays.
  * All pointers DEVICE; no allocation, no synchronisation.
@@ -347,8 +348,9 @@ ccr_status ccr_workspace_outputs(const ccr_workspace* ws, void** rows, uint8_t**
 
 /* The same join with HOST buffers (the request payload of Section 6.1.3 arrives in host memory):
  * copies the inputs to the workspace, runs ccr_join_batch, copies rows and mask back — all enqueued
- * on `stream`, nothing synchronised.  Pinned host memory makes the copies asynchronous; a payload whose arrays
- * are all pinned and 16-byte aligned is fetched by one kernel instead of one copy per array.
+ * on `stream`, nothing synchronised.  Pinned host memory makes the copies asynchronous; a payload of at most 16 MiB whose arrays are
+ * all pinned and 16-byte aligned is fetched by one kernel instead of one copy per array, and the mask goes back by a kernel as
+ * well when its buffer is pinned and 16-byte aligned (these two are not in ccr_docstore_launch_count; rows always go by a copy).
  * total_edges = edge_offsets[n_req].  Sizes beyond the workspace give CCR_ERR_INVALID_ARG; with a store other than the one the
  * workspace was created for (same device), its edge, request and output rows must fit the workspace's buffers in bytes.
  * A batch of at least three requests and 786,432 candidates is pipelined: the requests are cut into three

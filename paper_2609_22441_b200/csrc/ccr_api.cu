@@ -46,8 +46,15 @@ constexpr size_t kStageBytes = 16u << 20;  // staging block of second-degree sto
 #ifndef CCR_HOST_GROUP_CANDS
 #define CCR_HOST_GROUP_CANDS (2 * kSmallLaunchCands)
 #endif
-// Host payloads up to this size are fetched by one kernel (ccr_copy.cuh), larger ones by the copy engine: the kernel is ahead by the
-// gaps between the copies (3 MB 249 -> 221 us a call), from about 16 MB on the two are level (387 against 398 us, alone 387 / 414).
+// Host payloads up to this size are fetched by one kernel (ccr_copy.cuh), larger ones by the copy engine.  us a call of
+// ccr_join_batch_host, rows left on the device, copies / kernel, for pinned buffers that the host has rewritten before every call (back to
+// back over a ring of them; one call at a time) and for buffers that the device has never touched (back to back; one at a time):
+//   payload   16 KB   48 / 16    57 / 29    48 / 18    56 / 30         4.2 MB  254 / 179   230 / 179   174 / 158   188 / 173
+//            256 KB   58 / 24    71 / 41    61 / 28    70 / 40         6.3 MB  312 / 249   337 / 251   253 / 238   260 / 252
+//            1.0 MB   89 / 63   120 / 81    92 / 65   106 / 80        12.7 MB  471 / 413   531 / 412   410 / 405   409 / 410
+//            2.0 MB  161 / 111  165 / 128  134 / 116  202 / 147       19.2 MB  646 / 554   649 / 546   548 / 550   532 / 537
+// Ahead by the gaps between the copies, and on fresh data by what the copy engine takes to read it; level on untouched buffers from
+// about 13 MB on, hence the limit.
 constexpr size_t kKernelCopyBytes = 16u << 20;
 constexpr int kHostGroups = CCR_HOST_GROUPS;         // most request groups of a pipelined host-buffer join
 constexpr int kSchedRegions = 64;                    // launches of one store that may be in flight at once

@@ -118,10 +118,12 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int n) {
 }
 
 // 16-byte chunks a lane has in flight while it moves rows of run-time widths: as many loads as a warp of the tuned
-// variants keeps (16 + 4).  592-byte rows, 37 x 17,003 candidates: one chunk at a time with a division per chunk
-// 198 us, 8 / 12 / 16 / 20 / 24 in flight 142 / 137 / 133 / 123 / 132 us; batches of equal length (13 + 12 + 12 chunks
-// of 37 instead of 20 + 17) 138 us.  Second-degree joins and
-// the cosine section keep more beside the loads and have the registers for 8.
+// variants keeps (16 + 4).  37 x 17,003 candidates, us with 12 / 16 / 20 / 24 in flight, by the 16-byte chunks of a row:
+//   11  52.3 /  54.4 /  55.0 /  57.1      24   83.9 /  88.0 /  91.5 /  85.4      32  115.9 / 110.0 / 112.4 / 120.5
+//   37   137 /   134 /   123 /   132      45  153.5 / 148.6 / 152.0 / 147.9      72    210 /   210 /   203 /   205
+// No number is the best for all (what counts is how a row's chunks divide into batches: 37 as 20 + 17 beats 13 + 12 + 12, 138 us);
+// 20 has the smallest sum and is within 9 % of the best everywhere.  One chunk at a time with a division per chunk took 198 us
+// at 37.  Second-degree joins and the cosine section keep more beside the loads and have the registers for 8.
 constexpr int kGenericUnroll = 20;
 constexpr int kGenericUnrollSecond = 8;
 constexpr int kGenericUnrollSecondTwoPhase = 12;  // the two-phase kernel's 128 registers hold more (16 was no faster)

@@ -15,8 +15,8 @@
 // by the windows' traffic and by instruction issue rather than by the chain of rounds; there a warp takes 32 queries at
 // a time, searches the staged level a lane per query (the same instructions serve 32 queries instead of 8) and hands the
 // queries to the lane groups by shuffles, four per group in flight; see kResolveWarpMin.  Measured and slower: wider windows (128 bytes with eight lanes
-// per query; 256 bytes in two rounds), a lane per query with 1-8 queries in flight, and a larger staged top
-// level (it takes shared memory from the L1 and start-up time from every block).
+// per query; 256 bytes in two rounds), a lane per query with 1-8 queries in flight, and, with eight blocks per SM as small
+// batches have them, a larger staged top level (it takes shared memory from the L1 and start-up time from every block).
 #pragma once
 
 #include "ccr_device.cuh"
