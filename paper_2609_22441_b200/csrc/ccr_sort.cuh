@@ -283,24 +283,29 @@ __device__ __forceinline__ void sort_words_merge128(unsigned long long* w, int n
   merge_passes<4>(w, n, 128);
 }
 
-// Rows follow their keys: output chunk c (16 bytes) comes from row source_of(c / row_ch) of the input.  One block
-// moves a whole list, so every thread keeps kSortGatherUnroll loads in flight.
+// Rows follow their keys: output chunk c (16 bytes) comes from row source_of(c / row_ch) of the input.  One block moves the rows of
+// n records, every thread with kSortGatherUnroll loads in flight; a thread steps from chunk to chunk by additions.
 constexpr int kSortGatherUnroll = 8;
 template <typename SourceOf>
-__device__ __forceinline__ void gather_rows(const uint4* src, uint4* dst, long long chunks, int row_ch, SourceOf source_of) {
-  for (long long c0 = threadIdx.x; c0 < chunks; c0 += static_cast<long long>(blockDim.x) * kSortGatherUnroll) {
+__device__ __forceinline__ void gather_rows(const uint4* src, uint4* dst, int n, int row_ch, SourceOf source_of) {
+  const int threads = static_cast<int>(blockDim.x), step_row = threads / row_ch, step_piece = threads - step_row * row_ch;
+  int row = static_cast<int>(threadIdx.x) / row_ch, piece = static_cast<int>(threadIdx.x) - row * row_ch;
+  const long long chunks = static_cast<long long>(n) * row_ch;
+  for (long long c0 = threadIdx.x; c0 < chunks; c0 += static_cast<long long>(threads) * kSortGatherUnroll) {
     uint4 v[kSortGatherUnroll];
 #pragma unroll
     for (int u = 0; u < kSortGatherUnroll; ++u) {
-      const long long c = c0 + static_cast<long long>(u) * blockDim.x;
-      if (c < chunks) {
-        const int row = static_cast<int>(c / row_ch), piece = static_cast<int>(c - static_cast<long long>(row) * row_ch);
-        v[u] = ldg128(src + source_of(row) * row_ch + piece);
+      if (row < n) v[u] = ldg128(src + source_of(row) * row_ch + piece);
+      row += step_row;
+      piece += step_piece;
+      if (piece >= row_ch) {
+        piece -= row_ch;
+        ++row;
       }
     }
 #pragma unroll
     for (int u = 0; u < kSortGatherUnroll; ++u) {
-      const long long c = c0 + static_cast<long long>(u) * blockDim.x;
+      const long long c = c0 + static_cast<long long>(u) * threads;
       if (c < chunks) st128_stream(dst + c, v[u]);
     }
   }
@@ -650,26 +655,40 @@ __global__ void __launch_bounds__(kSortGatherThreads) gather_all_kernel(const So
 // that owns the place — the lanes that share a digit found with one ballot per digit bit.  Keys whose differing bits
 // leave no room for the index (the far outlier of a clustered list is enough) are sorted in two rounds: by their low 32
 // bits, then by the rest.
+// Five passes and more are replaced by three over a prefix of the differing bits when few records share one (every warp looks at 32
+// records: four with the same prefix say no); the records that do share one are then put in order by comparing each with its
+// neighbours, and a list where more than 64 do after all takes every pass.  Spread keys cost the same whatever their range is: one list of
+// 4,096 records over 2^26 / 2^40 / 2^64 21.2 / 22.5 / 23.4 us (a pass per digit: 23.7 / 31.7 / 48.9; chunks and merges 30.5 /
+// 30.5 / 73.1), 16 lists of 20,000 34.5 / 40.5 / 44.0 us (37.1 / 48.0 / 75.4; 55.7 / 55.7 / 651).  From four passes on, or by two
+// digits, it does not pay: the comparing costs more than a pass (production batch 98 and 104 us).
 // A pass is bound by instruction issue (about 50 instructions a word and pass; over 20,000 words on one SM 11 us), hence
 // the cluster: a list takes as many blocks as hold it, the others of its cluster leave at once.  Blocks of up to 4,096
-// records each, 3 resident per SM at 80 registers: with 1,024 / 2,048 / 3,072 wanted per block the 256-list batch below
-// takes 104 / 100 / 97 us instead of 94 (cluster barriers and blocks that leave at once), a single list of 20,000 31
-// instead of 34; __match_any_sync for the ballots 99; 64 registers, 4 resident 96.
-// Lists of up to kListNetwork records have too few words for the passes to pay: sorted by sort_words_merge128 instead (256
-// lists of 900-1,000 records, 2^40 keys: 37 -> 29 us; one list of 200 records 12.9 -> 9.7 us).
-// 256 lists <= 20,000 (700,000 records of 128-byte rows): 141 us as chunks and merges, 90 us this way; 4 such lists
-// 38.7 -> 29 us; 64 lists <= 5,000 (61,823 records) 44 -> 28 us; a request flow with 4 lists <= 9,214 that hold a far outlier
-// each 164 -> 92 us.
+// records each, 512 threads of 8 words, 2 resident per SM: a single list of 4,096 records at 2^26 21.2 us against 25.8 with 256
+// threads of 16 words, the 256-list batch below 89.8 against 87.7 (less of a pass is latency, but 8 of a block's warps idle on
+// lists below half its share); less than 4,096 wanted per block is slower (cluster barriers and blocks that leave at once).
+// Lists of up to kListCount records: the place of a record is the number of those in front of it (256 lists of 22 records 9.5 us by the
+// network, or 14.7-22.5 for wide keys, 8.7 us this way).  Up to kListNetwork there are too few words for the passes to pay:
+// sort_words_merge128, once or, for wide keys, once by each half.
+// 256 lists <= 20,000 (700,000 records of 128-byte rows): 141 us as chunks and merges, 90 us this way, at 2^40 94 us.
 constexpr int kListRadixBits = 7, kListDigits = 1 << kListRadixBits;
 constexpr int kListStride = kListDigits + 1;  // counters of a warp; odd, so that the scan's column reads spread over the banks
-constexpr int kListThreads = 256, kListPer = 16, kListWarps = kListThreads / 32;
-constexpr int kListBlockMax = kListThreads * kListPer;  // 4,096 words of a block: 32 registers of a thread
-constexpr int kListNetwork = 1024;  // lists up to this length are sorted as one block's merge sort behind a register network
+constexpr int kListThreads = 512, kListPer = 8, kListWarps = kListThreads / 32;
+constexpr int kListScanThreads = kListWarps / 4;  // threads that share a digit in the scan over the warps' counters
+constexpr int kListBlockMax = kListThreads * kListPer;  // 4,096 words of a block: 16 registers of a thread
+constexpr int kListCount = 256;     // lists up to this length are sorted by counting
+constexpr int kListNetwork = 1024;  // ... up to this length as one block's merge sort behind a register network
 constexpr int kListRowsHere = 512;  // batches of lists up to this length move their rows in the sorting kernel
+// prefix passes: digits of the prefix, fewest passes they replace, most records that share a prefix on either side of one that are still
+// put in order, most of a warp's 32 sampled records that may share one
+constexpr int kListPrefixDigits = 3, kListPrefixMin = 5, kListPrefixTies = 64, kListSampleSame = 3;
+static_assert(kListCount <= kListThreads, "a record per thread");
 static_assert(kListNetwork <= 4 * kListThreads, "sort_words_merge128 takes four words a thread");
+static_assert(kListNetwork + kListNetwork / 2 <= kListBlockMax, "wide keys keep an index per record behind their words");
+static_assert(kListWarps * kListStride * 4 >= kListBlockMax, "the counters' memory holds a byte per word between the passes");
 constexpr int kListMaxCluster = 8;                      // the portable size
 constexpr int kListMax = kListBlockMax * kListMaxCluster;
 static_assert(kListDigits * kListWarps == 4 * kListThreads, "in the scan a thread has four warps' counters of one digit");
+static_assert(kListScanThreads >= 1 && 32 % kListScanThreads == 0, "a digit's counters lie within one warp");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -695,17 +714,25 @@ __device__ __forceinline__ unsigned cluster_ld32(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ unsigned long long cluster_ld64(uint32_t addr) {
+  unsigned long long v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void cluster_st64(uint32_t addr, unsigned long long v) {
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortArgs a) {
+__global__ void __launch_bounds__(kListThreads, 2) sort_lists_kernel(const SortArgs a) {
   chain_enter(a.more_follow != 0);
   __shared__ unsigned long long w[kListBlockMax];
   __shared__ unsigned cnt[kListWarps * kListStride];       // [warp][digit]
   __shared__ unsigned block_count[kListDigits];            // this block's words with each digit, read by the whole cluster
   __shared__ unsigned digit_base[kListDigits];             // place of this block's first word with each digit
-  __shared__ unsigned warp_total[kListWarps], or_bits[2];
+  __shared__ unsigned warp_total[kListWarps], or_bits[2], votes[2];
+  // kept here and not in registers, which the passes need: the list's first record, its first key
+  __shared__ volatile long long s_e0;
+  __shared__ volatile unsigned long long s_key0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const int cs = static_cast<int>(cluster_size()), rank = static_cast<int>(cluster_rank());
@@ -718,6 +745,29 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
   const int R = (K + blocks * kListThreads - 1) / (blocks * kListThreads), per = R * kListThreads;  // words per thread, per block
   const int n = min(per, K - rank * per);  // words of this block
   if (rank >= blocks || n <= 0) return;    // (nobody reads the shared memory of a block without words)
+  if (K <= kListCount) {  // a record per thread: its place is the number of records in front of it
+    const int i = static_cast<int>(threadIdx.x);
+    const int64_t k = i < K ? gload(a.keys_in + e0 + i) : 0;
+    if (i < K) w[i] = static_cast<unsigned long long>(k);
+    __syncthreads();
+    if (i < K) {
+      int p = 0;
+#pragma unroll 8
+      for (int j = 0; j < K; ++j) {
+        const int64_t o = static_cast<int64_t>(w[j]);
+        p += (o < k || (o == k && j < i)) ? 1 : 0;
+      }
+      gstore(a.keys_out + e0 + p, k);
+      if (a.perm_out) gstore(a.perm_out + e0 + p, i);
+      cnt[p] = static_cast<unsigned>(i);
+    }
+    if (a.rows_here) {
+      __syncthreads();
+      gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + e0 * a.row_ch, K, a.row_ch,
+                  [&](int row) { return static_cast<long long>(cnt[row]); });
+    }
+    return;
+  }
   const int used_blocks = (K + per - 1) / per;
   auto sync_all = [&]() {
     if (used_blocks > 1) cluster_sync();
@@ -729,6 +779,10 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
 
   constexpr unsigned long long kSign = 0x8000000000000000ull;  // signed keys as unsigned words of the same order
   const unsigned long long key0 = static_cast<unsigned long long>(gload(keys)) ^ kSign;
+  if (threadIdx.x == 0) {
+    s_e0 = e0;
+    s_key0 = key0;
+  }
   unsigned long long v[kListPer];
   unsigned lo = 0, hi = 0;
   if (threadIdx.x < 2) or_bits[threadIdx.x] = 0u;
@@ -772,49 +826,125 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
   for (int r = 0; r < kListPer; ++r)
     v[r] = ((v[r] & (two ? 0xffffffffull : suffix)) << idx_bits) | static_cast<unsigned>(rank * per + first + 32 * r);
 
-  const bool network = K <= kListNetwork && used_blocks == 1 && !two;
+  const auto key_at = [&](unsigned i) { return static_cast<unsigned long long>(gload(a.keys_in + s_e0 + i)) ^ kSign; };
+  const bool network = K <= kListNetwork;
   if (network) {
+    unsigned* from = reinterpret_cast<unsigned*>(w + kListNetwork);  // wide keys: the record at each place of the first round
+    for (int round = 0;; ++round) {
 #pragma unroll
-    for (int r = 0; r < kListPer; ++r)
-      if (r < R && first + 32 * r < n) w[first + 32 * r] = v[r];
-    __syncthreads();
-    sort_words_merge128(w, n);
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) w[first + 32 * r] = v[r];
+      __syncthreads();
+      sort_words_merge128(w, n);
 #pragma unroll
-    for (int r = 0; r < kListPer; ++r)
-      if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
-  }
-  for (int round = 0; round < (network ? 0 : (two ? 2 : 1)); ++round) {
-    if (round == 1) {
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
+      if (!two || round == 1) break;
+      // sorted by the low half; the second round is by the high half and, so that equal ones keep this order, the place
 #pragma unroll
       for (int r = 0; r < kListPer; ++r) {
         if (r < R && first + 32 * r < n) {
           const unsigned i = static_cast<unsigned>(v[r]) & low;
-          v[r] = (((static_cast<unsigned long long>(gload(keys + i)) ^ kSign) >> 32) << idx_bits) | i;
+          from[first + 32 * r] = i;
+          v[r] = ((key_at(i) >> 32) << idx_bits) | static_cast<unsigned>(first + 32 * r);
         }
       }
     }
-    const unsigned long long bits = !two ? used : (round == 0 ? used & 0xffffffffull : used >> 32);
-    for (int bit = 0; bit < 64 && (bits >> bit) != 0; bit += kListRadixBits) {
-      if (((bits >> bit) & (kListDigits - 1)) == 0) continue;
-      const int shift = idx_bits + bit;
+    if (two) {
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) v[r] = from[static_cast<unsigned>(v[r]) & low];  // (the key is read from the input below)
+    }
+  }
+  // the words of the records this thread holds: key bits of `mask`, those below `base` left out
+  const auto make_words = [&](unsigned long long mask, int base) {
+#pragma unroll
+    for (int r = 0; r < kListPer; ++r) {
+      if (r < R && first + 32 * r < n) {
+        const unsigned i = static_cast<unsigned>(v[r]) & low;
+        v[r] = (((key_at(i) & mask) >> base) << idx_bits) | i;
+      }
+    }
+  };
+  const auto any_of_list = [&](bool mine, int slot) -> bool {
+    const int here = __syncthreads_or(mine);
+    if (used_blocks == 1) return here != 0;
+    if (threadIdx.x == 0) votes[slot] = static_cast<unsigned>(here);
+    cluster_sync();
+    const unsigned x = lane < used_blocks ? cluster_ld32(cluster_addr(smem_u32(votes + slot), static_cast<uint32_t>(lane))) : 0u;
+    return __any_sync(kFull, x != 0);
+  };
+  const auto put_word = [&](unsigned p, unsigned long long x) {  // to place p of the list
+    if (used_blocks > 1) {
+      const unsigned q = __umulhi(p, per_inv);
+      cluster_st64(cluster_addr(smem_u32(w + (p - q * per)), q), x);
+    } else {
+      w[p] = x;
+    }
+  };
+  const auto word_at = [&](unsigned p) {
+    if (used_blocks == 1) return w[p];
+    const unsigned q = __umulhi(p, per_inv);
+    return q == static_cast<unsigned>(rank) ? w[p - q * per] : cluster_ld64(cluster_addr(smem_u32(w + (p - q * per)), q));
+  };
+  const auto digits_of = [](unsigned long long m) {
+    int c = 0;
+    for (; m != 0; ++c) m &= ~(static_cast<unsigned long long>(kListDigits - 1) << (__ffsll(static_cast<long long>(m)) - 1));
+    return c;
+  };
+
+  const unsigned long long low_used = two ? used & 0xffffffffull : used;
+  const int passes = network ? 0 : digits_of(low_used) + (two ? digits_of(used >> 32) : 0);
+  int drop = 0, cut = 0;  // prefix passes: key bits left out of the word to make room for the index, lowest key bit of the prefix
+  bool prefix = passes >= kListPrefixMin;
+  if (prefix) {
+    unsigned long long m = used;
+#pragma unroll
+    for (int d = 0; d < kListPrefixDigits; ++d) {
+      if (m != 0) cut = max(64 - kListRadixBits - __clzll(static_cast<long long>(m)), 0);
+      m &= (1ull << cut) - 1;
+    }
+    drop = two ? 1 + idx_bits - __clzll(static_cast<long long>(used)) : 0;
+    prefix = cut >= drop;
+  }
+  if (prefix) {
+    const bool live = first < n;
+    unsigned long long t = ~static_cast<unsigned long long>(lane);
+    if (live) t = two ? (key_at(static_cast<unsigned>(rank * per + first)) & suffix) >> cut : v[0] >> (idx_bits + cut);
+    prefix = !any_of_list(__popc(__match_any_sync(kFull, t)) > kListSampleSame, 0);
+    if (prefix && two) make_words(suffix, drop);
+  }
+  for (int round = 0; passes > 0; ++round) {
+    if (round == 1) make_words(~0ull << 32, 32);
+    const int base = prefix ? drop : (round == 1 ? 32 : 0);  // the key bit that is the word's lowest
+    unsigned long long bits = (prefix ? (used >> cut) << cut : (round == 1 ? used : low_used)) >> base;
+    while (bits != 0) {
+      const int bit = __ffsll(static_cast<long long>(bits)) - 1, shift = idx_bits + bit;
+      bits &= ~(static_cast<unsigned long long>(kListDigits - 1) << bit);
       for (int t = threadIdx.x; t < kListWarps * kListStride; t += kListThreads) cnt[t] = 0u;
       __syncthreads();
 #pragma unroll
       for (int r = 0; r < kListPer; ++r)
         if (r < R && first + 32 * r < n) atomicAdd(cnt + warp * kListStride + (static_cast<unsigned>(v[r] >> shift) & (kListDigits - 1)), 1u);
       __syncthreads();
-      // counts -> places: a thread has four warps' counters of digit d; two neighbouring threads share a digit
-      const int d = threadIdx.x >> 1, w0 = (threadIdx.x & 1) * 4;
+      // counts -> places: a thread has four warps' counters of digit d; kListScanThreads neighbouring threads share a digit
+      const int d = threadIdx.x / kListScanThreads, part = threadIdx.x % kListScanThreads, w0 = part * 4;
       unsigned c[4], sum = 0;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         c[j] = cnt[(w0 + j) * kListStride + d];
         sum += c[j];
       }
-      const unsigned other = __shfl_xor_sync(kFull, sum, 1);
-      if (w0 == 0) block_count[d] = sum + other;
+      unsigned upto = sum;  // words with digit d of this thread's warps and the ones before them
+#pragma unroll
+      for (int s = 1; s < kListScanThreads; s <<= 1) {
+        const unsigned t = __shfl_up_sync(kFull, upto, s);
+        if (part >= s) upto += t;
+      }
+      const unsigned in_block = __shfl_sync(kFull, upto, lane | (kListScanThreads - 1));
+      if (part == 0) block_count[d] = in_block;
       sync_all();
-      unsigned total = sum + other, before_me = 0;  // words with digit d in the list, in the blocks before this one
+      unsigned total = in_block, before_me = 0;  // words with digit d in the list, in the blocks before this one
       if (used_blocks > 1) {
         total = 0;
         const uint32_t mine = smem_u32(block_count + d);
@@ -827,7 +957,7 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
           }
         }
       }
-      unsigned incl = w0 == 0 ? total : 0u;  // one of the two threads of a digit carries it
+      unsigned incl = part == 0 ? total : 0u;  // one of the threads of a digit carries it
       const unsigned own = incl;
 #pragma unroll
       for (int s = 1; s < 32; s <<= 1) {
@@ -837,9 +967,9 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
       if (lane == 31) warp_total[warp] = incl;
       __syncthreads();
       const unsigned warps_before = __reduce_add_sync(kFull, lane < warp ? warp_total[lane & (kListWarps - 1)] : 0u);
-      if (w0 == 0) digit_base[d] = warps_before + incl - own + before_me;
+      if (part == 0) digit_base[d] = warps_before + incl - own + before_me;
       __syncwarp();
-      unsigned at = digit_base[d] + (w0 == 0 ? 0u : other);
+      unsigned at = digit_base[d] + upto - sum;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         cnt[(w0 + j) * kListStride + d] = at;
@@ -865,37 +995,81 @@ __global__ void __launch_bounds__(kListThreads, 3) sort_lists_kernel(const SortA
           __syncwarp();
           if (live) {
             const unsigned p = start + before;
-            if (used_blocks > 1) {
-              const unsigned q = __umulhi(p, per_inv);
-              cluster_st64(cluster_addr(smem_u32(w + (p - q * per)), q), v[r]);
-            } else {
-              w[p] = v[r];
-            }
+            put_word(p, v[r]);
           }
         }
       }
       sync_all();
 #pragma unroll
       for (int r = 0; r < kListPer; ++r)
-        if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
-      // (the next pass writes any block's w only behind a barrier that every block reaches after these loads)
+        if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];      // (the next pass writes any block's w only behind a barrier that every block reaches after these loads)
     }
+    if (!prefix) {
+      if (!two || round == 1) break;
+      continue;
+    }
+    // Words with the same prefix stand together.  Each counts those in front of it that belong behind it, and the reverse.
+    const int tie = idx_bits + cut - drop;
+    signed char* moved = reinterpret_cast<signed char*>(cnt);  // by how many places; a byte per word of the block
+    bool too_many = false;
+#pragma unroll 4
+    for (int r = 0; r < R; ++r) {
+      const int e = first + 32 * r, p = rank * per + e;
+      if (e >= n) break;
+      const unsigned long long x = w[e];
+      const unsigned long long before = e > 0 ? w[e - 1] : (rank > 0 ? word_at(static_cast<unsigned>(p - 1)) : ~x);
+      const unsigned long long after = e < n - 1 ? w[e + 1] : (p < K - 1 ? word_at(static_cast<unsigned>(p + 1)) : ~x);
+      int by = 0;
+      if ((before >> tie) == (x >> tie) || (after >> tie) == (x >> tie)) {
+        for (int side = -1; side <= 1; side += 2) {
+          for (int q = p + side; q >= 0 && q < K; q += side) {
+            const unsigned long long u = word_at(static_cast<unsigned>(q));
+            if ((u >> tie) != (x >> tie)) break;
+            if (side * (q - p) > kListPrefixTies) {
+              too_many = true;
+              break;
+            }
+            bool u_first = u < x;
+            if (drop > 0 && (u >> idx_bits) == (x >> idx_bits)) {  // the bits that were left out decide
+              const unsigned long long ku = key_at(static_cast<unsigned>(u) & low), kx = key_at(static_cast<unsigned>(x) & low);
+              u_first = ku != kx ? ku < kx : u_first;
+            }
+            if (u_first == (side > 0)) by += side;
+          }
+        }
+      }
+      moved[e] = static_cast<signed char>(by);
+    }
+    if (!any_of_list(too_many, 1)) {
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) put_word(static_cast<unsigned>(rank * per + first + 32 * r + moved[first + 32 * r]), v[r]);
+      sync_all();
+#pragma unroll
+      for (int r = 0; r < kListPer; ++r)
+        if (r < R && first + 32 * r < n) v[r] = w[first + 32 * r];
+      break;
+    }
+    // too many share a prefix after all: all passes, from the words as they stand (equal keys have kept their order)
+    prefix = false;
+    make_words(two ? 0xffffffffull : suffix, 0);
+    round = -1;
   }
 #pragma unroll
   for (int r = 0; r < kListPer; ++r) {
     const int e = first + 32 * r;
     if (r < R && e < n) {
       const unsigned i = static_cast<unsigned>(v[r]) & low;
-      const long long k = two ? gload(keys + i) : static_cast<long long>(((key0 & ~suffix) | (v[r] >> idx_bits)) ^ kSign);
-      gstore(a.keys_out + e0 + rank * per + e, k);
-      if (a.perm_out) gstore(a.perm_out + e0 + rank * per + e, static_cast<int>(i));
+      const long long k = two ? static_cast<long long>(key_at(i) ^ kSign) : static_cast<long long>(((s_key0 & ~suffix) | (v[r] >> idx_bits)) ^ kSign);
+      gstore(a.keys_out + s_e0 + rank * per + e, k);
+      if (a.perm_out) gstore(a.perm_out + s_e0 + rank * per + e, static_cast<int>(i));
       if (a.rows_here) w[e] = v[r];
     }
   }
   if (a.rows_here) {
     __syncthreads();
-    gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + (e0 + rank * per) * a.row_ch,
-                static_cast<long long>(n) * a.row_ch, a.row_ch, [&](int row) { return static_cast<long long>(static_cast<unsigned>(w[row]) & low); });
+    gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + s_e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + (s_e0 + rank * per) * a.row_ch,
+                n, a.row_ch, [&](int row) { return static_cast<long long>(static_cast<unsigned>(w[row]) & low); });
   }
 }
 
@@ -926,7 +1100,7 @@ __global__ void __launch_bounds__(kSortRowsTile) sort_rows_kernel(const SortArgs
     if (static_cast<int>(threadIdx.x) < n) s_src[threadIdx.x] = gload(a.perm_out + e0 + first + threadIdx.x);
     __syncthreads();
     gather_rows(reinterpret_cast<const uint4*>(a.feats_in) + e0 * a.row_ch, reinterpret_cast<uint4*>(a.feats_out) + (e0 + first) * a.row_ch,
-                static_cast<long long>(n) * a.row_ch, a.row_ch, [&](int row) { return static_cast<long long>(s_src[row]); });
+                n, a.row_ch, [&](int row) { return static_cast<long long>(s_src[row]); });
     __syncthreads();  // s_src is rewritten by the next item
   }
 }

@@ -100,3 +100,77 @@ def test_many_long_lists_of_equal_keys():
         assert np.array_equal(k_out.cpu().numpy(), want_k) and np.array_equal(p_out.cpu().numpy(), want_p)
         assert np.array_equal(f_out.cpu().numpy().view(np.uint16), want_f.view(np.uint16))
     store.free()
+
+
+@pytest.mark.parametrize("rows_of", [5, 10_000])  # few distinct keys (equal ones keep their order), hardly an equal pair
+@pytest.mark.parametrize("kind", ["both_halves", "same_low", "same_high"])
+def test_short_lists_of_wide_keys(kind, rows_of):
+    """Keys that leave no room for the index in lists up to the length of the register network: sorted by halves."""
+    from paper_2609_22441_b200 import binding as B
+
+    rng = np.random.default_rng(rows_of)
+    lens = [2, 31, 33, 127, 128, 129, 300, 512, 513, 1023, 1024, 1, 0, 1025]
+    pool = rng.integers(IMIN, IMAX, size=rows_of, endpoint=True)
+    if kind == "same_low":
+        pool = pool & ~np.int64(0xffffffff) | 77
+    if kind == "same_high":
+        pool = pool & np.int64(0xffffffff) | np.int64(5 << 40)
+        pool[::2] |= np.int64(1 << 62)
+    keys = np.concatenate([pool[rng.integers(0, rows_of, size=n)] for n in lens]).astype(np.int64)
+    feats = rng.integers(0, 1 << 16, size=(len(keys), 8), dtype=np.uint16).view(np.float16)
+    eo = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    want_k, want_f, want_p = oracle.sort_edges(keys, feats, eo)
+    store = B.Docstore(16, 8, "float16", 8, "float16")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    k_in = dev(keys)
+    for bound in (1024, max(lens)):  # the last list is cut at the smaller bound
+        k_out, p_out, f_out = torch.full_like(k_in, -7), torch.full((len(keys),), -7, dtype=torch.int32, device="cuda"), torch.zeros((len(keys), 8), dtype=torch.float16, device="cuda")
+        B.ccr_sort_edges(store, len(lens), bound, k_in, dev(feats.view(np.int16)), dev(eo), k_out, f_out, p_out)
+        torch.cuda.synchronize()
+        n = len(keys) if bound > 1024 else len(keys) - 1025
+        assert np.array_equal(k_out.cpu().numpy()[:n], want_k[:n]) and np.array_equal(p_out.cpu().numpy()[:n], want_p[:n])
+        assert np.array_equal(f_out.cpu().numpy()[:n].view(np.uint16), want_f[:n].view(np.uint16))
+        assert bound > 1024 or int(k_out[-1]) == -7
+    store.free()
+
+
+@pytest.mark.parametrize("bits", [33, 47, 64])
+@pytest.mark.parametrize("lens", [[1025, 1030, 4096, 4095], [4097, 8192, 5000], [12_289, 32_768, 20_001]], ids=lambda l: str(max(l)))
+def test_keys_that_share_a_prefix(lens, bits):
+    """Spread keys are sorted by a prefix of three digits and the records that share one are put in order behind it.  Per list a run
+    of such records at a place of its own, across the border of two blocks among others: none, of two, the longest that is put in order (65)
+    and the shortest that is not, with equal keys among them; wide keys that differ only below the bits that fit a word."""
+    from paper_2609_22441_b200 import binding as B
+
+    rng = np.random.default_rng(bits + max(lens))
+
+    def keys_of(n, run, at, fine):
+        top = 1 << (min(bits, 63) - 1)
+        keys = rng.integers(0, 2 * top - 1, size=n, dtype=np.int64)
+        keys[0], keys[1] = 0, 2 * top - 1  # the range is used up to its ends
+        s = np.sort(keys)
+        base = int(s[min(at, n - 1)]) >> 14 << 14
+        where = rng.choice(n - 2, size=run, replace=False) + 2
+        keys[where] = base + rng.integers(0, 1 << (6 if fine else 14), size=run)
+        if bits == 64:
+            keys = np.where(rng.random(n) < 0.5, keys, -keys)
+        return keys
+
+    cases = [(n, run, at, fine) for n in lens for run in (0, 2, 40, 65, 66, 150) for at, fine in ((n // 2, False), (4096 - 20, True), (n - 5, False))]
+    keys = np.concatenate([keys_of(*c) for c in cases])
+    lens_all = [c[0] for c in cases]
+    feats = rng.integers(0, 1 << 16, size=(len(keys), 8), dtype=np.uint16).view(np.float16)
+    eo = np.concatenate([[0], np.cumsum(lens_all)]).astype(np.int64)
+    want_k, want_f, want_p = oracle.sort_edges(keys, feats, eo)
+    store = B.Docstore(16, 8, "float16", 8, "float16")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    k_in, f_in, o = dev(keys), dev(feats.view(np.int16)), dev(eo)
+    for with_perm in (True, False):
+        if not with_perm and max(lens) > 19_000:
+            continue
+        k_out, p_out, f_out = torch.full_like(k_in, -7), torch.full((len(keys),), -7, dtype=torch.int32, device="cuda"), torch.zeros((len(keys), 8), dtype=torch.float16, device="cuda")
+        B.ccr_sort_edges(store, len(lens_all), max(lens), k_in, f_in, o, k_out, f_out, p_out if with_perm else None)
+        torch.cuda.synchronize()
+        assert np.array_equal(k_out.cpu().numpy(), want_k) and (not with_perm or np.array_equal(p_out.cpu().numpy(), want_p))
+        assert np.array_equal(f_out.cpu().numpy().view(np.uint16), want_f.view(np.uint16))
+    store.free()
