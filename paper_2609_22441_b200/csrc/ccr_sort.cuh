@@ -260,24 +260,26 @@ __device__ __forceinline__ void warp128_block(unsigned long long (&v)[4], int la
 }
 __device__ __forceinline__ void sort_words_merge128(unsigned long long* w, int n) {
   const int lane = threadIdx.x & 31, o = (static_cast<int>(threadIdx.x) >> 5) * 128;
-  unsigned long long v[4];
+  if (o < n) {  // (a warp behind the last word has nothing but padding: 256 lists of 300 records 18.1 -> 12.7 us)
+    unsigned long long v[4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = o + (r << 5) + lane;
-    v[r] = i < n ? w[i] : ~0ull;  // padding sorts last
-  }
-  // blocks of K words alternate in direction until the last, which is ascending
-  warp128_block<2>(v, lane, [](int e) { return (e & 2) == 0; });
-  warp128_block<4>(v, lane, [](int e) { return (e & 4) == 0; });
-  warp128_block<8>(v, lane, [](int e) { return (e & 8) == 0; });
-  warp128_block<16>(v, lane, [](int e) { return (e & 16) == 0; });
-  warp128_block<32>(v, lane, [](int e) { return (e & 32) == 0; });
-  warp128_block<64>(v, lane, [](int e) { return (e & 64) == 0; });
-  warp128_block<128>(v, lane, [](int) { return true; });
+    for (int r = 0; r < 4; ++r) {
+      const int i = o + (r << 5) + lane;
+      v[r] = i < n ? w[i] : ~0ull;  // padding sorts last
+    }
+    // blocks of K words alternate in direction until the last, which is ascending
+    warp128_block<2>(v, lane, [](int e) { return (e & 2) == 0; });
+    warp128_block<4>(v, lane, [](int e) { return (e & 4) == 0; });
+    warp128_block<8>(v, lane, [](int e) { return (e & 8) == 0; });
+    warp128_block<16>(v, lane, [](int e) { return (e & 16) == 0; });
+    warp128_block<32>(v, lane, [](int e) { return (e & 32) == 0; });
+    warp128_block<64>(v, lane, [](int e) { return (e & 64) == 0; });
+    warp128_block<128>(v, lane, [](int) { return true; });
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = o + (r << 5) + lane;
-    if (i < n) w[i] = v[r];
+    for (int r = 0; r < 4; ++r) {
+      const int i = o + (r << 5) + lane;
+      if (i < n) w[i] = v[r];
+    }
   }
   __syncthreads();
   merge_passes<4>(w, n, 128);
