@@ -36,7 +36,7 @@ extern "C" {
 
 typedef struct ccr_docstore ccr_docstore;   /* opaque; owns its device memory */
 typedef struct ccr_workspace ccr_workspace; /* opaque; device staging for the host-buffer entry */
-typedef struct ccr_idindex ccr_idindex;     /* opaque; sorted document ids + sampled search levels on the device */
+typedef struct ccr_idindex ccr_idindex;     /* opaque; document ids and positions in hashed regions, search levels over these, on the device */
 
 typedef enum {
   CCR_OK = 0,
@@ -325,10 +325,11 @@ ccr_status ccr_sort_edges(const ccr_docstore* store, int32_t n_req, int64_t max_
 /* Document-id resolution on the GPU (Section 6.3.1 "Document ID Resolution", Eq. 6): pos(q) = position of
  * document id q in the index, or -1 when q is not indexed.
  *
- * ccr_idindex_create copies n_ids ascending, unique ids (HOST or DEVICE source per src_on_device) into device
- * memory and builds the sampled search levels above them (every 8th key, repeatedly, until at most 2,048
- * keys remain).  `positions` (optional, int32[n_ids], same source side) gives the store position of each id;
- * NULL means the position of an id is its rank.  Synchronous; allocates 9.2 bytes per id (+4 with positions).
+ * ccr_idindex_create builds the index from n_ids ascending, unique ids (HOST or DEVICE source per src_on_device; the
+ * arrays are not needed afterwards): regions of at most 4,096 consecutive ids, a hash table of 32-byte buckets each, and
+ * sampled search levels over the regions' last ids.  `positions` (optional, int32[n_ids], same source side) gives the store
+ * position of each id; NULL means the position of an id is its rank.  Synchronous; allocates 16 bytes per id, with or without
+ * positions, or 32 where the ids of some region span 2^32 or more (host sources: 96 MB more while it runs).
  * ccr_resolve_ids writes out_pos[i] = position of query_ids[i] or -1 for n_queries DEVICE queries: one kernel
  * on `stream`, no allocation, no sync.  Ids that break the ascending order give unspecified positions but
  * every access stays in bounds.  The output is what ccr_join_batch takes as cand_idx (-1 = unresolved).      */

@@ -441,7 +441,7 @@ def ccr_join_payload_static(store: Docstore, n_req: int, total_cands: int, max_e
 
 
 class IdIndex:
-    """ccr_idindex handle: sorted document ids (+ optional positions) with sampled search levels on the device."""
+    """ccr_idindex handle: document ids and their positions on the device, built from ascending ids (+ optional positions)."""
 
     def __init__(self, sorted_ids, positions=None, device: int = 0):
         self._h = ctypes.c_void_p()

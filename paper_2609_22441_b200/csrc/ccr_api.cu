@@ -39,6 +39,7 @@ constexpr long long kSmallLaunchCands = 131072;  // plain launches up to this si
 constexpr int kAutoSmemBudget = 160 * 1024;  // shared memory the warp-specialised kernel takes by default
 constexpr long long kIdsInL2Bytes = 64LL << 20;  // an author-id array up to this size is taken to stay in the 126 MB L2
 constexpr int kMaxTile = ccr::kMaxTileCands;
+constexpr int64_t kIdStage = 8 << 20;  // most ids of a host-sourced index on their way at a time (12 bytes each)
 constexpr size_t kStageBytes = 16u << 20;  // staging block of second-degree stores (ids uploaded from the host)
 #ifndef CCR_HOST_GROUPS
 #define CCR_HOST_GROUPS 3  // config 1, rows staying on the device: 1 group 0.514 ms, 2 0.431, 3 0.413, 4 0.437, 6 0.456, 8 0.495
@@ -132,9 +133,12 @@ struct ccr_idindex {
   int n_sms;
   int64_t n_ids;
   int n_levels;
-  int64_t* level[ccr::kResolveMaxLevels];  // level[0] = sorted ids (owned copy)
-  long long count[ccr::kResolveMaxLevels];
-  int32_t* positions;                      // owned copy, or null
+  int64_t* level[ccr::kResolveMaxLevels];  // level[0] = last id of every region but the last one
+  int count[ccr::kResolveMaxLevels];
+  unsigned* table;                         // n_regions x n_buckets sectors
+  uint32_t n_buckets, n_regions;
+  bool wide;                               // form of the buckets (ccr_resolve.cuh)
+  int64_t min_id, max_id;
   int* dbg_word;                           // bounds-checked build: set by a kernel whose access left the registered buffers
   int64_t launches;
 };
@@ -732,11 +736,47 @@ ccr_status ccr_idindex_free(ccr_idindex* ix) {
   DeviceScope scope(ix->device);
   ix->magic = 0;
   for (int l = 0; l < ccr::kResolveMaxLevels; ++l) cudaFree(ix->level[l]);
-  cudaFree(ix->positions);
+  cudaFree(ix->table);
   cudaFree(ix->dbg_word);
   delete ix;
   return CCR_OK;
 }
+
+}  // extern "C"
+
+namespace {
+// The ends of an index's regions: their last ids on the device (level 0), the smallest and the largest id, the form of the buckets.
+bool index_ends(ccr_idindex* ix, const int64_t* ids, int per_region, int src_on_device) {
+  const int n_regions = static_cast<int>(ix->n_regions);
+  if (src_on_device) {
+    int* flag = nullptr;
+    int wide = 0;
+    bool ok = cudaMalloc(&flag, 256) == cudaSuccess && cudaMemset(flag, 0, 4) == cudaSuccess;
+    if (ok) ccr::region_ends_kernel<<<static_cast<unsigned>((n_regions + 255) / 256), 256>>>(ids, ix->n_ids, per_region, ix->level[0], n_regions, flag);
+    ix->launches++;
+    ok = ok && cudaGetLastError() == cudaSuccess && cudaMemcpy(&wide, flag, 4, cudaMemcpyDeviceToHost) == cudaSuccess;
+    ok = ok && cudaMemcpy(&ix->min_id, ids, 8, cudaMemcpyDeviceToHost) == cudaSuccess;
+    ok = ok && cudaMemcpy(&ix->max_id, ids + ix->n_ids - 1, 8, cudaMemcpyDeviceToHost) == cudaSuccess;
+    cudaFree(flag);
+    ix->wide = wide != 0;
+    return ok;
+  }
+  int64_t* last = new (std::nothrow) int64_t[n_regions];
+  if (last == nullptr) return false;
+  for (int64_t r = 0; r < n_regions; ++r) {
+    last[r] = ids[std::min<int64_t>(ix->n_ids, (r + 1) * per_region) - 1];
+    const int64_t begin = r > 0 ? last[r - 1] : ids[0];
+    if (((static_cast<uint64_t>(last[r]) - static_cast<uint64_t>(begin)) >> 32) != 0) ix->wide = true;
+  }
+  ix->min_id = ids[0];
+  ix->max_id = last[n_regions - 1];
+  const bool ok = n_regions == 1 || cudaMemcpy(ix->level[0], last, static_cast<size_t>(n_regions - 1) * 8, cudaMemcpyHostToDevice) == cudaSuccess;
+  delete[] last;
+  return ok;
+}
+}  // namespace
+
+extern "C" {
 
 ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sorted_ids, const int32_t* positions,
                               int src_on_device, ccr_idindex** out) {
@@ -751,45 +791,33 @@ ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sort
   }
   DeviceScope scope(device);
   if (!scope.ok) return CCR_ERR_CUDA;
-  // level sizes: sample every 8th key until the top level is small enough to stage per block
-  long long count[ccr::kResolveMaxLevels];
+  const int64_t n_regions = std::max<int64_t>(1, (n_ids + ccr::kIdRegion - 1) / ccr::kIdRegion);
+  const int per_region = static_cast<int>(std::max<int64_t>(1, (n_ids + n_regions - 1) / n_regions));
+  // levels over the regions' last ids: every 8th key until the top level is small enough to stage per block
+  int count[ccr::kResolveMaxLevels];
   int n_levels = 1;
-  count[0] = n_ids;
+  count[0] = static_cast<int>(n_regions - 1);
   while (count[n_levels - 1] > ccr::kResolveTopMax) {
     if (n_levels == ccr::kResolveMaxLevels) return CCR_ERR_UNSUPPORTED;
     count[n_levels] = count[n_levels - 1] >> ccr::kResolveFanLog2;
     ++n_levels;
   }
-  if (n_levels == 1) {  // a tiny index still gets a (possibly empty) top level of its own
-    count[1] = count[0] >> ccr::kResolveFanLog2;
-    n_levels = 2;
-  }
-  size_t need = 4096 + (positions ? static_cast<size_t>(n_ids) * 4 : 0);
-  for (int l = 0; l < n_levels; ++l) need += static_cast<size_t>(count[l]) * 8 + 256;
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return CCR_ERR_CUDA;
-  if (need > free_b) return CCR_ERR_OOM;
   ccr_idindex* ix = new (std::nothrow) ccr_idindex();
   if (ix == nullptr) return CCR_ERR_OOM;
   std::memset(ix, 0, sizeof(*ix));
   ix->device = device;
   ix->n_ids = n_ids;
   ix->n_levels = n_levels;
+  ix->n_regions = static_cast<uint32_t>(n_regions);
+  ix->min_id = 1;  // an empty index: no id is in range
   bool ok = cudaDeviceGetAttribute(&ix->n_sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
   for (int l = 0; l < n_levels && ok; ++l) {
     ix->count[l] = count[l];
     ok = cudaMalloc(&ix->level[l], static_cast<size_t>(count[l]) * 8 + 256) == cudaSuccess;
   }
-  const cudaMemcpyKind kind = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  if (ok && n_ids > 0) ok = cudaMemcpy(ix->level[0], sorted_ids, static_cast<size_t>(n_ids) * 8, kind) == cudaSuccess;
-  if (ok && positions && n_ids > 0) {
-    ok = cudaMalloc(&ix->positions, static_cast<size_t>(n_ids) * 4) == cudaSuccess;
-    ok = ok && cudaMemcpy(ix->positions, positions, static_cast<size_t>(n_ids) * 4, kind) == cudaSuccess;
-  }
+  if (ok && n_ids > 0) ok = index_ends(ix, sorted_ids, per_region, src_on_device);
   for (int l = 1; l < n_levels && ok; ++l) {
-    if (count[l] == 0) continue;
-    const unsigned blocks = static_cast<unsigned>((count[l] + 255) / 256 < 8192 ? (count[l] + 255) / 256 : 8192);
-    ccr::build_level_kernel<<<blocks, 256>>>(ix->level[l - 1], count[l - 1], ix->level[l], count[l]);
+    ccr::build_level_kernel<<<static_cast<unsigned>((count[l] + 255) / 256), 256>>>(ix->level[l - 1], ix->level[l], count[l]);
     ix->launches++;
     ok = cudaGetLastError() == cudaSuccess;
   }
@@ -798,20 +826,47 @@ ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sort
     ix->launches++;
     ok = cudaGetLastError() == cudaSuccess;
   }
+  // host ids pass through a block on the device, whole regions at a time
+  const int64_t chunk_regions = src_on_device ? n_regions : std::min<int64_t>(n_regions, kIdStage / per_region);
+  const size_t stage_ids = static_cast<size_t>(chunk_regions) * per_region;
+  ix->n_buckets = ix->wide ? ccr::IdBucket<true>::buckets(per_region) : ccr::IdBucket<false>::buckets(per_region);
+  const size_t table_bytes = static_cast<size_t>(n_regions) * ix->n_buckets * 32;
+  size_t free_b = 0, total_b = 0;
+  ok = ok && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess;
+  const bool room = table_bytes + (src_on_device ? 0 : stage_ids * 12) + 4096 <= free_b;
+  int64_t* stage = nullptr;
+  ok = ok && room && cudaMalloc(&ix->table, table_bytes) == cudaSuccess;
+  if (!src_on_device) ok = ok && cudaMalloc(&stage, stage_ids * 12) == cudaSuccess;
+  const auto build = ix->wide ? ccr::build_regions_kernel<true> : ccr::build_regions_kernel<false>;
+  const size_t build_smem = static_cast<size_t>(ix->n_buckets) * 36;
+  ok = ok && cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(build_smem)) == cudaSuccess;
+  for (int64_t r = 0; n_ids > 0 && r < n_regions && ok; r += chunk_regions) {
+    const int64_t o = r * per_region, m = std::min<int64_t>(static_cast<int64_t>(stage_ids), n_ids - o);
+    const int64_t* ids = sorted_ids + o;
+    const int32_t* pos = positions ? positions + o : nullptr;
+    if (!src_on_device) {
+      int32_t* stage_pos = reinterpret_cast<int32_t*>(stage + stage_ids);
+      ok = cudaMemcpy(stage, ids, static_cast<size_t>(m) * 8, cudaMemcpyHostToDevice) == cudaSuccess;
+      if (pos) ok = ok && cudaMemcpy(stage_pos, pos, static_cast<size_t>(m) * 4, cudaMemcpyHostToDevice) == cudaSuccess;
+      ids = stage;
+      if (pos) pos = stage_pos;
+    }
+    const unsigned blocks = static_cast<unsigned>((m + per_region - 1) / per_region);
+    if (ok) build<<<blocks, ccr::kIdBuildThreads, build_smem>>>(ids, pos, n_ids, per_region, r, ix->table, ix->n_buckets);
+    ix->launches++;
+    ok = ok && cudaGetLastError() == cudaSuccess;
+  }
 #ifdef CCR_DEBUG_BOUNDS
   ok = ok && cudaMalloc(&ix->dbg_word, 256) == cudaSuccess && cudaMemset(ix->dbg_word, 0, 256) == cudaSuccess;
 #endif
   ok = ok && cudaDeviceSynchronize() == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(ccr::resolve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  ccr::kResolveTopMax * 8 + 256) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(ccr::resolve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  ((ccr::kResolveTopMax + 1) << ccr::kResolveFanLog2) * 8 + 256) == cudaSuccess;
+  cudaFree(stage);
   ix->magic = kIxMagic;
   handle_add(ix);
   if (!ok) {
     cudaGetLastError();
     ccr_idindex_free(ix);
-    return CCR_ERR_CUDA;
+    return room ? CCR_ERR_CUDA : CCR_ERR_OOM;
   }
   *out = ix;
   return CCR_OK;
@@ -833,7 +888,10 @@ ccr_status ccr_resolve_ids(const ccr_idindex* cix, int64_t n_queries, const int6
     a.count[l] = ix->count[l];
   }
   a.n_levels = ix->n_levels;
-  a.positions = ix->positions;
+  a.table = ix->table;
+  a.n_buckets = ix->n_buckets;
+  a.min_id = ix->min_id;
+  a.max_id = ix->max_id;
   a.n_queries = n_queries;
   a.queries = query_ids;
   a.out_pos = out_pos;
@@ -845,23 +903,18 @@ ccr_status ccr_resolve_ids(const ccr_idindex* cix, int64_t n_queries, const int6
     }
     DbgRegistrar reg;
     for (int l = 0; l < ix->n_levels; ++l) reg.add(ix->level[l], static_cast<size_t>(ix->count[l] + ccr::kResolvePad) * 8);
-    reg.add(ix->positions, static_cast<size_t>(ix->n_ids) * 4);
+    reg.add(ix->table, static_cast<size_t>(ix->n_regions) * ix->n_buckets * 32);
     reg.add(query_ids, static_cast<size_t>(n_queries) * 8);
     reg.add(out_pos, static_cast<size_t>(n_queries) * 4);
     if (!reg.commit(ix->dbg_word)) return CCR_ERR_CUDA;
   }
 #endif
-  const long long per_block = static_cast<long long>(ccr::kResolveThreads);
-  const long long lanes = 1LL << (ccr::kResolveFanLog2 - 1);  // lanes that share a query
-  long long blocks = (n_queries * lanes + per_block - 1) / per_block;
-  const long long cap = static_cast<long long>(ix->n_sms) * ccr::kResolveBlocksPerSm;  // the top level is re-read by every block
-  if (blocks > cap) blocks = cap;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const bool wide = n_queries >= (ix->n_ids * 8 <= kIdsInL2Bytes ? ccr::kResolveWarpMinInL2 : ccr::kResolveWarpMin);
-  if (wide && a.n_levels > 2) --a.n_levels;  // the level below the top is staged (the leaf level never is)
-  const size_t smem = static_cast<size_t>(a.count[a.n_levels - 1]) * 8 + 16;
-  if (wide) ccr::resolve_kernel<true><<<static_cast<unsigned>(ix->n_sms), ccr::kResolveWideThreads, smem, st>>>(a);
-  else ccr::resolve_kernel<false><<<static_cast<unsigned>(blocks), ccr::kResolveThreads, smem, st>>>(a);
+  const auto kernel = a.n_levels > 1 ? (ix->wide ? ccr::resolve_kernel<true, true> : ccr::resolve_kernel<true, false>)
+                                     : (ix->wide ? ccr::resolve_kernel<false, true> : ccr::resolve_kernel<false, false>);
+  const long long blocks = std::min<long long>((n_queries + ccr::kResolveThreads - 1) / ccr::kResolveThreads,
+                                               static_cast<long long>(ix->n_sms) * ccr::kResolveBlocksPerSm);  // the top level is re-read by every block
+  launch_chained(kernel, dim3(static_cast<unsigned>(blocks)), dim3(ccr::kResolveThreads), static_cast<size_t>(a.count[a.n_levels - 1]) * 8 + 16,
+                 static_cast<cudaStream_t>(stream), a);
   ix->launches++;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
 #ifdef CCR_DEBUG_BOUNDS
