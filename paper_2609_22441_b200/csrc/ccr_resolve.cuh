@@ -94,18 +94,29 @@ __global__ void __launch_bounds__(kIdBuildThreads) build_regions_kernel(const in
     Bucket::put(tab + b * 8 + s * Bucket::kStep, id, positions != nullptr ? positions[at0 + i] : static_cast<int>(rank0 + i));
   }
   __syncthreads();
-  for (unsigned b = threadIdx.x; b < n_buckets; b += kIdBuildThreads) {
-    unsigned* e = tab + b * 8;
-    int s = static_cast<int>(min(came[b], static_cast<unsigned>(Bucket::kSlots)));
-    if (s == 0) Bucket::put(e, ids[at0], positions != nullptr ? positions[at0] : static_cast<int>(rank0));
-    if (WIDE) e[3] = e[7] = 0u;
-    for (s = max(s, 1); s < Bucket::kSlots; ++s)
-      for (int k = 0; k < (WIDE ? 3 : 2); ++k) e[s * Bucket::kStep + k] = e[k];
-  }
-  __syncthreads();
+  // out they go, half a bucket a thread, the slots without an id filled on the way
   const uint4* from = reinterpret_cast<const uint4*>(tab);
   uint4* to = reinterpret_cast<uint4*>(table + static_cast<size_t>(region) * n_buckets * 8);
-  for (unsigned c = threadIdx.x; c < n_buckets * 2; c += kIdBuildThreads) to[c] = from[c];
+  const int64_t id0 = ids[at0];
+  const int pos0 = positions != nullptr ? positions[at0] : static_cast<int>(rank0);
+  for (unsigned c = threadIdx.x; c < n_buckets * 2; c += kIdBuildThreads) {
+    const unsigned b = c >> 1, got = came[b], s = (c & 1u) * (Bucket::kSlots / 2);  // s: first slot of this half
+    uint4 x = from[c];
+    if (WIDE) {
+      if (got <= s) x = got > 0 ? from[c - 1] : make_uint4(static_cast<unsigned>(id0), static_cast<unsigned>(static_cast<unsigned long long>(id0) >> 32), static_cast<unsigned>(pos0), 0u);
+      x.w = 0u;
+    } else if (got <= s + 1) {
+      uint2 f = make_uint2(static_cast<unsigned>(id0), static_cast<unsigned>(pos0));
+      if (got > 0) f = *reinterpret_cast<const uint2*>(tab + b * 8);
+      if (got <= s) {
+        x.x = f.x;
+        x.y = f.y;
+      }
+      x.z = f.x;
+      x.w = f.y;
+    }
+    to[c] = x;
+  }
 }
 
 // Last ids of all regions but the last one, and whether the ids of some region (with the gap in front of it) span 2^32 or more.
