@@ -100,7 +100,8 @@ enum {
                                            stream (see "Back-to-back joins" at ccr_join_batch)                       */
   CCR_FLAG_WARP_SEARCH       = 1u << 12, /* lists that are searched in global memory (CCR_FLAG_FORCE_GLOBAL, key capacity 0)
                                            use the warp-cooperative 32-ary search: one id at a time, 32 pivots per round
-                                           picked by ballot (comparison aid: the lane-per-id binary search is faster)     */
+                                           picked by ballot (comparison aid: the lane-per-id binary search is faster; in
+                                           first-degree joins without the cosine section, others take the binary search)  */
   CCR_FLAG_WARP_SPECIALISED  = 1u << 9  /* take the warp-specialised kernel whatever the launch size (by default a
                                            ragged launch of at most 131,072 candidates — a single request —
                                            runs on the two-phase kernel, which has the shorter start-up)      */

@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
               }
               bool af[4];
               int ap[4];
-              keys.find_batch<4>(act, af, ap);
+              keys.find_batch<4, false, true>(act, af, ap);
 #pragma unroll
               for (int sl = 0; sl < 4; ++sl) {
                 if (af[sl]) {

@@ -80,6 +80,55 @@ __device__ __forceinline__ void key_hash(long long id, unsigned nbk, unsigned& b
   tag = (v << kSlotPosBits) | 0x80000000u;
 }
 
+// The warp-cooperative form of the search in global memory (all 32 lanes must call, converged), one id a lane: index of the id
+// or -1; id < 0 is nothing to look up.  The warp serves one id at a time — 32 pivots spread over the remaining range are read
+// by the 32 lanes, a ballot counts the pivots below the id and picks the sub-range, so a list of 20,000 keys takes 3 rounds
+// (+ 1 read for the equality test) instead of 15 dependent probes, and the last round's 32 keys are one coalesced 256-byte read.
+// Four ids are in flight at once.  The price is that the ids of a batch are served one after the other rather than side by side.
+// Not inlined, one id by value: looping over the arrays of find_batch, it kept them in local memory in every kernel that can
+// reach it, taken or not (second-degree joins 30,000 x 64 311 -> 280 us without, 50,000 x 256 2,644 -> 2,423 us; single requests of
+// 50,000 14.6 -> 13.6 us), and unrolled it is half of a kernel's code.
+__device__ __noinline__ int find_warp(const int64_t* gk, int K, long long id) {
+  const int lane = threadIdx.x & 31;
+  int pos = -1;
+#pragma unroll 1
+  for (int src = 0; src < 32; src += 4) {
+    long long q[4];
+    int lo[4], n[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      q[t] = __shfl_sync(kFull, id, src + t);
+      lo[t] = 0;
+      n[t] = q[t] >= 0 ? K : 0;
+    }
+    while (n[0] > 0 || n[1] > 0 || n[2] > 0 || n[3] > 0) {  // warp-uniform: q, lo and n are the same in every lane
+      long long kv[4];
+      int step[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        step[t] = (n[t] + 31) >> 5;
+        const long long p = static_cast<long long>(lo[t]) + static_cast<long long>(lane + 1) * step[t] - 1;
+        kv[t] = (n[t] > 0 && p < lo[t] + n[t]) ? gload(gk + p) : 0x7fffffffffffffffLL;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (n[t] > 0) {
+          const int c = __popc(__ballot_sync(kFull, kv[t] < q[t]));
+          const int nlo = min(lo[t] + c * step[t], lo[t] + n[t]);
+          n[t] = min(step[t] - 1, lo[t] + n[t] - nlo);
+          lo[t] = nlo;
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const bool f = q[t] >= 0 && lo[t] < K && gload(gk + lo[t]) == q[t];
+      if (lane == src + t && f) pos = lo[t];
+    }
+  }
+  return pos;
+}
+
 // Keys of the request a block is currently serving.
 struct StagedKeys {
   const int64_t* sk;  // shared-memory copy (index i = key i when s_log == 0, sample i otherwise)
@@ -89,7 +138,7 @@ struct StagedKeys {
   int M;              // staged entries (0 = nothing staged)
   int s_log;          // log2 of the sampling stride
   unsigned nbk;       // buckets of the table (0 = none)
-  bool warp_search;   // global-memory searches run warp-cooperatively (find_batch_warp)
+  bool warp_search;   // global-memory searches run warp-cooperatively (find_warp)
   bool declined;      // no table only because the segment it was staged for had too few lookups to pay for one
 
   // Algorithm 1 steps 2-3 for one id by binary search: found = some key equals id; pos = its index (meaningful
@@ -112,78 +161,80 @@ struct StagedKeys {
     return pos < K && gload(gk + pos) == id;
   }
 
-  // U independent lookups with their memory accesses interleaved: one round of table reads (two buckets per id),
-  // then one round of verifying key reads (only ids with a matching fingerprint).  Lists without a table, and the
-  // ids the table cannot answer, take find().  id < 0 is "nothing to look up".
-  // The warp-cooperative form of the search in global memory (all 32 lanes must call, converged): the warp serves
-  // one id at a time — 32 pivots spread over the remaining range are read by the 32 lanes, a ballot counts the
-  // pivots below the id and picks the sub-range, so a list of 20,000 keys takes 3 rounds (+ 1 read for the
-  // equality test) instead of 15 dependent probes, and the last round's 32 keys are one coalesced 256-byte read.
-  // Four ids are in flight at once.  The price is that the 32 x U ids of a batch are served one after the other
-  // rather than side by side.
+  // find() for U ids whose probes go out together: the searches of a list take the same steps whatever the id is.
   template <int U>
-  __device__ __forceinline__ void find_batch_warp(const int64_t (&id)[U], bool (&found)[U], int (&pos)[U]) const {
-    const int lane = threadIdx.x & 31;
+  __device__ __forceinline__ void find_side_by_side(const int64_t (&id)[U], bool (&found)[U], int (&pos)[U]) const {
+    int lo[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
+      lo[u] = 0;
       found[u] = false;
       pos[u] = 0;
     }
     if (K == 0) return;
-#pragma unroll 1
-    for (int u = 0; u < U; ++u) {
-#pragma unroll 1
-      for (int src = 0; src < 32; src += 4) {
-        long long q[4];
-        int lo[4], n[4];
+    for (int n = M; n > 0;) {  // lower bound among the staged keys or samples
+      const int half = (n + 1) >> 1;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          q[t] = __shfl_sync(kFull, id[u], src + t);
-          lo[t] = 0;
-          n[t] = q[t] >= 0 ? K : 0;
-        }
-        while (n[0] > 0 || n[1] > 0 || n[2] > 0 || n[3] > 0) {  // warp-uniform: q, lo and n are the same in every lane
-          long long kv[4];
-          int step[4];
+      for (int u = 0; u < U; ++u) lo[u] = sk[lo[u] + half - 1] < id[u] ? lo[u] + half : lo[u];
+      n -= half;
+    }
+    const bool whole = M > 0 && s_log == 0;
+    if (!whole) {
+      // sample i is key (i+1)*2^s - 1: c samples below id means blocks 0..c-1 are entirely below it
+      int n = K;
+      if (M > 0) {
+        n = 1 << s_log;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            step[t] = (n[t] + 31) >> 5;
-            const long long p = static_cast<long long>(lo[t]) + static_cast<long long>(lane + 1) * step[t] - 1;
-            kv[t] = (n[t] > 0 && p < lo[t] + n[t]) ? gload(gk + p) : 0x7fffffffffffffffLL;
-          }
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            if (n[t] > 0) {
-              const int c = __popc(__ballot_sync(kFull, kv[t] < q[t]));
-              const int nlo = min(lo[t] + c * step[t], lo[t] + n[t]);
-              n[t] = min(step[t] - 1, lo[t] + n[t] - nlo);
-              lo[t] = nlo;
-            }
-          }
-        }
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const bool f = q[t] >= 0 && lo[t] < K && gload(gk + lo[t]) == q[t];
-          if (lane == src + t) {
-            found[u] = f;
-            pos[u] = f ? lo[t] : 0;
-          }
-        }
+        for (int u = 0; u < U; ++u) lo[u] <<= s_log;
       }
+      while (n > 0) {
+        const int half = (n + 1) >> 1;
+        int64_t k[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int p = lo[u] + half - 1;
+          k[u] = id[u] >= 0 && p < K ? gload(gk + p) : 0x7fffffffffffffffLL;  // (the last block may be short)
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) lo[u] = k[u] < id[u] ? lo[u] + half : lo[u];
+        n -= half;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      found[u] = id[u] >= 0 && lo[u] < K && (whole ? sk[lo[u]] : gload(gk + lo[u])) == id[u];
+      if (found[u]) pos[u] = lo[u];
     }
   }
 
-  template <int U>
+  // U independent lookups with their memory accesses interleaved: one round of table reads (two buckets per id),
+  // then one round of verifying key reads (only ids with a matching fingerprint).  Lists without a table, and the
+  // ids the table cannot answer, take find().  id < 0 is "nothing to look up".  WARP: the kernel carries find_warp().
+  // SIDE: without a table, find_side_by_side().  That is for the engager slots of a candidate (single requests of 20,000 candidates
+  // against 20,000 keys 18.8 -> 17.5 us, 1,000 against 15,900 24.6 -> 22.5); the candidates of a thread are mostly just one in a
+  // launch whose lists get no table, and the searches of the others would be made for nothing (10.6 -> 11.3 us).
+  template <int U, bool WARP = false, bool SIDE = false>
   __device__ __forceinline__ void find_batch(const int64_t (&id)[U], bool (&found)[U], int (&pos)[U]) const {
-    if (nbk == 0 && warp_search && M == 0) {
-      find_batch_warp<U>(id, found, pos);
-      return;
+    if constexpr (WARP) {
+      if (nbk == 0 && warp_search && M == 0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int p = find_warp(gk, K, id[u]);
+          found[u] = p >= 0;
+          pos[u] = found[u] ? p : 0;
+        }
+        return;
+      }
     }
     if (nbk == 0) {
+      if constexpr (SIDE) {
+        find_side_by_side<U>(id, found, pos);
+      } else {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        pos[u] = 0;
-        found[u] = id[u] >= 0 && find(id[u], pos[u]);
+        for (int u = 0; u < U; ++u) {
+          pos[u] = 0;
+          found[u] = id[u] >= 0 && find(id[u], pos[u]);
+        }
       }
       return;
     }

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   extern __shared__ __align__(16) unsigned char smem_ws[];
   unsigned char* smem = smem_ws;
   constexpr bool COS = CNP != 0;
+  constexpr bool kWarpSearch = !SECOND && !COS;  // CCR_FLAG_WARP_SEARCH: in these only, the call costs the others registers
   constexpr int kSlots = REBAL ? kRebalSlots : kWsSlots;
   static_assert(!(REBAL && COS), "the rebalanced form carries no cosine section");
   const int n_req_cached = a.n_req <= kWsMaxCachedReq ? a.n_req : 0;
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
             int pq[FB];
 #pragma unroll
             for (int q = 0; q < FB; ++q) idq[q] = auth[h + q];
-            keys.find_batch<FB>(idq, fq, pq);
+            keys.find_batch<FB, kWarpSearch>(idq, fq, pq);
 #pragma unroll
             for (int q = 0; q < FB; ++q) {
               found[h + q] = fq[q];
@@ -405,7 +406,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
               }
               bool fq[FBW];
               int pq[FBW];
-              keys.find_batch<FBW>(idq, fq, pq);
+              keys.find_batch<FBW, false, true>(idq, fq, pq);
 #pragma unroll
               for (int q = 0; q < FBW; ++q) {
                 const int wi = w0 + q * 32 + lane;
