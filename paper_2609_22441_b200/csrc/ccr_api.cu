@@ -260,7 +260,19 @@ struct Variant {
   int doc_ch, edge_ch, req_ch;
   KernelFn first, second, merge;
   WsKernelFn ws_first, ws_second, ws_first_cos, ws_second_cos, ws_second_rebal;
+  WsKernelFn ws_second_staged;  // document rows pass through shared memory, match indices of 16 bits (null: run-time widths)
 };
+
+template <int D, int E, int R>
+constexpr WsKernelFn rebal_kernel() {
+  if constexpr (kRebalBuilt && E < 8) return ccr::join_ws_kernel<D, E, R, true, 0, true>;
+  else return nullptr;
+}
+template <int D, int E, int R>
+constexpr WsKernelFn staged_kernel() {
+  if constexpr (D > 0) return ccr::join_ws_kernel<D, E, R, true, 0, true, true, true>;
+  else return nullptr;
+}
 
 #define CCR_VARIANT(D, E, R)                                                                                      \
   Variant {                                                                                                       \
@@ -269,7 +281,7 @@ struct Variant {
         ccr::join_ws_kernel<D, E, R, false>, ccr::join_ws_kernel<D, E, R, true>,                                  \
         ccr::join_ws_kernel<D, E, R, false, (D > 0 ? kTunedCosPieces : -1)>,                                      \
         ccr::join_ws_kernel<D, E, R, true, (D > 0 ? kTunedCosPieces : -1)>,                                       \
-        ccr::join_ws_kernel<D, E, R, true, 0, kRebalBuilt>                                                        \
+        rebal_kernel<D, E, R>(), staged_kernel<D, E, R>()                                                         \
   }
 
 const Variant kVariants[] = {
@@ -309,10 +321,10 @@ ccr_status allow_large_smem() {
       cudaGetLastError();
       return CCR_ERR_CUDA;
     }
-    const WsKernelFn ws[5] = {kVariants[i].ws_first, kVariants[i].ws_second, kVariants[i].ws_first_cos,
-                              kVariants[i].ws_second_cos, kVariants[i].ws_second_rebal};
+    const WsKernelFn ws[6] = {kVariants[i].ws_first, kVariants[i].ws_second, kVariants[i].ws_first_cos,
+                              kVariants[i].ws_second_cos, kVariants[i].ws_second_rebal, kVariants[i].ws_second_staged};
     for (WsKernelFn f : ws) {
-      if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemBytes) != cudaSuccess) {
+      if (f != nullptr && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         return CCR_ERR_CUDA;
       }
@@ -1101,7 +1113,15 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   }
   // second-degree joins on the default warp split take the register-rebalanced form (12 + 8 warps); a configured
   // split, a configured sub-tile and the cosine section keep the 16-warp kernel
-  const bool rebal = kRebalBuilt && use_ws && second && !cos && s->ws_streamers == 0 && s->tile == 0 && !(flags & CCR_FLAG_NO_REBALANCE);
+  const bool cos_tuned = cos && (s->cos_dim + 7) / 8 == kTunedCosPieces;
+  const Variant& v = (cos && !cos_tuned) ? kVariants[kNumVariants - 1] : pick_variant(s->doc_b / 16, s->edge_b / 16, s->req_b / 16);
+  const bool rebalanced = use_ws && second && !cos && s->ws_streamers == 0 && s->tile == 0 && !(flags & CCR_FLAG_NO_REBALANCE);
+  // ... and, over rows of the tuned widths, its form with staged document rows, unless an explicit key capacity may need the shared
+  // memory that these take or a match index may not fit 16 bits.  (128-byte edge rows then take the 16-warp form: 387 us on 30,000 x 64
+  // with 64-byte request rows, 502 us rebalanced, 343 us staged; 64-byte ones 335, 284 and 287 us.)
+  const bool explicit_cap = (flags & CCR_FLAG_FORCE_SMEM) || s->key_cap > 0;
+  const bool staged = rebalanced && v.ws_second_staged != nullptr && !explicit_cap && max_edge_len < ccr::kNoPos16;
+  const bool rebal = staged || (rebalanced && v.ws_second_rebal != nullptr);
   // Default split of the 16-warp kernel: 12 streamers + 4 resolvers; over a store whose author ids do not stay in L2
   // (the id array, or the 64-byte id records of a store with engagers, beyond kIdsInL2Bytes) every candidate's id is a trip to HBM and a fifth resolver pays for the
   // streamer it replaces (50M documents: 1666 -> 1639 us, sorted candidates 1643 -> 1615 us; 10 + 6: 1643 us; on the
@@ -1123,7 +1143,8 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   auto smem_for = [&](int t, int area) -> size_t {
     return use_ws ? static_cast<size_t>(ccr::WsLayout(t, second, area, n_req <= ccr::kWsMaxCachedReq ? n_req : 0, cos_bytes, n_res,
                                                       rebal ? ccr::kRebalSlots : ccr::kWsSlots,
-                                                      rebal ? ccr::kRebalInFlight * 128 : ccr::kWsWorkItems).bytes)
+                                                      rebal ? ccr::kRebalInFlight * 128 : ccr::kWsWorkItems,
+                                                      staged ? n_str * ccr::ws_docs_bytes(s->doc_b) : 0, staged ? 2 : 4).bytes)
                   : static_cast<size_t>(ccr::TileLayout(t, second, merge, area).bytes);
   };
   // bytes that hold a list of K keys in its best form: staged next to its table (the merge path builds no table)
@@ -1153,11 +1174,11 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     key_cap = static_cast<int>(max_edge_len);
     const long long tiles = (total_cands + tile - 1) / tile;
     const bool streaming_bound = tiles >= 2LL * s->n_sms * n_res;
-    if (streaming_bound) budget = kAutoSmemBudget;
+    // (The form with staged document rows loads little through L1 and takes all of the shared memory: 208 KB cost it 2-4 %.)
+    if (streaming_bound && !staged) budget = kAutoSmemBudget;
   }
   // sub-tile size: the configured one, shrunk (in steps of 256) until the kernel's arrays leave room for the keys
   // of the longest list an explicit capacity promises to stage (the automatic capacity adapts to the room instead)
-  const bool explicit_cap = (flags & CCR_FLAG_FORCE_SMEM) || s->key_cap > 0;
   const int must_fit = explicit_cap ? ccr::search_keys_bytes(key_cap) : 0;
   while (tile > 256 && static_cast<long long>(smem_for(tile, must_fit)) > kMaxSmemBytes) tile -= 256;
   const long long fixed = static_cast<long long>(smem_for(tile, 0));
@@ -1258,14 +1279,12 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     if (s->status_host[1] != 0) return CCR_ERR_VALIDATION;
   }
 
-  const bool cos_tuned = cos && (s->cos_dim + 7) / 8 == kTunedCosPieces;
-  const Variant& v = (cos && !cos_tuned) ? kVariants[kNumVariants - 1] : pick_variant(a.doc_ch, a.edge_ch, a.req_ch);
   const long long groups = (total_cands + 31) / 32;
   if (use_ws) {
     // one persistent warp-specialised block per SM (fewer when there are fewer 32-row groups than SMs)
     long long blocks = s->n_sms;
     if (blocks > groups) blocks = groups;
-    const WsKernelFn fn = cos ? (second ? v.ws_second_cos : v.ws_first_cos) : (second ? (rebal ? v.ws_second_rebal : v.ws_second) : v.ws_first);
+    const WsKernelFn fn = cos ? (second ? v.ws_second_cos : v.ws_first_cos) : (second ? (staged ? v.ws_second_staged : (rebal ? v.ws_second_rebal : v.ws_second)) : v.ws_first);
     // dynamic chunk scheduling through a pair of device words; each launch takes the next pair in turn, so
     // up to kSchedRegions launches of one store may be in flight at once (on any streams)
     // Small launches (fewer tiles than two rounds per block) are split evenly instead: drawing whole rounds

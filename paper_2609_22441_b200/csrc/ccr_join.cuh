@@ -276,24 +276,34 @@ __device__ __forceinline__ uint4 cosine_section(const JoinArgs& a, const uint4* 
   return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), 0u, 0u);
 }
 
-template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0, int GU = kGenericUnrollSecond>
+// Match indices in shared memory: 32 bits, or 16 where every list is shorter than kNoPos16; -1 = not found.
+constexpr int kNoPos16 = 0xffff;
+__device__ __forceinline__ int match_index(const int* p, int i) { return p[i]; }
+__device__ __forceinline__ int match_index(const uint16_t* p, int i) { return p[i] == kNoPos16 ? -1 : p[i]; }
+__device__ __forceinline__ int4 match_indices(const int4* p, int i) { return p[i]; }
+__device__ __forceinline__ int4 match_indices(const ushort4* p, int i) {
+  const ushort4 v = p[i];
+  return make_int4(v.x == kNoPos16 ? -1 : v.x, v.y == kNoPos16 ? -1 : v.y, v.z == kNoPos16 ? -1 : v.z, v.w == kNoPos16 ? -1 : v.w);
+}
+
+template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0, int GU = kGenericUnrollSecond, bool DOCS = true, typename Pos = int, typename Pos4 = int4>
 __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC_CH, EDGE_CH, REQ_CH, SECOND, CNP != 0>& sh,
-                                           const int* s_idx, const int* s_pos, const int4* s_apos,
+                                           const int* s_idx, const Pos* s_pos, const Pos4* s_apos,
                                            const uint8_t* edge_base, const uint8_t* req_src, uint8_t* out, int cnt,
                                            int lane, const float4* cosM = nullptr, uint4* stage = nullptr,
-                                           uint8_t* mask_out = nullptr, const unsigned* s_types = nullptr) {
+                                           uint8_t* mask_out = nullptr, const uint8_t* s_types = nullptr) {
   const long long out_b = sh.out_b;
   // mask bytes of the group (callers that resolved the candidates elsewhere and did not write them): lane = row;
   // bit 0 author found, bits 1-4 engager slot found, bits 5-7 engagement types of the found slots
   if (mask_out != nullptr && lane < cnt) {
-    unsigned m = s_pos[lane] >= 0 ? 1u : 0u;
+    unsigned m = match_index(s_pos, lane) >= 0 ? 1u : 0u;
     if constexpr (SECOND) {
-      const int4 ap4 = s_apos[lane];
+      const int4 ap4 = match_indices(s_apos, lane);
       const int ap[4] = {ap4.x, ap4.y, ap4.z, ap4.w};
       const unsigned ty = s_types[lane];
 #pragma unroll
       for (int sl = 0; sl < 4; ++sl)
-        if (ap[sl] >= 0) m |= (1u << (1 + sl)) | (1u << (5 + ((ty >> (8 * sl)) & 0xffu) % 3u));
+        if (ap[sl] >= 0) m |= (1u << (1 + sl)) | (1u << (5 + ((ty >> (2 * sl)) & 3u)));
     }
     gstore(mask_out + lane, m);
   }
@@ -308,28 +318,32 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
   if constexpr (kCos) __syncwarp();  // the previous group's read-back is done before the block is rewritten
   if constexpr (DOC_CH > 0 && EDGE_CH > 0) {
     // every load of the group is issued before its first store
-    uint4 dv[DOC_CH], ev[EDGE_CH];
+    uint4 dv[DOCS ? DOC_CH : 1], ev[EDGE_CH];
+    if constexpr (DOCS) {
 #pragma unroll
-    for (int i = 0; i < DOC_CH; ++i) {
-      const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;
-      const int ridx = row < cnt ? s_idx[row] : -1;
-      dv[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (ridx >= 0) dv[i] = ldg128_once(a.doc_feats + static_cast<long long>(ridx) * (DOC_CH * 16) + piece * 16);
+      for (int i = 0; i < DOC_CH; ++i) {
+        const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;
+        const int ridx = row < cnt ? s_idx[row] : -1;
+        dv[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (ridx >= 0) dv[i] = ldg128_once(a.doc_feats + static_cast<long long>(ridx) * (DOC_CH * 16) + piece * 16);
+      }
     }
 #pragma unroll
     for (int i = 0; i < EDGE_CH; ++i) {
       const int c = i * 32 + lane, row = c / EDGE_CH, piece = c % EDGE_CH;
-      const int rpos = row < cnt ? s_pos[row] : -1;
+      const int rpos = row < cnt ? match_index(s_pos, row) : -1;
       ev[i] = make_uint4(0u, 0u, 0u, 0u);
       if (rpos >= 0) ev[i] = ldg128(edge_base + static_cast<long long>(rpos) * (EDGE_CH * 16) + piece * 16);
     }
+    if constexpr (DOCS) {
 #pragma unroll
-    for (int i = 0; i < DOC_CH; ++i) {
-      const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;
-      if (row < cnt) st128_stream(out + row * out_b + piece * 16, dv[i]);
-      if constexpr (kCos) {
-        const int q = piece - p0;
-        if (q >= 0 && q < np) stage[row * sstride + q] = dv[i];
+      for (int i = 0; i < DOC_CH; ++i) {
+        const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;
+        if (row < cnt) st128_stream(out + row * out_b + piece * 16, dv[i]);
+        if constexpr (kCos) {
+          const int q = piece - p0;
+          if (q >= 0 && q < np) stage[row * sstride + q] = dv[i];
+        }
       }
     }
 #pragma unroll
@@ -358,7 +372,7 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
         if constexpr (kCos) at_stage[u] = -1;
         if ((i0 + u) * 32 + lane < n_chunks) {
           const bool is_doc = piece < sh.doc_ch, is_edge = !is_doc && piece < edge_end;
-          const int src_row = is_doc ? s_idx[row] : (is_edge ? s_pos[row] : 0);
+          const int src_row = is_doc ? s_idx[row] : (is_edge ? match_index(s_pos, row) : 0);
           const uint8_t* base = is_doc ? a.doc_feats : (is_edge ? edge_base : req_src);
           const int width = is_doc ? sh.doc_b : sh.edge_b, first = is_doc ? 0 : (is_edge ? sh.doc_ch : edge_end);
           if (src_row >= 0) v[u] = ldg128(base + static_cast<long long>(src_row) * width + (piece - first) * 16);
@@ -391,7 +405,7 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
   // made every case slower, 309 -> 392 us at the worst): 64 x 50,000 candidates with 128-byte edge rows 698 -> 664 us,
   // single requests of 50,000 20.0 -> 18.5 us, 64-byte edge rows (30,000 x 64) no change at 309 us.
   if constexpr (SECOND) {
-    const int4 ap = lane < cnt ? s_apos[lane] : make_int4(-1, -1, -1, -1);
+    const int4 ap = lane < cnt ? match_indices(s_apos, lane) : make_int4(-1, -1, -1, -1);
     // (rows of one chunk: a pass covers all 32 rows as it is, counting them off would only add to it)
     const unsigned with = __ballot_sync(kFull, sh.edge_ch > 1 ? (ap.x & ap.y & ap.z & ap.w) >= 0 : lane < cnt);  // indices are >= 0, -1 = not found
     uint8_t* out2 = out + sh.doc_b + sh.edge_b;
@@ -406,7 +420,7 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
       const int row = nth_set_bit(with, nth);
       int rp[4] = {-1, -1, -1, -1};
       if (c < n_chunks) {
-        const int4 p = s_apos[row];
+        const int4 p = match_indices(s_apos, row);
         rp[0] = p.x;
         rp[1] = p.y;
         rp[2] = p.z;

@@ -25,7 +25,18 @@
 // one equal contiguous slice.  (Contiguous slices with work stealing between them — fewer key stagings per block —
 // were measured and lost 7-9 % on every configuration: all blocks walking one window of the candidate range
 // together is what the memory system likes.)
+//
+// PIPE (second-degree joins of the tuned widths): a streamer's document rows pass through shared memory.  What kept these
+// joins from the memory's rate was the time a streamer spends on the edge2 section with no document row under way, and the
+// registers of its row loads.  Here a warp has a buffer of 32 rows: one bulk copy per row fetches the next group's while
+// the edge, edge2 and request sections of the group under way are written, so the warp needs no registers for them, both roles fit 96
+// (nothing spills, no setmaxnreg), and match indices of 16 bits make room in the ring.  50,000 x 256 with 128-byte edge
+// rows 2,423 -> 2,289 us, 30,000 x 64 with 128-byte edge rows 333-502 -> 315-343 us, with 64-byte ones 280 +- 4 us either way.  Measured and
+// slower: the same for first-degree joins (206 -> 222, 1,658 -> 1,906 us: their rows already fill the time) and with the cosine section
+// (request flow 321 -> 396 us); 8 + 8, 8 + 12, 10 + 10, 12 + 10 and 12 + 12 warps; four candidates per resolver lane.
 #pragma once
+
+#include <type_traits>
 
 #include "ccr_join.cuh"
 
@@ -91,14 +102,17 @@ __host__ __device__ inline int ws_cos_bytes(int n_streamers, int stage_per_warp)
   return kWsSlots * kCosSlotFloat4 * 16 + n_streamers * stage_per_warp;
 }
 
+// staging of a streamer's document rows (32 of them) and its barrier
+__host__ __device__ inline int ws_docs_bytes(int doc_b) { return doc_b * 32 + 16; }
+
 struct WsLayout {
-  int off_full, off_empty, off_slots, off_grab, off_offs, off_idx, off_pos, off_apos, off_types, off_cos, off_wl, off_keys, bytes;
+  int off_full, off_empty, off_slots, off_grab, off_offs, off_idx, off_pos, off_apos, off_types, off_cos, off_wl, off_docs, off_keys, bytes;
   // n_req_cached: requests whose offsets are mirrored in shared memory (0 = read them from global memory)
   // cos_bytes: shared memory of the derived cosine section (0 = off): a block of member-embedding floats per
   // ring slot, then one embedding staging block per streamer warp
   // n_res: resolver warps (second-degree joins give each a work list of engager lookups)
   __host__ __device__ WsLayout(int tile, bool second, int search_area, int n_req_cached, int cos_bytes, int n_res,
-                               int n_slots = kWsSlots, int wl_items = kWsWorkItems) {
+                               int n_slots = kWsSlots, int wl_items = kWsWorkItems, int docs_bytes = 0, int pos_bytes = 4) {
     off_full = kSmemHeader;                 // after the key-staging mbarrier
     off_empty = off_full + n_slots * 8;
     off_slots = off_empty + n_slots * 8;
@@ -107,18 +121,19 @@ struct WsLayout {
     off_idx = off_offs + (n_req_cached > 0 ? 2 * (n_req_cached + 1) * 8 : 0);
     off_idx = (off_idx + 15) & ~15;
     off_pos = off_idx + n_slots * tile * 4;
-    off_apos = off_pos + n_slots * tile * 4;
-    off_types = off_apos + (second ? n_slots * tile * 16 : 0);
-    off_cos = off_types + (second ? n_slots * tile * 4 : 0);
+    off_apos = off_pos + n_slots * tile * pos_bytes;
+    off_types = off_apos + (second ? n_slots * tile * 4 * pos_bytes : 0);
+    off_cos = off_types + (second ? n_slots * tile : 0);
     off_wl = off_cos + cos_bytes;
-    off_keys = off_wl + (second ? n_res * wl_items * (8 + 2) : 0);
+    off_docs = (off_wl + (second ? n_res * wl_items * (8 + 2) : 0) + 127) & ~127;
+    off_keys = off_docs + docs_bytes;
     off_keys = (off_keys + 15) & ~15;
     bytes = off_keys + search_area;
   }
 };
 
 // CNP: 0 = no derived section; > 0 = the item embedding spans exactly CNP 16-byte pieces (tuned); < 0 = any shape
-template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0, bool REBAL = false>
+template <int DOC_CH, int EDGE_CH, int REQ_CH, bool SECOND, int CNP = 0, bool REBAL = false, bool PIPE = false, bool NARROW = false>
 __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join_ws_kernel(const JoinArgs a, int n_streamers) {
   extern __shared__ __align__(16) unsigned char smem_ws[];
   unsigned char* smem = smem_ws;
@@ -126,15 +141,18 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   constexpr bool kWarpSearch = !SECOND && !COS;  // CCR_FLAG_WARP_SEARCH: in these only, the call costs the others registers
   constexpr int kSlots = REBAL ? kRebalSlots : kWsSlots;
   static_assert(!(REBAL && COS), "the rebalanced form carries no cosine section");
+  static_assert(!PIPE || (REBAL && DOC_CH > 0), "second-degree joins of the tuned widths");
+  using Pos = typename std::conditional<NARROW, uint16_t, int>::type;
+  using Pos4 = typename std::conditional<NARROW, ushort4, int4>::type;
   const int n_req_cached = a.n_req <= kWsMaxCachedReq ? a.n_req : 0;
   const WsLayout lay(a.tile, SECOND, a.search_area, n_req_cached, COS ? ws_cos_bytes(n_streamers, a.cos_stage) : 0,
-                     (static_cast<int>(blockDim.x) >> 5) - n_streamers, kSlots, REBAL ? kRebalInFlight * 128 : kWsWorkItems);
+                     (static_cast<int>(blockDim.x) >> 5) - n_streamers, kSlots, REBAL ? kRebalInFlight * 128 : kWsWorkItems, PIPE ? n_streamers * ws_docs_bytes(DOC_CH * 16) : 0, sizeof(Pos));
   WsSlot* slots = reinterpret_cast<WsSlot*>(smem + lay.off_slots);
   int* grab = reinterpret_cast<int*>(smem + lay.off_grab);
   int* s_idx = reinterpret_cast<int*>(smem + lay.off_idx);
-  int* s_pos = reinterpret_cast<int*>(smem + lay.off_pos);
-  int4* s_apos = reinterpret_cast<int4*>(smem + lay.off_apos);
-  unsigned* s_types = reinterpret_cast<unsigned*>(smem + lay.off_types);
+  Pos* s_pos = reinterpret_cast<Pos*>(smem + lay.off_pos);
+  Pos4* s_apos = reinterpret_cast<Pos4*>(smem + lay.off_apos);
+  uint8_t* s_types = smem + lay.off_types;
   float4* s_cos = reinterpret_cast<float4*>(smem + lay.off_cos);
   const SearchSmem ssm = carve_search(smem + lay.off_keys, a.search_area, true);
   const uint32_t bar = smem_u32(smem);
@@ -164,6 +182,9 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, static_cast<uint32_t>(n_streamers));
     }
+    if constexpr (PIPE) {
+      for (int s = 0; s < n_streamers; ++s) mbar_init(smem_u32(smem + lay.off_docs + n_streamers * (DOC_CH * 16 * 32) + 16 * s), 1);
+    }
     fence_proxy_async_smem();
   }
   __syncthreads();
@@ -182,45 +203,151 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   const int role_rank = (n_threads >> 5) - 1 - warp;  // resolvers are the last n_res warps
   if (role_rank >= n_res) {
     // ============================ streamers ============================
-    if constexpr (REBAL) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRebalStreamerRegs));
+    if constexpr (REBAL && !PIPE) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRebalStreamerRegs));
     // this warp's embedding staging block (derived cosine section), behind the per-slot member blocks
     [[maybe_unused]] uint4* cos_stage = reinterpret_cast<uint4*>(
         smem + lay.off_cos + kWsSlots * kCosSlotFloat4 * 16 + (role_rank - n_res) * (COS ? a.cos_stage : 0));
-    for (unsigned it = 0;; ++it) {
-      const int s = it % kSlots;
-      if (!mbar_wait_bounded(full0 + 8 * s, (it / kSlots) & 1u)) {
-        if (lane == 0) atomicExch(a.status, kDevWaitExpired);
-        break;
+    if constexpr (PIPE) {
+      // this warp's document rows: fetched by bulk copies while the rest of the group before is under way
+      constexpr int kDocB = DOC_CH * 16;
+      unsigned char* docs = smem + lay.off_docs + (role_rank - n_res) * (kDocB * 32);
+      const uint32_t docs_bar = smem_u32(smem + lay.off_docs + n_streamers * (kDocB * 32) + 16 * (role_rank - n_res));
+      uint32_t docs_phase = 0;
+      unsigned it = 0;             // sub-tile the next group comes from
+      bool open = false;           // that sub-tile is known to be there
+      int cur_s = -1, cur_g = 0;   // the group under way: ring slot, first row
+      int nxt_s = -1, nxt_g = 0;
+      unsigned valid = 0;          // rows of the fetched group that have a document
+      bool stop = false, release = false, waited = false;  // release: the slot of the group under way is exhausted
+      // The next group, without waiting for a sub-tile unless `block`.  Slots that run out are handed back; the one the group under
+      // way is in only when that group is done.
+      auto next_group = [&](bool block) -> bool {
+        for (;;) {
+          const int s = it % kSlots;
+          if (!open) {
+            if (!block && !__all_sync(kFull, mbar_try_wait(full0 + 8 * s, (it / kSlots) & 1u))) return false;
+            if (block && !mbar_wait_bounded(full0 + 8 * s, (it / kSlots) & 1u)) {
+              if (lane == 0) atomicExch(a.status, kDevWaitExpired);
+              stop = true;
+              return false;
+            }
+            open = true;
+          }
+          const int n = slots[s].n;
+          if (n == 0) {
+            stop = true;
+            return false;
+          }
+          int g = 0;
+          if (lane == 0) g = atomicAdd(&slots[s].next, 1);
+          g = __shfl_sync(kFull, g, 0) * 32;
+          if (g < n) {
+            nxt_s = s;
+            nxt_g = g;
+            return true;
+          }
+          if (s == cur_s) {
+            release = true;
+          } else {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty0 + 8 * s);
+          }
+          ++it;
+          open = false;
+        }
+      };
+      auto fetch_docs = [&]() {
+        const int p = nxt_g + lane < slots[nxt_s].n ? s_idx[nxt_s * a.tile + nxt_g + lane] : -1;
+        const uint8_t* src = a.doc_feats + static_cast<long long>(p) * kDocB;
+        const bool ok = p >= 0 && CCR_CHK(src, kDocB);
+        valid = __ballot_sync(kFull, ok);
+        if (lane == 0) mbar_arrive_expect_tx(docs_bar, static_cast<uint32_t>(__popc(valid)) * kDocB);
+        __syncwarp();
+        if (ok) bulk_copy_g2s(smem_u32(docs + lane * kDocB), src, kDocB, docs_bar);
+      };
+      bool got = next_group(true);
+      if (got) fetch_docs();
+      while (got) {
+        cur_s = nxt_s;
+        cur_g = nxt_g;
+        const WsSlot& d = slots[cur_s];
+        const int cnt = min(32, d.n - cur_g);
+        uint8_t* out = a.out_rows + (d.out0 + cur_g) * sh.out_b;
+        if (!mbar_wait_bounded(docs_bar, docs_phase)) {
+          if (lane == 0) atomicExch(a.status, kDevWaitExpired);
+          mbar_wait_bounded(docs_bar, docs_phase);
+          break;
+        }
+        docs_phase ^= 1u;
+        if (!waited) {
+          pdl_wait();  // the first rows are about to be written: the launch before this one must be done
+          waited = true;
+        }
+#pragma unroll 4
+        for (int i = 0; i < DOC_CH; ++i) {
+          const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;
+          uint4 v = *reinterpret_cast<const uint4*>(docs + c * 16);
+          if (!((valid >> row) & 1u)) v = make_uint4(0u, 0u, 0u, 0u);
+          if (row < cnt) st128_stream(out + row * sh.out_b + piece * 16, v);
+        }
+        __syncwarp();
+        got = next_group(false);
+        if (got) fetch_docs();
+        const int o = cur_s * a.tile + cur_g;
+        emit_group<DOC_CH, EDGE_CH, REQ_CH, SECOND, CNP, kGenericUnrollSecond, false>(
+            a, sh, s_idx + o, s_pos + o, s_apos + o, a.edge_feats + d.kb * sh.edge_b,
+            sh.req_ch ? a.req_feats + static_cast<long long>(d.r) * sh.req_b : nullptr, out, cnt, lane, nullptr, nullptr,
+            a.out_mask + d.out0 + cur_g, s_types + o);
+        __syncwarp();
+        if (release) {
+          if (lane == 0) mbar_arrive(empty0 + 8 * cur_s);
+          release = false;
+        }
+        cur_s = -1;
+        if (!got && !stop) {
+          got = next_group(true);
+          if (got) fetch_docs();
+        }
       }
-      const WsSlot d = slots[s];
-      if (d.n == 0) break;
-      if (it == 0) pdl_wait();  // the first rows are about to be written: the launch before this one must be done
-      const uint8_t* edge_base = a.edge_feats + d.kb * sh.edge_b;
-      const uint8_t* req_src = sh.req_ch ? a.req_feats + static_cast<long long>(d.r) * sh.req_b : nullptr;
-      const int* idx = s_idx + s * a.tile;
-      const int* pos = s_pos + s * a.tile;
-      const int4* apos = s_apos + s * a.tile;
-      const unsigned* types = s_types + s * a.tile;
-      // groups are handed out one at a time, so a warp that finishes early simply takes more
-      for (;;) {
-        int g = 0;
-        if (lane == 0) g = atomicAdd(&slots[s].next, 1);
-        g = __shfl_sync(kFull, g, 0) * 32;
-        if (g >= d.n) break;
-        emit_group<DOC_CH, EDGE_CH, REQ_CH, SECOND, CNP>(a, sh, idx + g, pos + g, apos + g, edge_base, req_src,
-                                                         a.out_rows + (d.out0 + g) * sh.out_b, min(32, d.n - g), lane,
-                                                         COS ? s_cos + s * kCosSlotFloat4 : nullptr,
-                                                         COS ? cos_stage : nullptr, a.out_mask + d.out0 + g, types + g);
+      pdl_wait();  // (a launch never completes before the one in front of it)
+      return;
+    } else {
+      for (unsigned it = 0;; ++it) {
+        const int s = it % kSlots;
+        if (!mbar_wait_bounded(full0 + 8 * s, (it / kSlots) & 1u)) {
+          if (lane == 0) atomicExch(a.status, kDevWaitExpired);
+          break;
+        }
+        const WsSlot d = slots[s];
+        if (d.n == 0) break;
+        if (it == 0) pdl_wait();  // the first rows are about to be written: the launch before this one must be done
+        const uint8_t* edge_base = a.edge_feats + d.kb * sh.edge_b;
+        const uint8_t* req_src = sh.req_ch ? a.req_feats + static_cast<long long>(d.r) * sh.req_b : nullptr;
+        const int* idx = s_idx + s * a.tile;
+        const Pos* pos = s_pos + s * a.tile;
+        const Pos4* apos = s_apos + s * a.tile;
+        const uint8_t* types = s_types + s * a.tile;
+        // groups are handed out one at a time, so a warp that finishes early simply takes more
+        for (;;) {
+          int g = 0;
+          if (lane == 0) g = atomicAdd(&slots[s].next, 1);
+          g = __shfl_sync(kFull, g, 0) * 32;
+          if (g >= d.n) break;
+          emit_group<DOC_CH, EDGE_CH, REQ_CH, SECOND, CNP>(a, sh, idx + g, pos + g, apos + g, edge_base, req_src,
+                                                           a.out_rows + (d.out0 + g) * sh.out_b, min(32, d.n - g), lane,
+                                                           COS ? s_cos + s * kCosSlotFloat4 : nullptr,
+                                                           COS ? cos_stage : nullptr, a.out_mask + d.out0 + g, types + g);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty0 + 8 * s);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty0 + 8 * s);
+      pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
+      return;
     }
-    pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
-    return;
   }
 
   // ============================ resolvers ============================
-  if constexpr (REBAL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRebalResolverRegs));
+  if constexpr (REBAL && !PIPE) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRebalResolverRegs));
   // All resolver warps walk the same sequence of sub-tiles; warp q fills every n_resolvers-th one on its own
   // (own bounded wait for the slot, own publish), so several sub-tiles are being resolved at any time.  They
   // meet on a named barrier only to draw the next chunk and to stage a new request's keys.
@@ -313,9 +440,9 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
         }
         const long long out0 = a.n_max > 0 ? r * a.n_max + (sub - co[r]) : sub;
         int* out_idx = s_idx + s * a.tile;
-        int* out_pos = s_pos + s * a.tile;
-        int4* out_apos = s_apos + s * a.tile;
-        [[maybe_unused]] unsigned* out_types = s_types + s * a.tile;
+        Pos* out_pos = s_pos + s * a.tile;
+        Pos4* out_apos = s_apos + s * a.tile;
+        [[maybe_unused]] uint8_t* out_types = s_types + s * a.tile;
         for (int base = 0; base < n; base += 32 * U) {
           int idx[U];
           int64_t auth[U];
@@ -368,12 +495,15 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
             // shared memory (lane-major, so workers read consecutive entries) and the lanes share them out,
             // four interleaved lookups at a time; a hit writes its key index straight into the slot's
             // position array, which the owner lane has preset to -1.
-            int* apos_i = reinterpret_cast<int*>(out_apos);
+            Pos* apos_i = reinterpret_cast<Pos*>(out_apos);
             int mine = 0;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
               const int i = base + u * 32 + lane;
-              if (i < n) out_apos[i] = make_int4(-1, -1, -1, -1);
+              if (i < n) {
+                if constexpr (NARROW) out_apos[i] = make_ushort4(kNoPos16, kNoPos16, kNoPos16, kNoPos16);
+                else out_apos[i] = make_int4(-1, -1, -1, -1);
+              }
 #pragma unroll
               for (int sl = 0; sl < 4; ++sl) mine += act[u][sl] >= 0 ? 1 : 0;
             }
@@ -410,7 +540,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
 #pragma unroll
               for (int q = 0; q < FBW; ++q) {
                 const int wi = w0 + q * 32 + lane;
-                if (wi < total && fq[q]) apos_i[wl_tag[wi]] = pq[q];
+                if (wi < total && fq[q]) apos_i[wl_tag[wi]] = static_cast<Pos>(pq[q]);
               }
             }
 #pragma unroll
@@ -418,8 +548,9 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
               const int i = base + u * 32 + lane;
               if (i < n) {
                 out_idx[i] = idx[u];
-                out_pos[i] = found[u] ? pos[u] : -1;
-                out_types[i] = types[u];  // the streamers derive the mask byte from the match indices and these
+                out_pos[i] = static_cast<Pos>(found[u] ? pos[u] : -1);
+                // the streamers derive the mask byte from the match indices and these (the types modulo 3, two bits a slot)
+                out_types[i] = static_cast<uint8_t>((types[u] & 0xffu) % 3u | (((types[u] >> 8) & 0xffu) % 3u) << 2 | (((types[u] >> 16) & 0xffu) % 3u) << 4 | ((types[u] >> 24) % 3u) << 6);
               }
             }
           } else {
@@ -428,7 +559,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
               const int i = base + u * 32 + lane;
               if (i < n) {
                 out_idx[i] = idx[u];
-                out_pos[i] = found[u] ? pos[u] : -1;
+                out_pos[i] = static_cast<Pos>(found[u] ? pos[u] : -1);
               }
             }
           }

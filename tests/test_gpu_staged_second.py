@@ -1,0 +1,69 @@
+"""GPU parity of the second-degree join whose document rows pass through shared memory: rows of the tuned widths, groups and sub-tiles of
+every remainder, groups without any document, the largest bound on the list length that 16-bit match indices hold and the next
+one, ragged and padded output."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2609_22441_b200 import workloads as W
+
+from helpers import gpu_join, tiny_workload
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _workload(seed, edge_dim, req_dim, lengths):
+    wl = tiny_workload(seed, 900, 3_000, len(lengths), 700, 1, True, req_dim, doc_dim=128, doc_dtype=np.float16, edge_dim=edge_dim,
+                       sum_mask=0xA5A5_0FF0_3C3C_FFFF & ((1 << edge_dim) - 1))
+    rng = np.random.default_rng(seed + 1)
+    b = wl.batch
+    b.cand_offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    b.cand_idx = rng.integers(-1, wl.store.n_docs + 1, size=int(b.cand_offsets[-1])).astype(np.int32)
+    b.cand_idx[40:140] = -1  # whole groups without a document
+    return wl
+
+
+@pytest.mark.parametrize("edge_dim,req_dim", [(32, 0), (32, 16), (64, 0), (64, 16)])
+@pytest.mark.parametrize("bound", [0, 65_534, 65_535])
+def test_remainders_bounds_and_empty_groups(edge_dim, req_dim, bound):
+    from paper_2609_22441_b200 import binding as B
+
+    lengths = [1, 0, 31, 32, 33, 127, 128, 129, 5_000, 0, 4_095, 255]
+    wl = _workload(edge_dim + req_dim, edge_dim, req_dim, lengths)
+    want_rows, want_mask = oracle.join_workload(wl)
+    store = B.store_from_workload(wl)
+    db = B.DeviceBatch(wl.batch)
+    db.max_edge_len = max(db.max_edge_len, bound)
+    for flags in (B.CCR_FLAG_WARP_SPECIALISED, B.CCR_FLAG_WARP_SPECIALISED | B.CCR_FLAG_FORCE_GLOBAL):
+        rows, mask = gpu_join(store, db, flags)
+        assert np.array_equal(mask, want_mask) and np.array_equal(rows, want_rows)
+    T, M, offs, src = B.join_batch_padded(store, db, n_max=4_097)
+    torch.cuda.synchronize()
+    s, b = wl.store, wl.batch
+    want = oracle.join_padded(s.doc_feats, s.author_ids, b.edge_keys, b.edge_feats, b.edge_offsets, b.cand_idx, b.cand_offsets, n_max=4_097,
+                              req_feats=b.req_feats, actor_ids=s.actor_ids, actor_types=s.actor_types, reduce_sum_mask=s.reduce_sum_mask)
+    assert np.array_equal(T.cpu().numpy(), want[0]) and np.array_equal(M.cpu().numpy(), want[1])
+    assert store.device_status() == B.CCR_OK
+    store.free()
+
+
+def test_back_to_back_and_on_two_streams():
+    """Launches that overlap on one stream and run at the same time on two."""
+    from paper_2609_22441_b200 import binding as B
+
+    wl = W.config1(n_docs=40_000, n_req=24, n_cand=9_001, second_degree=True)
+    want_rows, want_mask = oracle.join_workload(wl, n_threads=4)
+    store = B.store_from_workload(wl)
+    db = B.DeviceBatch(wl.batch)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [(torch.empty((db.total_cands, store.out_row_bytes()), dtype=torch.uint8, device="cuda"),
+             torch.empty(db.total_cands, dtype=torch.uint8, device="cuda")) for _ in streams]
+    torch.cuda.synchronize()
+    for i in range(12):
+        B.join_batch(store, db, 0, *outs[i % 2], stream=streams[i % 2])
+    torch.cuda.synchronize()
+    for rows, mask in outs:
+        assert np.array_equal(rows.cpu().numpy(), want_rows) and np.array_equal(mask.cpu().numpy(), want_mask)
+    assert store.device_status() == B.CCR_OK
+    store.free()
