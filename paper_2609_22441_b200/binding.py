@@ -179,11 +179,16 @@ def _dtype_code(dt) -> int:
     raise ValueError("feature dtype must be float16 or float32")
 
 
+# A small call is bound by the host: what runs once per argument or per call goes without attribute lookups (one request of 1,000
+# candidates 10.3 -> 7.0 us a call together with the stream below, which took 3 us of it).
+_Tensor = torch.Tensor
+
+
 def _ptr(x) -> Optional[int]:
     """Address of a torch tensor (device or host) or numpy array; None stays NULL."""
     if x is None:
         return None
-    if isinstance(x, torch.Tensor):
+    if isinstance(x, _Tensor):
         if not x.is_contiguous():
             raise ValueError("tensors passed to the library must be contiguous")
         return x.data_ptr()
@@ -195,8 +200,8 @@ def _ptr(x) -> Optional[int]:
 
 
 def _stream_ptr(stream) -> Optional[int]:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+    if stream is None:  # the handle of torch.cuda.current_stream() without the stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return int(stream) or None
