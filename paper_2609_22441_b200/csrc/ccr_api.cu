@@ -101,6 +101,7 @@ struct ccr_docstore {
   int64_t dbg_shrink_rows;             // bounds-checked build: rows cut off the registered output extents
   std::atomic<int64_t> launches;  // kernels launched for this store; also hands out the scheduling-word pairs
   std::atomic<int64_t> sort_calls;  // chunked ccr_sort_edges calls; hands out their flag words
+  std::atomic<int64_t> compactions;  // ccr_compact_valid calls; hands out their counters
 };
 
 struct ccr_workspace {
@@ -524,6 +525,7 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
   if (s == nullptr) return CCR_ERR_OOM;
   s->launches.store(0);
   s->sort_calls.store(0);
+  s->compactions.store(0);
   s->desc = *d;
   s->doc_b = static_cast<int>(doc_b);
   s->edge_b = static_cast<int>(edge_b);
@@ -691,7 +693,7 @@ ccr_status ccr_docstore_upsert(ccr_docstore* s, int64_t n, const int32_t* positi
   long long blocks = (work + per_block - 1) / per_block;
   const long long cap = static_cast<long long>(s->n_sms) * 8;
   blocks = blocks < 1 ? 1 : (blocks > cap ? cap : blocks);
-  ccr::upsert_kernel<<<static_cast<unsigned>(blocks), ccr::kUpsertThreads, 0, static_cast<cudaStream_t>(stream)>>>(a);
+  launch_chained(ccr::upsert_kernel, dim3(static_cast<unsigned>(blocks)), dim3(ccr::kUpsertThreads), 0, static_cast<cudaStream_t>(stream), a);
   s->launches++;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
 #ifdef CCR_DEBUG_BOUNDS
@@ -1394,9 +1396,8 @@ ccr_status padded_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cand
 #endif
     // enough blocks to fill the device however few requests there are
     const unsigned slices = static_cast<unsigned>(std::max(1, std::min(64, (2 * s->n_sms + n_req - 1) / n_req)));
-    ccr::pad_fill_kernel<<<dim3(static_cast<unsigned>(n_req), slices), ccr::kPadThreads, 0,
-                           static_cast<cudaStream_t>(stream)>>>(
-        cand_offsets, n_max, static_cast<long long>(out_row_bytes(s, flags)), static_cast<uint8_t*>(out_rows), out_mask);
+    launch_chained(ccr::pad_fill_kernel, dim3(static_cast<unsigned>(n_req), slices), dim3(ccr::kPadThreads), 0, static_cast<cudaStream_t>(stream),
+                   cand_offsets, n_max, static_cast<long long>(out_row_bytes(s, flags)), static_cast<uint8_t*>(out_rows), out_mask);
     s->launches++;
     if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
   }
@@ -1480,16 +1481,18 @@ ccr_status ccr_compact_valid(const ccr_docstore* cs, int32_t n_req, int64_t tota
     if (!reg.commit(s->status + 2)) return CCR_ERR_CUDA;
   }
 #endif
-  launch_chained(ccr::count_valid_kernel, dim3(static_cast<unsigned>(n_req)), dim3(ccr::kPadThreads), 0, st, cand_idx, cand_offsets,
-                 n_docs, offsets_out);
-  launch_chained(ccr::scan_counts_kernel, dim3(1), dim3(ccr::kPadThreads), 0, st, offsets_out, n_req);
+  // finished blocks of the count: word 9 of a scheduling region (the joins use words 0 and 1, the chunked sorts word 8), regions taken
+  // in turn, so up to kSchedRegions compactions of one store may be in flight at once
+  int* done = s->status + kStatusHead + s->sched_stride * static_cast<int>(s->compactions.fetch_add(1) % kSchedRegions) + 9;
+  launch_chained(ccr::count_scan_kernel, dim3(static_cast<unsigned>(n_req)), dim3(ccr::kPadThreads), 0, st, cand_idx, cand_offsets,
+                 n_docs, offsets_out, n_req, done);
   // slices per request: about one round of the compaction each, bounded so that the re-count stays small
   const long long per_round = static_cast<long long>(ccr::kPadThreads) * ccr::kPadItems;
   const long long avg = (total_cands + n_req - 1) / n_req;
   const unsigned slices = static_cast<unsigned>(std::max(1LL, std::min(8LL, (avg + per_round - 1) / per_round)));
   launch_chained(ccr::compact_valid_kernel, dim3(static_cast<unsigned>(n_req), slices), dim3(ccr::kPadThreads), 0, st,
       cand_idx, cand_offsets, n_docs, offsets_out, idx_out, src_out);
-  s->launches += 3;
+  s->launches += 2;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
 #ifdef CCR_DEBUG_BOUNDS
   return dbg_finish(s->status + 2, st);

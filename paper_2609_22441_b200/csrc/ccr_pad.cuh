@@ -62,37 +62,39 @@ __device__ __forceinline__ int block_count_valid(const int32_t* cand_idx, long l
   return total;
 }
 
-// Step 1a: valid candidates per request -> counts[r + 1] (counts[0] = 0).  One block per request.
+// Step 1a + b: valid candidates per request, one block each, and by the block that finishes last their inclusive scan in place:
+// offsets[r + 1] = valid candidates of requests 0 .. r.  `done` counts finished blocks and is zero between calls.  (The scan as a launch
+// of its own cost a chain of small launches about 3 us.)
 __global__ void __launch_bounds__(kPadThreads)
-count_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, int64_t* counts) {
-  chain_enter(true);
-  __shared__ int warp_sums[kPadThreads / 32];
-  const int r = blockIdx.x;
-  const int total = block_count_valid(cand_idx, gload(cand_offsets + r), gload(cand_offsets + r + 1), n_docs, warp_sums);
-  if (threadIdx.x == 0) {
-    gstore(counts + r + 1, total);
-    if (r == 0) gstore(counts, 0);
-  }
-}
-
-// Step 1b: in-place inclusive scan of counts[1 .. n_req] (one block; n_req is a batch size, a few hundred).
-__global__ void __launch_bounds__(kPadThreads) scan_counts_kernel(int64_t* counts, int n_req) {
+count_scan_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, int64_t* offsets, int n_req, int* done) {
   chain_enter(true);
   __shared__ int warp_sums[kPadThreads / 32];
   __shared__ long long carry_s;
-  if (threadIdx.x == 0) carry_s = 0;
+  __shared__ int last_s;
+  const int r = blockIdx.x;
+  const int mine = block_count_valid(cand_idx, gload(cand_offsets + r), gload(cand_offsets + r + 1), n_docs, warp_sums);
+  if (threadIdx.x == 0) {
+    gstore(offsets + r + 1, mine);
+    if (r == 0) gstore(offsets, 0);
+    __threadfence();
+    last_s = atomicAdd(done, 1) == n_req - 1;
+    carry_s = 0;
+  }
   __syncthreads();
+  if (!last_s) return;
+  __threadfence();
   for (int base = 0; base < n_req; base += kPadThreads) {
-    const int r = base + threadIdx.x;
-    const int v = r < n_req ? static_cast<int>(gload_rw(counts + r + 1)) : 0;
+    const int q = base + threadIdx.x;
+    const int v = q < n_req ? static_cast<int>(gload_once_written(offsets + q + 1)) : 0;
     int total;
     const int inc = block_scan_inclusive(v, warp_sums, total);
     const long long carry = carry_s;
-    if (r < n_req) gstore(counts + r + 1, carry + inc);
+    if (q < n_req) gstore(offsets + q + 1, carry + inc);
     __syncthreads();
     if (threadIdx.x == 0) carry_s = carry + total;
     __syncthreads();
   }
+  if (threadIdx.x == 0) *done = 0;
 }
 
 // Step 1c + 2: the request's valid positions, in their input order, at [offsets_out[r], offsets_out[r + 1]);
@@ -154,6 +156,10 @@ compact_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long 
 // request r's pad range; 16-byte streaming stores (out_b is a multiple of 16).
 __global__ void __launch_bounds__(kPadThreads)
 pad_fill_kernel(const int64_t* cand_offsets, long long n_max, long long out_b, uint8_t* out_rows, uint8_t* out_mask) {
+  // The join behind it may start at once: it writes other rows, and what it reads was written before this kernel, which has waited
+  // for that (request flow 317.5 -> 313.9 us, with the scan that count_scan_kernel saves).
+  pdl_wait();
+  pdl_trigger();
   const int r = blockIdx.x;
   long long n_r = gload(cand_offsets + r + 1) - gload(cand_offsets + r);
   n_r = n_r < 0 ? 0 : (n_r > n_max ? n_max : n_r);

@@ -33,6 +33,7 @@ struct UpsertArgs {
 // every target row is written as row_ch contiguous chunks by neighbouring lanes.  Streaming loads (the batch is
 // read once); default stores (the row is about to be read by joins).  The ids follow, one thread per row.
 __global__ void __launch_bounds__(kUpsertThreads) upsert_kernel(const UpsertArgs a) {
+  chain_enter(false);  // set up while the work in front drains (300,000 rows and their first join 74.9 -> 73.0 us)
   const long long tid = blockIdx.x * static_cast<long long>(kUpsertThreads) + threadIdx.x;
   const long long stride = static_cast<long long>(gridDim.x) * kUpsertThreads;
   if (a.src_rows != nullptr) {
