@@ -309,8 +309,6 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
           if (got) fetch_docs();
         }
       }
-      pdl_wait();  // (a launch never completes before the one in front of it)
-      return;
     } else {
       for (unsigned it = 0;; ++it) {
         const int s = it % kSlots;
@@ -341,9 +339,9 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + 8 * s);
       }
-      pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
-      return;
     }
+    pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
+    return;
   }
 
   // ============================ resolvers ============================
