@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
             const int64_t id4[4] = {auth[h], auth[h + 1], auth[h + 2], auth[h + 3]};
             bool f4[4];
             int p4[4];
-            keys.find_batch<4>(id4, f4, p4);
+            keys.find_batch<4, false, SECOND>(id4, f4, p4);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               found[h + q] = f4[q];

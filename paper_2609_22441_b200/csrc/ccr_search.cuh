@@ -210,9 +210,9 @@ struct StagedKeys {
   // U independent lookups with their memory accesses interleaved: one round of table reads (two buckets per id),
   // then one round of verifying key reads (only ids with a matching fingerprint).  Lists without a table, and the
   // ids the table cannot answer, take find().  id < 0 is "nothing to look up".  WARP: the kernel carries find_warp().
-  // SIDE: without a table, find_side_by_side().  That is for the engager slots of a candidate (single requests of 20,000 candidates
-  // against 20,000 keys 18.8 -> 17.5 us, 1,000 against 15,900 24.6 -> 22.5); the candidates of a thread are mostly just one in a
-  // launch whose lists get no table, and the searches of the others would be made for nothing (10.6 -> 11.3 us).
+  // SIDE: without a table, find_side_by_side().  That is for second-degree joins (single requests of 20,000 candidates against
+  // 20,000 keys 18.8 -> 16.2 us, 1,153 against 15,900 24.6 -> 22.5; engager slots alone 20.6); in first-degree ones the candidates of
+  // a thread are mostly just one where a list gets no table, and the searches of the others are made for nothing (10.6 -> 11.3 us).
   template <int U, bool WARP = false, bool SIDE = false>
   __device__ __forceinline__ void find_batch(const int64_t (&id)[U], bool (&found)[U], int (&pos)[U]) const {
     if constexpr (WARP) {
