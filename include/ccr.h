@@ -219,8 +219,8 @@ ccr_status ccr_join_batch(const ccr_docstore* store,
  * scores can be carried back to the caller's candidate order (CCR_ERR_UNSUPPORTED when total_cands exceeds
  * 2^31 - 1, the range of those indices).  idx_out needs room for cand_offsets[n_req]
  * entries (all candidates may be valid); idx_out / offsets_out must not alias the inputs.  All pointers are
- * DEVICE pointers; two small kernels on `stream`, nothing allocated, no synchronisation; at most 64 calls may be in flight on
- * one store at once (each takes a counter word of the store's in turn).  total_cands only
+ * DEVICE pointers; two small kernels on `stream`, nothing allocated, no synchronisation, no state kept in the store: any
+ * number of calls may be in flight, captured and replayed ones among them.  total_cands only
  * chooses how many blocks share a request (from the mean request length); the count pass uses one block per
  * request, so the cost grows with the longest request rather than with the batch.
  *

@@ -101,7 +101,6 @@ struct ccr_docstore {
   int64_t dbg_shrink_rows;             // bounds-checked build: rows cut off the registered output extents
   std::atomic<int64_t> launches;  // kernels launched for this store; also hands out the scheduling-word pairs
   std::atomic<int64_t> sort_calls;  // chunked ccr_sort_edges calls; hands out their flag words
-  std::atomic<int64_t> compactions;  // ccr_compact_valid calls; hands out their counters
 };
 
 struct ccr_workspace {
@@ -525,7 +524,6 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
   if (s == nullptr) return CCR_ERR_OOM;
   s->launches.store(0);
   s->sort_calls.store(0);
-  s->compactions.store(0);
   s->desc = *d;
   s->doc_b = static_cast<int>(doc_b);
   s->edge_b = static_cast<int>(edge_b);
@@ -1481,11 +1479,8 @@ ccr_status ccr_compact_valid(const ccr_docstore* cs, int32_t n_req, int64_t tota
     if (!reg.commit(s->status + 2)) return CCR_ERR_CUDA;
   }
 #endif
-  // finished blocks of the count: word 9 of a scheduling region (the joins use words 0 and 1, the chunked sorts word 8), regions taken
-  // in turn, so up to kSchedRegions compactions of one store may be in flight at once
-  int* done = s->status + kStatusHead + s->sched_stride * static_cast<int>(s->compactions.fetch_add(1) % kSchedRegions) + 9;
-  launch_chained(ccr::count_scan_kernel, dim3(static_cast<unsigned>(n_req)), dim3(ccr::kPadThreads), 0, st, cand_idx, cand_offsets,
-                 n_docs, offsets_out, n_req, done);
+  launch_chained(ccr::count_valid_kernel, dim3(static_cast<unsigned>(n_req)), dim3(ccr::kPadThreads), 0, st, cand_idx, cand_offsets,
+                 n_docs, offsets_out);
   // slices per request: about one round of the compaction each, bounded so that the re-count stays small
   const long long per_round = static_cast<long long>(ccr::kPadThreads) * ccr::kPadItems;
   const long long avg = (total_cands + n_req - 1) / n_req;

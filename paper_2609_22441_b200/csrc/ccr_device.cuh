@@ -199,8 +199,8 @@ __device__ __forceinline__ T gload_rw(const T* p) {
   if (!CCR_CHK(p, static_cast<int>(sizeof(T)))) return T{};
   return *p;
 }
-// load past L1 of what other blocks of the same launch have written (behind a fence)
-__device__ __forceinline__ int64_t gload_once_written(const int64_t* p) {
+// load past L1 of what other blocks of the same launch may be writing
+__device__ __forceinline__ int64_t gload_shared_out(const int64_t* p) {
   if (!CCR_CHK(p, 8)) return 0;
   return __ldcg(reinterpret_cast<const long long*>(p));
 }

@@ -62,42 +62,50 @@ __device__ __forceinline__ int block_count_valid(const int32_t* cand_idx, long l
   return total;
 }
 
-// Step 1a + b: valid candidates per request, one block each, and by the block that finishes last their inclusive scan in place:
-// offsets[r + 1] = valid candidates of requests 0 .. r.  `done` counts finished blocks and is zero between calls.  (The scan as a launch
-// of its own cost a chain of small launches about 3 us.)
+// Step 1a: valid candidates per request, one block each: offsets[r + 1] = ~(valid candidates of request r), which is negative, so that
+// an entry tells a count from a final offset; offsets[0] = 0.
 __global__ void __launch_bounds__(kPadThreads)
-count_scan_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, int64_t* offsets, int n_req, int* done) {
+count_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, int64_t* offsets) {
   chain_enter(true);
   __shared__ int warp_sums[kPadThreads / 32];
-  __shared__ long long carry_s;
-  __shared__ int last_s;
   const int r = blockIdx.x;
   const int mine = block_count_valid(cand_idx, gload(cand_offsets + r), gload(cand_offsets + r + 1), n_docs, warp_sums);
   if (threadIdx.x == 0) {
-    gstore(offsets + r + 1, mine);
+    gstore(offsets + r + 1, ~static_cast<int64_t>(mine));
     if (r == 0) gstore(offsets, 0);
-    __threadfence();
-    last_s = atomicAdd(done, 1) == n_req - 1;
-    carry_s = 0;
   }
-  __syncthreads();
-  if (!last_s) return;
-  __threadfence();
-  for (int base = 0; base < n_req; base += kPadThreads) {
-    const int q = base + threadIdx.x;
-    const int v = q < n_req ? static_cast<int>(gload_once_written(offsets + q + 1)) : 0;
-    int total;
-    const int inc = block_scan_inclusive(v, warp_sums, total);
-    const long long carry = carry_s;
-    if (q < n_req) gstore(offsets + q + 1, carry + inc);
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s = carry + total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *done = 0;
 }
 
-// Step 1c + 2: the request's valid positions, in their input order, at [offsets_out[r], offsets_out[r + 1]);
+// Step 1b: valid candidates in front of request r, by the whole block, from entries 0 .. r of which each may still be a count or
+// already be a final offset (the blocks of the compaction turn theirs over while others read): the counts behind the last final offset
+// are added to it.  Any mixture gives the same sum, so nobody waits for anybody and no counter outlives the call: calls may run side
+// by side and be captured and replayed in any number.  Entries are read from r downwards, kPadThreads at a time; of many requests the
+// blocks in front have mostly finished, and the first round finds one of their offsets.
+__device__ __forceinline__ long long block_offset_of(const int64_t* offsets, int r, long long* warp_part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  long long before = 0;
+  for (long long at = r;; at -= kPadThreads) {
+    const long long q = at - threadIdx.x;
+    const long long v = q >= 0 ? gload_shared_out(offsets + q) : 0;
+    const unsigned final_lanes = __ballot_sync(kFull, v >= 0);  // (entry 0 is final, so lanes in front of it never count)
+    const int last = final_lanes != 0 ? __ffs(final_lanes) - 1 : 32;
+    long long part = lane < last ? ~v : (lane == last ? v : 0);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(kFull, part, d);
+    if (lane == 0) warp_part[warp] = final_lanes != 0 ? ~part : part;  // negative: ends with a final offset
+    __syncthreads();
+    bool done = false;
+    for (int w = 0; w < kPadThreads / 32 && !done; ++w) {
+      const long long p = warp_part[w];
+      done = p < 0;
+      before += done ? ~p : p;
+    }
+    __syncthreads();  // warp_part may be reused at once
+    if (done) return before;
+  }
+}
+
+// Step 1c + 2: the request's valid positions, in their input order, at [offsets[r], offsets[r + 1]), and the final offsets[r + 1];
 // src_out[k] (optional) is the flat input index of kept candidate k, so scores can be carried back.
 // Blocks (r, 0 .. gridDim.y) each take one slice of request r; a block first counts the valid candidates in
 // the slices before its own (a re-read of at most the request's positions, which sit in L2), then walks its
@@ -105,17 +113,21 @@ count_scan_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long lon
 // groups of 32 candidates from w * 32 * kPadItems: a ballot per group ranks its valid lanes, so loads and
 // stores are both contiguous per warp instruction and the order is kept without a second pass.
 __global__ void __launch_bounds__(kPadThreads)
-compact_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, const int64_t* offsets_out,
-                     int32_t* idx_out, int32_t* src_out) {
+compact_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long long n_docs, int64_t* offsets, int32_t* idx_out,
+                     int32_t* src_out) {
   chain_enter(false);
   __shared__ int warp_sums[kPadThreads / 32];
+  __shared__ long long warp_part[kPadThreads / 32];
   const int r = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long j0 = gload(cand_offsets + r), j1 = gload(cand_offsets + r + 1);
   const long long slice = (((j1 - j0) + gridDim.y - 1) / gridDim.y + 31) / 32 * 32;
   const long long s0 = min(j1, j0 + blockIdx.y * slice), s1 = min(j1, s0 + slice);
-  if (s0 >= s1) return;
-  long long out = gload(offsets_out + r) + block_count_valid(cand_idx, j0, s0, n_docs, warp_sums);
+  if (s0 >= s1 && blockIdx.y > 0) return;
+  long long out = block_offset_of(offsets, r, warp_part);
+  if (blockIdx.y == 0 && threadIdx.x == 0)  // nobody else writes entry r + 1, and it still holds the count
+    gstore(offsets + r + 1, out + ~gload_shared_out(offsets + r + 1));
+  out += block_count_valid(cand_idx, j0, s0, n_docs, warp_sums);
   for (long long base = s0; base < s1; base += kPadThreads * kPadItems) {
     const long long jw = base + static_cast<long long>(warp) * (32 * kPadItems) + lane;
     int p[kPadItems];
