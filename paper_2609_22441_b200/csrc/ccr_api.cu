@@ -850,8 +850,11 @@ ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sort
   ok = ok && room && cudaMalloc(&ix->table, table_bytes) == cudaSuccess;
   if (!src_on_device) ok = ok && cudaMalloc(&stage, stage_ids * 12) == cudaSuccess;
   const auto build = ix->wide ? ccr::build_regions_kernel<true> : ccr::build_regions_kernel<false>;
-  const size_t build_smem = static_cast<size_t>(ix->n_buckets) * 36;
-  ok = ok && cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(build_smem)) == cudaSuccess;
+  const size_t build_smem = static_cast<size_t>(ix->n_buckets) * ccr::kIdBucketSmem;
+  // (the limit of the largest region, whatever this index needs: the attribute is the process's, and another thread may be setting it
+  // for an index of its own between this and the launch)
+  const unsigned most = ix->wide ? ccr::IdBucket<true>::buckets(ccr::kIdRegion) : ccr::IdBucket<false>::buckets(ccr::kIdRegion);
+  ok = ok && cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most * ccr::kIdBucketSmem)) == cudaSuccess;
   for (int64_t r = 0; n_ids > 0 && r < n_regions && ok; r += chunk_regions) {
     const int64_t o = r * per_region, m = std::min<int64_t>(static_cast<int64_t>(stage_ids), n_ids - o);
     const int64_t* ids = sorted_ids + o;

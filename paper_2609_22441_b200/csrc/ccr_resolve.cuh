@@ -27,6 +27,7 @@ constexpr int kResolveThreads = 256;
 constexpr int kResolveBlocksPerSm = 8;
 constexpr int kResolveUnroll = 4;                  // queries a group of lanes descends with at a time
 constexpr int kIdBuildThreads = 512;
+constexpr unsigned kIdBucketSmem = 36;             // shared memory of a bucket while its region is built: the sector and a counter
 constexpr long long kResolveInf = 0x7fffffffffffffffLL;  // stands for the keys beyond the end of a level
 
 // A bucket is a 32-byte sector.  Narrow: four entries {low 32 bits of the id, position}, used when the ids of every region span
