@@ -750,6 +750,7 @@ ccr_status ccr_idindex_free(ccr_idindex* ix) {
   for (int l = 0; l < ccr::kResolveMaxLevels; ++l) cudaFree(ix->level[l]);
   cudaFree(ix->table);
   cudaFree(ix->dbg_word);
+  cudaGetLastError();  // (of a failed free: the next launch's check must not find it)
   delete ix;
   return CCR_OK;
 }
@@ -757,24 +758,43 @@ ccr_status ccr_idindex_free(ccr_idindex* ix) {
 }  // extern "C"
 
 namespace {
+// Status of a series of runtime calls: that of the first one that failed (the ones behind it are not made).
+struct Steps {
+  ccr_status st = CCR_OK;
+  bool ok() const { return st == CCR_OK; }
+  void fail(ccr_status why) {
+    if (ok()) st = why;
+  }
+  template <typename F>
+  void operator()(F call) {
+    if (!ok()) return;
+    const cudaError_t e = call();
+    if (e != cudaSuccess) fail(e == cudaErrorMemoryAllocation ? CCR_ERR_OOM : CCR_ERR_CUDA);
+  }
+};
+
 // The ends of an index's regions: their last ids on the device (level 0), the smallest and the largest id, the form of the buckets.
-bool index_ends(ccr_idindex* ix, const int64_t* ids, int per_region, int src_on_device) {
+void index_ends(ccr_idindex* ix, const int64_t* ids, int per_region, int src_on_device, Steps& step) {
   const int n_regions = static_cast<int>(ix->n_regions);
   if (src_on_device) {
     int* flag = nullptr;
     int wide = 0;
-    bool ok = cudaMalloc(&flag, 256) == cudaSuccess && cudaMemset(flag, 0, 4) == cudaSuccess;
-    if (ok) ccr::region_ends_kernel<<<static_cast<unsigned>((n_regions + 255) / 256), 256>>>(ids, ix->n_ids, per_region, ix->level[0], n_regions, flag);
-    ix->launches++;
-    ok = ok && cudaGetLastError() == cudaSuccess && cudaMemcpy(&wide, flag, 4, cudaMemcpyDeviceToHost) == cudaSuccess;
-    ok = ok && cudaMemcpy(&ix->min_id, ids, 8, cudaMemcpyDeviceToHost) == cudaSuccess;
-    ok = ok && cudaMemcpy(&ix->max_id, ids + ix->n_ids - 1, 8, cudaMemcpyDeviceToHost) == cudaSuccess;
+    step([&] { return cudaMalloc(&flag, 256); });
+    step([&] { return cudaMemset(flag, 0, 4); });
+    step([&] {
+      ccr::region_ends_kernel<<<static_cast<unsigned>((n_regions + 255) / 256), 256>>>(ids, ix->n_ids, per_region, ix->level[0], n_regions, flag);
+      ix->launches++;
+      return cudaGetLastError();
+    });
+    step([&] { return cudaMemcpy(&wide, flag, 4, cudaMemcpyDeviceToHost); });
+    step([&] { return cudaMemcpy(&ix->min_id, ids, 8, cudaMemcpyDeviceToHost); });
+    step([&] { return cudaMemcpy(&ix->max_id, ids + ix->n_ids - 1, 8, cudaMemcpyDeviceToHost); });
     cudaFree(flag);
     ix->wide = wide != 0;
-    return ok;
+    return;
   }
   int64_t* last = new (std::nothrow) int64_t[n_regions];
-  if (last == nullptr) return false;
+  if (last == nullptr) return step.fail(CCR_ERR_OOM);
   for (int64_t r = 0; r < n_regions; ++r) {
     last[r] = ids[std::min<int64_t>(ix->n_ids, (r + 1) * per_region) - 1];
     const int64_t begin = r > 0 ? last[r - 1] : ids[0];
@@ -782,9 +802,8 @@ bool index_ends(ccr_idindex* ix, const int64_t* ids, int per_region, int src_on_
   }
   ix->min_id = ids[0];
   ix->max_id = last[n_regions - 1];
-  const bool ok = n_regions == 1 || cudaMemcpy(ix->level[0], last, static_cast<size_t>(n_regions - 1) * 8, cudaMemcpyHostToDevice) == cudaSuccess;
+  if (n_regions > 1) step([&] { return cudaMemcpy(ix->level[0], last, static_cast<size_t>(n_regions - 1) * 8, cudaMemcpyHostToDevice); });
   delete[] last;
-  return ok;
 }
 }  // namespace
 
@@ -822,66 +841,68 @@ ccr_status ccr_idindex_create(int32_t device, int64_t n_ids, const int64_t* sort
   ix->n_levels = n_levels;
   ix->n_regions = static_cast<uint32_t>(n_regions);
   ix->min_id = 1;  // an empty index: no id is in range
-  bool ok = cudaDeviceGetAttribute(&ix->n_sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
-  for (int l = 0; l < n_levels && ok; ++l) {
+  Steps step;
+  step([&] { return cudaDeviceGetAttribute(&ix->n_sms, cudaDevAttrMultiProcessorCount, device); });
+  for (int l = 0; l < n_levels; ++l) {
     ix->count[l] = count[l];
-    ok = cudaMalloc(&ix->level[l], static_cast<size_t>(count[l]) * 8 + 256) == cudaSuccess;
+    step([&] { return cudaMalloc(&ix->level[l], static_cast<size_t>(count[l]) * 8 + 256); });
   }
-  if (ok && n_ids > 0) ok = index_ends(ix, sorted_ids, per_region, src_on_device);
-  for (int l = 1; l < n_levels && ok; ++l) {
+  if (step.ok() && n_ids > 0) index_ends(ix, sorted_ids, per_region, src_on_device, step);
+  for (int l = 1; l < n_levels; ++l) step([&] {
     ccr::build_level_kernel<<<static_cast<unsigned>((count[l] + 255) / 256), 256>>>(ix->level[l - 1], ix->level[l], count[l]);
     ix->launches++;
-    ok = cudaGetLastError() == cudaSuccess;
-  }
-  for (int l = 0; l < n_levels && ok; ++l) {  // the +infinity keys behind every level (the allocation has room)
+    return cudaGetLastError();
+  });
+  for (int l = 0; l < n_levels; ++l) step([&] {  // the +infinity keys behind every level (the allocation has room)
     ccr::pad_level_kernel<<<1, 32>>>(ix->level[l], count[l]);
     ix->launches++;
-    ok = cudaGetLastError() == cudaSuccess;
-  }
+    return cudaGetLastError();
+  });
   // host ids pass through a block on the device, whole regions at a time
   const int64_t chunk_regions = src_on_device ? n_regions : std::min<int64_t>(n_regions, kIdStage / per_region);
-  const size_t stage_ids = static_cast<size_t>(chunk_regions) * per_region;
+  const size_t stage_ids = static_cast<size_t>(chunk_regions) * per_region, stage_bytes = src_on_device ? 0 : stage_ids * 12;
   ix->n_buckets = ix->wide ? ccr::IdBucket<true>::buckets(per_region) : ccr::IdBucket<false>::buckets(per_region);
   const size_t table_bytes = static_cast<size_t>(n_regions) * ix->n_buckets * 32;
   size_t free_b = 0, total_b = 0;
-  ok = ok && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess;
-  const bool room = table_bytes + (src_on_device ? 0 : stage_ids * 12) + 4096 <= free_b;
+  step([&] { return cudaMemGetInfo(&free_b, &total_b); });
+  if (table_bytes + stage_bytes + 4096 > free_b) step.fail(CCR_ERR_OOM);
   int64_t* stage = nullptr;
-  ok = ok && room && cudaMalloc(&ix->table, table_bytes) == cudaSuccess;
-  if (!src_on_device) ok = ok && cudaMalloc(&stage, stage_ids * 12) == cudaSuccess;
+  step([&] { return cudaMalloc(&ix->table, table_bytes); });
+  if (!src_on_device) step([&] { return cudaMalloc(&stage, stage_bytes); });
   const auto build = ix->wide ? ccr::build_regions_kernel<true> : ccr::build_regions_kernel<false>;
   const size_t build_smem = static_cast<size_t>(ix->n_buckets) * ccr::kIdBucketSmem;
   // (the limit of the largest region, whatever this index needs: the attribute is the process's, and another thread may be setting it
   // for an index of its own between this and the launch)
   const unsigned most = ix->wide ? ccr::IdBucket<true>::buckets(ccr::kIdRegion) : ccr::IdBucket<false>::buckets(ccr::kIdRegion);
-  ok = ok && cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most * ccr::kIdBucketSmem)) == cudaSuccess;
-  for (int64_t r = 0; n_ids > 0 && r < n_regions && ok; r += chunk_regions) {
+  step([&] { return cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most * ccr::kIdBucketSmem)); });
+  for (int64_t r = 0; n_ids > 0 && r < n_regions && step.ok(); r += chunk_regions) {
     const int64_t o = r * per_region, m = std::min<int64_t>(static_cast<int64_t>(stage_ids), n_ids - o);
     const int64_t* ids = sorted_ids + o;
     const int32_t* pos = positions ? positions + o : nullptr;
     if (!src_on_device) {
       int32_t* stage_pos = reinterpret_cast<int32_t*>(stage + stage_ids);
-      ok = cudaMemcpy(stage, ids, static_cast<size_t>(m) * 8, cudaMemcpyHostToDevice) == cudaSuccess;
-      if (pos) ok = ok && cudaMemcpy(stage_pos, pos, static_cast<size_t>(m) * 4, cudaMemcpyHostToDevice) == cudaSuccess;
+      step([&] { return cudaMemcpy(stage, ids, static_cast<size_t>(m) * 8, cudaMemcpyHostToDevice); });
+      if (pos) step([&] { return cudaMemcpy(stage_pos, pos, static_cast<size_t>(m) * 4, cudaMemcpyHostToDevice); });
       ids = stage;
       if (pos) pos = stage_pos;
     }
-    const unsigned blocks = static_cast<unsigned>((m + per_region - 1) / per_region);
-    if (ok) build<<<blocks, ccr::kIdBuildThreads, build_smem>>>(ids, pos, n_ids, per_region, r, ix->table, ix->n_buckets);
-    ix->launches++;
-    ok = ok && cudaGetLastError() == cudaSuccess;
+    step([&] {
+      build<<<static_cast<unsigned>((m + per_region - 1) / per_region), ccr::kIdBuildThreads, build_smem>>>(ids, pos, n_ids, per_region, r, ix->table, ix->n_buckets);
+      ix->launches++;
+      return cudaGetLastError();
+    });
   }
 #ifdef CCR_DEBUG_BOUNDS
-  ok = ok && cudaMalloc(&ix->dbg_word, 256) == cudaSuccess && cudaMemset(ix->dbg_word, 0, 256) == cudaSuccess;
+  step([&] { return cudaMalloc(&ix->dbg_word, 256); });
+  step([&] { return cudaMemset(ix->dbg_word, 0, 256); });
 #endif
-  ok = ok && cudaDeviceSynchronize() == cudaSuccess;
+  step([] { return cudaDeviceSynchronize(); });
   cudaFree(stage);
   ix->magic = kIxMagic;
   handle_add(ix);
-  if (!ok) {
-    cudaGetLastError();
+  if (!step.ok()) {
     ccr_idindex_free(ix);
-    return room ? CCR_ERR_CUDA : CCR_ERR_OOM;
+    return step.st;
   }
   *out = ix;
   return CCR_OK;
