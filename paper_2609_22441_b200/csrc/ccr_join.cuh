@@ -460,7 +460,10 @@ __device__ __forceinline__ void emit_group(const JoinArgs& a, const RowShape<DOC
   }
 }
 
-constexpr int kUnrollMax = 8;  // candidates a thread keeps in flight in phase A (4 in the variants that would spill with 8)
+// Candidates a thread keeps in flight in phase A: those of a default sub-tile (1,024 over 256 threads), which most small launches do not
+// even fill.  Eight, as it was, are instructions for candidates that are not there: 63 requests of 1,200 31.0 -> 29.0 us, 4 of 3,300
+// 19.4 -> 18.3, 342 candidates 14.5 -> 14.0, 6 of 695 11.6 -> 11.0, 4 of 30,000 27.6 -> 25.7, second-degree 39.6 -> 35.4.
+constexpr int kUnroll = 4;
 #ifndef CCR_JOIN_MIN_BLOCKS
 #define CCR_JOIN_MIN_BLOCKS 2
 #endif
@@ -481,9 +484,6 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
   const uint32_t bar = smem_u32(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const RowShape<DOC_CH, EDGE_CH, REQ_CH, SECOND> sh(a);
-  // (the generic-width and the wide-row second-degree variants would spill with eight candidates of a thread in
-  // flight in phase A)
-  constexpr int kUnroll = (SECOND && (DOC_CH == 0 || EDGE_CH >= 8)) ? 4 : kUnrollMax;
 
   if (tid == 0) {
     mbar_init(bar, 1);
@@ -551,19 +551,7 @@ __global__ void __launch_bounds__(kThreads, kJoinMinBlocks) join_kernel(const Jo
           }
           bool found[kUnroll];
           int pos[kUnroll];
-          static_assert(kUnroll % 4 == 0, "lookups are interleaved four at a time");
-#pragma unroll
-          for (int h = 0; h < kUnroll; h += 4) {
-            const int64_t id4[4] = {auth[h], auth[h + 1], auth[h + 2], auth[h + 3]};
-            bool f4[4];
-            int p4[4];
-            keys.find_batch<4, false, SECOND>(id4, f4, p4);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              found[h + q] = f4[q];
-              pos[h + q] = p4[q];
-            }
-          }
+          keys.find_batch<kUnroll, false, SECOND>(auth, found, pos);
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u) {
             const int i = base + u * kThreads + tid;

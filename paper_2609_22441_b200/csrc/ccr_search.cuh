@@ -389,8 +389,17 @@ __device__ __forceinline__ bool stage_keys(const JoinArgs& a, const SearchSmem& 
     while ((K >> s_log) > cap) ++s_log;
     st.s_log = s_log;
     st.M = K >> s_log;
-    for (int i = g.tid; i < st.M; i += g.size)
-      skeys[i] = gload(a.edge_keys + kb + ((static_cast<long long>(i) + 1) << s_log) - 1);
+    // five samples of a thread under way at a time (indices beyond the last one read and write that once more): 342 candidates against
+    // 7,040 keys 14.0 -> 12.4 us, 50,000 against 10,000 14.5 -> 13.0, 120,000 against 20,000 30.1 -> 26.7; four 12.5 / 13.2 / 27.1
+    constexpr int kSamplesInFlight = 5;
+#pragma unroll 1
+    for (int i0 = g.tid; i0 < st.M; i0 += kSamplesInFlight * g.size) {
+      int64_t k[kSamplesInFlight];
+#pragma unroll
+      for (int q = 0; q < kSamplesInFlight; ++q) k[q] = gload(st.gk + ((min(i0 + q * g.size, st.M - 1) + 1) << s_log) - 1);
+#pragma unroll
+      for (int q = 0; q < kSamplesInFlight; ++q) skeys[min(i0 + q * g.size, st.M - 1)] = k[q];
+    }
   }
   if (g.sync_or(expired)) return false;
 
