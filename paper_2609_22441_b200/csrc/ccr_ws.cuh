@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
       int cur_s = -1, cur_g = 0;   // the group under way: ring slot, first row
       int nxt_s = -1, nxt_g = 0;
       unsigned valid = 0;          // rows of the fetched group that have a document
-      bool stop = false, release = false, waited = false;  // release: the slot of the group under way is exhausted
+      bool stop = false, release = false;  // release: the slot of the group under way is exhausted
       // The next group, without waiting for a sub-tile unless `block`.  Slots that run out are handed back; the one the group under
       // way is in only when that group is done.
       auto next_group = [&](bool block) -> bool {
@@ -266,7 +266,10 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
         if (ok) bulk_copy_g2s(smem_u32(docs + lane * kDocB), src, kDocB, docs_bar);
       };
       bool got = next_group(true);
-      if (got) fetch_docs();
+      if (got) {
+        pdl_wait();  // rows of the store are inputs that may just have been written: the launch before this one must be done
+        fetch_docs();
+      }
       while (got) {
         cur_s = nxt_s;
         cur_g = nxt_g;
@@ -279,10 +282,6 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
           break;
         }
         docs_phase ^= 1u;
-        if (!waited) {
-          pdl_wait();  // the first rows are about to be written: the launch before this one must be done
-          waited = true;
-        }
 #pragma unroll 4
         for (int i = 0; i < DOC_CH; ++i) {
           const int c = i * 32 + lane, row = c / DOC_CH, piece = c % DOC_CH;

@@ -67,3 +67,43 @@ def test_back_to_back_and_on_two_streams():
         assert np.array_equal(rows.cpu().numpy(), want_rows) and np.array_equal(mask.cpu().numpy(), want_mask)
     assert store.device_status() == B.CCR_OK
     store.free()
+
+
+@pytest.mark.parametrize("edge_dim", [32, 64])
+def test_rows_and_ids_written_by_the_upsert_in_front(edge_dim):
+    """Two batches of documents replace the same rows in turn, each followed by a join without a synchronisation in between."""
+    from paper_2609_22441_b200 import binding as B
+
+    n, lengths = 50_000, [9_000] * 20
+    wl = _workload(edge_dim, edge_dim, 16, lengths)
+    rng = np.random.default_rng(edge_dim)
+    s, b = wl.store, wl.batch
+    reps = n // s.n_docs + 1
+    s.doc_feats, s.author_ids, s.actor_ids, s.actor_types = (np.ascontiguousarray(np.concatenate([a] * reps)[:n])
+                                                             for a in (s.doc_feats, s.author_ids, s.actor_ids, s.actor_types))
+    s.n_docs = n
+    b.cand_idx = rng.integers(0, n, size=b.total_cands).astype(np.int32)
+    store, db = B.store_from_workload(wl), B.DeviceBatch(b)
+    pos = rng.permutation(n).astype(np.int32)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    batches, wants, outs = [], [], []
+    for _ in range(2):
+        order = rng.permutation(n)
+        new = (rng.standard_normal(s.doc_feats.shape).astype(np.float16), s.author_ids[order], s.actor_ids[order], s.actor_types[order])
+        state = oracle.upsert(s.doc_feats.copy(), s.author_ids.copy(), pos.astype(np.int64), new[0], new[1], s.actor_ids.copy(), s.actor_types.copy(),
+                              new[2], new[3])
+        wants.append(oracle.join(state[0], state[1], b.edge_keys, b.edge_feats, b.edge_offsets, b.cand_idx, b.cand_offsets, req_feats=b.req_feats,
+                                 actor_ids=state[2], actor_types=state[3], reduce_sum_mask=s.reduce_sum_mask, n_threads=4))
+        batches.append([dev(a) for a in new])
+        outs.append((torch.zeros((b.total_cands, store.out_row_bytes()), dtype=torch.uint8, device="cuda"),
+                     torch.zeros(b.total_cands, dtype=torch.uint8, device="cuda")))
+    pos = dev(pos)
+    torch.cuda.synchronize()
+    for i in range(20):
+        store.upsert(pos, *batches[i % 2])
+        B.join_batch(store, db, 0, *outs[i % 2])
+    torch.cuda.synchronize()
+    for (rows, mask), (want_rows, want_mask) in zip(outs, wants):
+        assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
+    assert store.device_status() == B.CCR_OK
+    store.free()

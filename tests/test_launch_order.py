@@ -31,3 +31,13 @@ def test_no_exit_of_a_join_kernel_without_the_wait(file, name):
     assert len(exits) == 2  # a block without work, and the streamers
     for e in exits:
         assert body[:e].rstrip().endswith(wait)
+
+
+def test_document_rows_are_fetched_behind_the_wait():
+    """Rows of the store are inputs that the launch in front may have written: an upsert followed by a join on one stream."""
+    body = _kernel_body("ccr_ws.cuh", "join_ws_kernel")
+    fetch = [m.start() for m in re.finditer(r"\bfetch_docs\(\);", body)]
+    assert body[:fetch[0]].rstrip().endswith("pdl_wait();")
+    role = body[body.index("if (role_rank >= n_res)"):]
+    first = role.index("pdl_wait();")
+    assert not re.search(r"\bemit_group\b|\bfetch_docs\(\)", role[:first])  # (the lambda is no call)
