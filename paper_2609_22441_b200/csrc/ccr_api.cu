@@ -1088,7 +1088,29 @@ ccr_status ccr_docstore_selftest_wait(ccr_docstore* s, void* stream) {
 }  // extern "C"
 
 namespace {
-// ccr_join_batch (n_max == 0, ragged output) and ccr_join_batch_padded (n_max > 0) share everything but the
+// The rows of a padded output that no candidate fills.  join_follows: the join of the same call is launched right behind (its
+// arguments have been checked) and may start beside them.
+ccr_status launch_pads(ccr_docstore* s, int32_t n_req, int64_t n_max, const int64_t* cand_offsets, void* out_rows, uint8_t* out_mask,
+                       uint32_t flags, cudaStream_t st, bool join_follows) {
+#ifdef CCR_DEBUG_BOUNDS
+  {
+    DbgRegistrar reg;
+    const size_t out_b = out_row_bytes(s, flags);
+    reg.add(cand_offsets, static_cast<size_t>(n_req + 1) * 8);
+    reg.add(out_rows, static_cast<size_t>(n_req) * n_max * out_b);
+    reg.add(out_mask, static_cast<size_t>(n_req) * n_max);
+    if (cudaStreamSynchronize(st) != cudaSuccess || !reg.commit(s->status + 2)) return CCR_ERR_CUDA;
+  }
+#endif
+  // enough blocks to fill the device however few requests there are
+  const unsigned slices = static_cast<unsigned>(std::max(1, std::min(64, (2 * s->n_sms + n_req - 1) / n_req)));
+  launch_chained(ccr::pad_fill_kernel, dim3(static_cast<unsigned>(n_req), slices), dim3(ccr::kPadThreads), 0, st, cand_offsets, n_max,
+                 static_cast<long long>(out_row_bytes(s, flags)), static_cast<uint8_t*>(out_rows), out_mask, join_follows ? 1 : 0);
+  s->launches++;
+  return cudaGetLastError() == cudaSuccess ? CCR_OK : CCR_ERR_CUDA;
+}
+
+// ccr_join_batch (n_max == 0, ragged output) and ccr_join_batch_padded (n_max > 0: the pads first) share everything but the
 // output addressing.
 // read_ahead false: the launch directly in front is a kernel that writes the inputs.  Its end is no point at which its writes are
 // promised to be visible to a launch that has not executed griddepcontrol.wait, so the warp-specialised kernel, which reads its
@@ -1260,6 +1282,10 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
   DeviceScope scope(s->desc.device);
   if (!scope.ok) return CCR_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (n_max > 0) {
+    const ccr_status pads = launch_pads(s, n_req, n_max, cand_offsets, out_rows, out_mask, flags, st, true);
+    if (pads != CCR_OK) return pads;
+  }
 #ifdef CCR_DEBUG_BOUNDS
   {
     // the true sizes of the ragged arrays are on the device: read them back (this build synchronises anyway)
@@ -1402,28 +1428,12 @@ ccr_status padded_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cand
   if (flags & CCR_FLAG_VALIDATE) return CCR_ERR_UNSUPPORTED;  // validate with ccr_join_batch semantics first
   if (n_req == 0) return CCR_OK;
   if (!cand_offsets || !out_rows || !out_mask) return CCR_ERR_INVALID_ARG;
-  ccr_docstore* s = const_cast<ccr_docstore*>(cs);
-  {
+  if (total_cands == 0) {
+    ccr_docstore* s = const_cast<ccr_docstore*>(cs);
     DeviceScope scope(s->desc.device);
     if (!scope.ok) return CCR_ERR_CUDA;
-#ifdef CCR_DEBUG_BOUNDS
-    {
-      DbgRegistrar reg;
-      const size_t out_b = out_row_bytes(s, flags);
-      reg.add(cand_offsets, static_cast<size_t>(n_req + 1) * 8);
-      reg.add(out_rows, static_cast<size_t>(n_req) * n_max * out_b);
-      reg.add(out_mask, static_cast<size_t>(n_req) * n_max);
-      if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess || !reg.commit(s->status + 2)) return CCR_ERR_CUDA;
-    }
-#endif
-    // enough blocks to fill the device however few requests there are
-    const unsigned slices = static_cast<unsigned>(std::max(1, std::min(64, (2 * s->n_sms + n_req - 1) / n_req)));
-    launch_chained(ccr::pad_fill_kernel, dim3(static_cast<unsigned>(n_req), slices), dim3(ccr::kPadThreads), 0, static_cast<cudaStream_t>(stream),
-                   cand_offsets, n_max, static_cast<long long>(out_row_bytes(s, flags)), static_cast<uint8_t*>(out_rows), out_mask);
-    s->launches++;
-    if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
+    return launch_pads(s, n_req, n_max, cand_offsets, out_rows, out_mask, flags, static_cast<cudaStream_t>(stream), false);
   }
-  if (total_cands == 0) return CCR_OK;
   return join_impl(cs, n_req, total_cands, max_edge_len, edge_keys, edge_feats, edge_offsets, cand_idx, cand_offsets,
                    req_feats, out_rows, out_mask, flags, stream, n_max, member_emb);
 }

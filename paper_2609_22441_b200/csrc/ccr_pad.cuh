@@ -167,11 +167,12 @@ compact_valid_kernel(const int32_t* cand_idx, const int64_t* cand_offsets, long 
 // Step 3's pads: rows [n_r, n_max) of request r are zero rows with mask 0.  Blocks (r, 0 .. gridDim.y) share
 // request r's pad range; 16-byte streaming stores (out_b is a multiple of 16).
 __global__ void __launch_bounds__(kPadThreads)
-pad_fill_kernel(const int64_t* cand_offsets, long long n_max, long long out_b, uint8_t* out_rows, uint8_t* out_mask) {
-  // The join behind it may start at once: it writes other rows, and what it reads was written before this kernel, which has waited
-  // for that (request flow 317.5 -> 313.9 us, with the scan that count_scan_kernel saves).
+pad_fill_kernel(const int64_t* cand_offsets, long long n_max, long long out_b, uint8_t* out_rows, uint8_t* out_mask, int join_follows) {
+  // The join of the same call may start at once: it writes other rows, and what it reads was written before this kernel, which has
+  // waited for that (request flow 317.5 -> 313.9 us, with a launch less in the compaction).  Nothing else may: whatever follows the
+  // pads of a call without a join could read them.
   pdl_wait();
-  pdl_trigger();
+  if (join_follows) pdl_trigger();
   const int r = blockIdx.x;
   long long n_r = gload(cand_offsets + r + 1) - gload(cand_offsets + r);
   n_r = n_r < 0 ? 0 : (n_r > n_max ? n_max : n_r);

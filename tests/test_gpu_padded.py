@@ -239,3 +239,31 @@ def test_config1_full_size_padded_equals_ragged_rows_in_place(B):
         assert store.device_status() == B.CCR_OK
     finally:
         store.free()
+
+
+def test_pads_without_a_join_are_there_for_the_launch_behind_them(B):
+    """A padded call without candidates, and directly behind it a join whose candidate positions are the padded rows."""
+    wl = W.config1(n_docs=20_000, n_req=1, n_cand=10)
+    store, db = B.store_from_workload(wl), B.DeviceBatch(wl.batch)
+    out_b, n_max = store.out_row_bytes(), 2_000
+    T = torch.zeros((4, n_max, out_b), dtype=torch.uint8, device="cuda")
+    M = torch.zeros((4, n_max), dtype=torch.uint8, device="cuda")
+    none = torch.zeros(5, dtype=torch.int64, device="cuda")
+    cands = T.view(torch.int32).reshape(-1)
+    n = cands.numel()
+    co = torch.tensor([0, n], dtype=torch.int64, device="cuda")
+    rows = torch.zeros((n, out_b), dtype=torch.uint8, device="cuda")
+    mask = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    b = wl.batch
+    two = W.assemble_batch([b.edge_keys], [b.edge_feats], [np.array([0, 7], np.int32)], b.req_feats, b.edge_dim, b.edge_dtype, b.req_dim, b.req_dtype)
+    want_rows, want_mask = oracle.join_workload(W.Workload("two", 0, wl.store, two))
+    assert not np.array_equal(want_rows[0], want_rows[1])
+    want = torch.from_numpy(want_rows[0]).cuda()
+    for _ in range(10):
+        cands.fill_(7)
+        torch.cuda.synchronize()
+        B.ccr_join_batch_padded(store, 4, 0, db.max_edge_len, n_max, db.edge_keys, db.edge_feats, none, db.cand_idx, none, db.req_feats, T, M)
+        B.ccr_join_batch(store, 1, n, db.max_edge_len, db.edge_keys, db.edge_feats, db.edge_offsets, cands, co, db.req_feats, rows, mask)
+        torch.cuda.synchronize()
+        assert bool((rows == want).all()) and bool((mask == int(want_mask[0])).all())
+    store.free()

@@ -24,3 +24,13 @@ def test_compaction_keeps_no_state_in_the_store():
     assert body.count("launch_chained(") == 2
     assert "status" not in body.replace("ccr_status", "") and "kSchedRegions" not in body
     assert "atomic" not in _function("ccr_pad.cuh", "count_valid_kernel(") + _function("ccr_pad.cuh", "compact_valid_kernel(")
+
+
+def test_pads_let_only_the_join_of_their_call_start_early():
+    """What follows the pads of a call without a join may read them: it is ordered behind their last store."""
+    kernel = _function("ccr_pad.cuh", "pad_fill_kernel(")
+    assert kernel.index("pdl_wait();") < kernel.index("if (join_follows) pdl_trigger();") and kernel.count("pdl_trigger") == 1
+    join, padded = _function("ccr_api.cu", "ccr_status join_impl("), _function("ccr_api.cu", "ccr_status padded_impl(")
+    assert "launch_pads(" in padded and ", false)" in padded[padded.index("launch_pads("):]
+    at = join.index("launch_pads(")
+    assert ", true)" in join[at:] and "CCR_ERR_INVALID_ARG" not in join[at:] and "CCR_ERR_UNSUPPORTED" not in join[at:]
