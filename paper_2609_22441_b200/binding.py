@@ -182,6 +182,8 @@ def _dtype_code(dt) -> int:
 # A small call is bound by the host: what runs once per argument or per call goes without attribute lookups (one request of 1,000
 # candidates 10.3 -> 7.0 us a call together with the stream below, which took 3 us of it).
 _Tensor = torch.Tensor
+# (an interface inside torch: a version without it takes the stream object)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _ptr(x) -> Optional[int]:
@@ -201,7 +203,9 @@ def _ptr(x) -> Optional[int]:
 
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:  # the handle of torch.cuda.current_stream() without the stream object around it
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device()) or None
+        return torch.cuda.current_stream().cuda_stream or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return int(stream) or None
