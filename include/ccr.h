@@ -185,13 +185,15 @@ size_t ccr_out_row_bytes(const ccr_docstore* store, uint32_t flags);
  * Back-to-back joins.  Both join kernels are launched with programmatic stream serialization.  The two-phase kernel (the
  * default for ragged launches of at most 131,072 candidates without the cosine section) waits for everything in front of it
  * on `stream` before it reads its inputs: it is in stream order.  The warp-specialised kernel reads ahead: when the work in
- * front of it is another warp-specialised join, its blocks take over each SM as soon as that join's block there has retired
- * and read their own inputs (offsets, keys, candidate positions, ids) while the earlier join drains; they write nothing —
- * rows, mask — before the earlier join has completed, so reusing the output buffers of the previous call is safe, and any
- * other kernel, copy or event on the stream orders the launch as usual, unless that kernel itself lets dependent launches in
- * before its last store (a programmatic launch trigger).  What is NOT ordered is a warp-specialised join that reads, as an
- * input, memory which such a kernel or the join directly in front of it writes (its rows or mask reinterpreted as keys or
- * positions): give such a call CCR_FLAG_NO_OVERLAP.                                                                  */
+ * front of it is another warp-specialised join of the same store, its blocks take over each SM as soon as that join's block
+ * there has retired and read some of their own inputs (offsets, keys, positions, ids, member embeddings; in a padded call also beside
+ * the pads of that call) while the earlier join drains; they read no feature rows and write nothing — rows, mask — before the
+ * earlier join has completed, so reusing the output buffers of the previous call is safe.  A block finds out on the device
+ * whether that join is still running; behind anything else — another kernel, copy or event, of this library or not — it waits
+ * for the end of that work before it reads at all, unless that is a kernel that itself lets dependent launches in before its
+ * last store (a programmatic launch trigger).  What is NOT ordered is a warp-specialised join that reads, as an input, memory
+ * which such a kernel or the join directly in front of it writes (its rows or mask reinterpreted as keys or positions): give
+ * such a call CCR_FLAG_NO_OVERLAP.                                                                                    */
 ccr_status ccr_join_batch(const ccr_docstore* store,
                           int32_t n_req, int64_t total_cands, int64_t max_edge_len,
                           const int64_t* edge_keys,    /* DEVICE [E]                               */

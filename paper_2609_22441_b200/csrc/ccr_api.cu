@@ -59,6 +59,7 @@ constexpr size_t kStageBytes = 16u << 20;  // staging block of second-degree sto
 constexpr size_t kKernelCopyBytes = 16u << 20;
 constexpr int kHostGroups = CCR_HOST_GROUPS;         // most request groups of a pipelined host-buffer join
 constexpr int kSchedRegions = 64;                    // launches of one store that may be in flight at once
+constexpr int kLastJoins = 8;                        // streams of a store whose last join is known
 constexpr int kStatusHead = 4;                       // [0] wait expiry, [1] validation code; then the scheduling words:
                                                      // kSchedRegions regions of sched_stride ints
 
@@ -101,6 +102,16 @@ struct ccr_docstore {
   int64_t dbg_shrink_rows;             // bounds-checked build: rows cut off the registered output extents
   std::atomic<int64_t> launches;  // kernels launched for this store; also hands out the scheduling-word pairs
   std::atomic<int64_t> sort_calls;  // chunked ccr_sort_edges calls; hands out their flag words
+  // the last warp-specialised join of each of a few streams (the oldest entry makes room), for the next one's look at what is in front
+  struct LastJoin {
+    cudaStream_t stream;
+    unsigned long long capture;  // the capture it became part of; 0: launched
+    int ticket;                  // 0: no entry
+  };
+  std::mutex last_joins_mutex;
+  LastJoin last_joins[kLastJoins];
+  int last_joins_next;
+  int* running;  // device: kSchedRegions x n_sms words (JoinArgs::running)
 };
 
 struct ccr_workspace {
@@ -365,6 +376,45 @@ ccr_status dbg_finish(int* word, cudaStream_t st) {
 }
 #endif
 
+// The capture that launches on `st` become part of (0: none; kNoCapture: cannot be told).  A ticket of a launch outside of it, or of
+// another capture, says nothing about what a replay finds in front.
+constexpr unsigned long long kNoCapture = ~0ull;
+unsigned long long capture_of(cudaStream_t st) {
+  if (st == cudaStreamPerThread) return kNoCapture;  // one handle, another stream for every thread
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return kNoCapture;
+  }
+  return status == cudaStreamCaptureStatusNone ? 0 : id;
+}
+
+int last_join(ccr_docstore* s, cudaStream_t st, unsigned long long capture) {
+  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
+  for (const auto& e : s->last_joins)
+    if (e.ticket != 0 && e.stream == st && e.capture == capture && capture != kNoCapture) return e.ticket;
+  return 0;
+}
+
+void forget_last_join(ccr_docstore* s, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
+  for (auto& e : s->last_joins)
+    if (e.stream == st) e.ticket = 0;
+}
+
+void set_last_join(ccr_docstore* s, cudaStream_t st, unsigned long long capture, int ticket) {
+  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
+  ccr_docstore::LastJoin* to = nullptr;
+  for (auto& e : s->last_joins)
+    if (e.stream == st) to = &e;
+  if (to == nullptr) {
+    to = &s->last_joins[s->last_joins_next];
+    s->last_joins_next = (s->last_joins_next + 1) % kLastJoins;
+  }
+  *to = {st, capture, ticket};
+}
+
 // Launch of a kernel that belongs to a chain of small launches (its first statement is chain_enter()): with
 // programmatic stream serialization the launch is set up while the kernel in front of it still runs.
 // `cluster` blocks form a thread-block cluster.
@@ -550,6 +600,8 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
   const size_t status_ints = kStatusHead + static_cast<size_t>(kSchedRegions) * s->sched_stride;
   ok = ok && cudaMalloc(&s->status, status_ints * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMemset(s->status, 0, status_ints * sizeof(int)) == cudaSuccess;
+  const size_t running_bytes = static_cast<size_t>(kSchedRegions) * s->n_sms * sizeof(int);
+  ok = ok && cudaMalloc(&s->running, running_bytes) == cudaSuccess && cudaMemset(s->running, 0, running_bytes) == cudaSuccess;
   ok = ok && cudaHostAlloc(&s->status_host, 4 * sizeof(int), cudaHostAllocDefault) == cudaSuccess;
   ccr_status st = ok ? allow_large_smem() : CCR_ERR_OOM;
   if (st != CCR_OK) {
@@ -559,6 +611,7 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
     cudaFree(s->id_recs);
     cudaFree(s->stage);
     cudaFree(s->status);
+    cudaFree(s->running);
     if (s->status_host) cudaFreeHost(s->status_host);
     delete s;
     return st;
@@ -578,6 +631,7 @@ ccr_status ccr_docstore_free(ccr_docstore* s) {
   cudaFree(s->id_recs);
   cudaFree(s->stage);
   cudaFree(s->status);
+  cudaFree(s->running);
   cudaFreeHost(s->status_host);
   delete s;
   return CCR_OK;
@@ -691,6 +745,7 @@ ccr_status ccr_docstore_upsert(ccr_docstore* s, int64_t n, const int32_t* positi
   long long blocks = (work + per_block - 1) / per_block;
   const long long cap = static_cast<long long>(s->n_sms) * 8;
   blocks = blocks < 1 ? 1 : (blocks > cap ? cap : blocks);
+  forget_last_join(s, static_cast<cudaStream_t>(stream));  // (it need not look for a join that has long completed)
   launch_chained(ccr::upsert_kernel, dim3(static_cast<unsigned>(blocks)), dim3(ccr::kUpsertThreads), 0, static_cast<cudaStream_t>(stream), a);
   s->launches++;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
@@ -1112,14 +1167,11 @@ ccr_status launch_pads(ccr_docstore* s, int32_t n_req, int64_t n_max, const int6
 
 // ccr_join_batch (n_max == 0, ragged output) and ccr_join_batch_padded (n_max > 0: the pads first) share everything but the
 // output addressing.
-// read_ahead false: the launch directly in front is a kernel that writes the inputs.  Its end is no point at which its writes are
-// promised to be visible to a launch that has not executed griddepcontrol.wait, so the warp-specialised kernel, which reads its
-// inputs before it waits, is then launched in plain stream order.
 ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands, int64_t max_edge_len,
                      const int64_t* edge_keys, const void* edge_feats, const int64_t* edge_offsets,
                      const int32_t* cand_idx, const int64_t* cand_offsets, const void* req_feats,
                      void* out_rows, uint8_t* out_mask, uint32_t flags, void* stream, int64_t n_max,
-                     const void* member_emb, int* sched_override = nullptr, bool read_ahead = true) {
+                     const void* member_emb, int* sched_override = nullptr) {
   if (!good(cs)) return CCR_ERR_BAD_HANDLE;
   ccr_docstore* s = const_cast<ccr_docstore*>(cs);  // only the launch counter and status words change
   if (n_req < 0 || total_cands < 0 || max_edge_len < 0) return CCR_ERR_INVALID_ARG;
@@ -1345,11 +1397,18 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     // (the pair is drawn from the atomic launch counter, so host threads that join against one store at the
     // same time never share a pair)
     const int64_t seq = s->launches.fetch_add(1);
+    a.n_words = s->n_sms;
+    a.running = s->running + (seq % kSchedRegions) * s->n_sms;
+    a.ticket = static_cast<int>(static_cast<uint32_t>(seq) | 0x80000000u);
+    const unsigned long long capture = capture_of(st);
+    a.front_ticket = last_join(s, st, capture);
+    a.front_running = a.front_ticket != 0 ? s->running + (static_cast<uint32_t>(a.front_ticket) % kSchedRegions) * s->n_sms : nullptr;
+    a.behind_pads = n_max > 0 ? 1 : 0;
     if (dynamic) a.sched = sched_override ? sched_override : s->status + kStatusHead + s->sched_stride * static_cast<int>(seq % kSchedRegions);
     // Launched with programmatic stream serialization: behind another join on the same stream the blocks become
     // resident as that join's blocks leave their SMs and prepare (barriers, offsets, first keys, first ids and
     // searches) while it drains; they store nothing before it has completed (griddepcontrol.wait in the kernel).
-    // Behind any other kernel, copy or event the launch is ordered as usual.
+    // Behind any other kernel, copy or event they read nothing before that wait either.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(blocks));
     cfg.blockDim = dim3(static_cast<unsigned>((n_str + n_res) * 32));
@@ -1359,11 +1418,12 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = ((flags & CCR_FLAG_NO_OVERLAP) || !read_ahead) ? 0 : 1;
+    cfg.numAttrs = (flags & CCR_FLAG_NO_OVERLAP) ? 0 : 1;
     if (cudaLaunchKernelEx(&cfg, fn, a, n_str) != cudaSuccess) {
       cudaGetLastError();
       return CCR_ERR_CUDA;
     }
+    set_last_join(s, st, capture, a.ticket);
   } else {
     // persistent two-phase kernel: as many blocks as stay resident, each with at least 64 candidates (a single
     // small request is spread over many SMs: 21.6 against 23.4 us for 1,000 candidates with 256 per block)
@@ -1683,7 +1743,7 @@ ccr_status ccr_join_batch_host(const ccr_docstore* s, ccr_workspace* w, int32_t 
     if (flags & CCR_FLAG_COSINE) return CCR_ERR_INVALID_ARG;  // the member embeddings come through ccr_join_batch_ex
     const ccr_status js = join_impl(s, n_req, total_cands, max_edge_len, w->edge_keys, w->edge_feats, w->edge_offsets, w->cand_idx,
                                     w->cand_offsets, s->req_b ? w->req_feats : nullptr, w->out_rows, w->out_mask, flags, stream, 0,
-                                    nullptr, nullptr, !by_kernel);
+                                    nullptr);
     if (js != CCR_OK) return js;
   } else {
     // group boundaries: request ranges [first[g], first[g + 1]) with about total_cands / n_groups candidates each
@@ -1879,7 +1939,7 @@ ccr_status ccr_join_payload_static(const ccr_docstore* s, int32_t n_req, int64_t
                                   base + o_feats, reinterpret_cast<const int64_t*>(base + o_eo),
                                   reinterpret_cast<const int32_t*>(base + o_idx),
                                   reinterpret_cast<const int64_t*>(base + o_co), s->req_b > 0 ? base + o_req : nullptr,
-                                  out_rows, out_mask, flags, stream, 0, nullptr, reinterpret_cast<int*>(base), !in.ok);
+                                  out_rows, out_mask, flags, stream, 0, nullptr, reinterpret_cast<int*>(base));
   return js;
 }
 

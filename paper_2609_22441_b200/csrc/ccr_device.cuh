@@ -73,6 +73,12 @@ struct JoinArgs {
   int warp_search;            // searches that run in global memory use the warp-cooperative 32-ary search (comparison aid)
   int* status;                // device status words
   int* sched;                 // two scheduling words (next tile, finished blocks), zero between launches; or null
+  // reading ahead (warp-specialised kernel): a word per block that holds the launch's ticket while the block runs
+  int* running;
+  const int* front_running;   // the same words of the last such launch on this stream; null: none
+  int ticket, front_ticket;   // never 0
+  int n_words;                // words of a launch
+  int behind_pads;            // the launch in front writes the pads of this call's output
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -140,7 +146,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
 }
 
 // Programmatic dependent launch.  A launch of the warp-specialised join right behind another one on the same stream may become
-// resident while the earlier one drains (as its blocks leave their SMs) and run everything that only reads its own inputs;
+// resident while the earlier one drains (as its blocks leave their SMs) and run everything that only reads its own inputs, provided
+// that one is still running (join_in_front() in ccr_ws.cuh);
 // pdl_wait() returns once the earlier grid has completed and its writes are visible, and comes before the first
 // global store.  The two-phase join waits before it reads anything.  pdl_trigger() tells the runtime that this block no longer
 // needs to hold back a dependent launch.  Both are no-ops for a launch without the attribute or without a predecessor that triggers.
@@ -151,7 +158,7 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // memory only after the launch in front of it has completed; when another kernel of the same chain follows
 // (more_follow), that launch may be set up right away and will wait in the same way, so the launch gaps inside the
 // chain overlap.  The LAST kernel of a chain never lets its successor in early: whatever is launched behind the chain
-// (a join, whose resolver warps read their inputs without waiting) starts only after the whole chain has completed.
+// starts only after the whole chain has completed.
 __device__ __forceinline__ void chain_enter(bool more_follow) {
   if (more_follow) pdl_trigger();
   pdl_wait();
@@ -199,7 +206,7 @@ __device__ __forceinline__ T gload_rw(const T* p) {
   if (!CCR_CHK(p, static_cast<int>(sizeof(T)))) return T{};
   return *p;
 }
-// load past L1 of what other blocks of the same launch may be writing
+// load past L1 of what another block, or the launch in front, may be writing
 __device__ __forceinline__ int64_t gload_shared_out(const int64_t* p) {
   if (!CCR_CHK(p, 8)) return 0;
   return __ldcg(reinterpret_cast<const long long*>(p));

@@ -109,3 +109,53 @@ def test_forced_staging_of_the_longest_lists(k):
     torch.cuda.synchronize()
     assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
     store.free()
+
+
+@pytest.mark.parametrize("second", [False, True])
+def test_positions_written_between_two_joins_on_many_streams_and_in_graphs(second):
+    """Joins with a kernel between them that writes the second one's candidate positions, on more streams than a store keeps the last
+    join of, launched and captured; the launches of a replay stand beside direct ones on other streams."""
+    from paper_2609_22441_b200 import binding as B
+
+    wl = W.config1(seed=3, n_docs=120_000, n_req=6, n_cand=24_000, second_degree=second)
+    b = wl.batch
+    cand_b = np.random.default_rng(4).permutation(b.cand_idx)
+    wants = [oracle.join_workload(w, n_threads=4) for w in (wl, W.Workload("b", 0, wl.store, W.Batch(**{**b.__dict__, "cand_idx": cand_b})))]
+    store, db = B.store_from_workload(wl), B.DeviceBatch(b)
+    cands = [db.cand_idx, torch.from_numpy(cand_b).cuda()]
+    out_b = store.out_row_bytes()
+    streams = [torch.cuda.Stream() for _ in range(11)]
+    bufs = [dict(scratch=cands[0].clone(), rows=torch.zeros((b.total_cands, out_b), dtype=torch.uint8, device="cuda"),
+                 mask=torch.zeros(b.total_cands, dtype=torch.uint8, device="cuda")) for _ in streams]
+
+    def join(buf, idx, st):
+        B.ccr_join_batch(store, db.n_req, db.total_cands, db.max_edge_len, db.edge_keys, db.edge_feats, db.edge_offsets, idx, db.cand_offsets,
+                         db.req_feats, buf["rows"], buf["mask"], 0, st)
+
+    def steps(i, buf, st):  # ends with batch i % 2 in the rows
+        join(buf, cands[1 - i % 2], st)
+        buf["scratch"].copy_(cands[i % 2])
+        join(buf, buf["scratch"], st)
+
+    torch.cuda.synchronize()
+    graphs = []
+    for k in range(2):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[k]):
+            steps(k, bufs[k], streams[k])
+            steps(k + 1, bufs[k], streams[k])
+        graphs.append(g)
+    torch.cuda.synchronize()
+    for i in range(12):
+        for k, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                if k < len(graphs):
+                    graphs[k].replay()
+                else:
+                    steps(i + k, bufs[k], st)
+    torch.cuda.synchronize()
+    for k, buf in enumerate(bufs):
+        want_rows, want_mask = wants[(k + 1) % 2 if k < len(graphs) else (11 + k) % 2]
+        assert np.array_equal(buf["mask"].cpu().numpy(), want_mask) and np.array_equal(buf["rows"].cpu().numpy(), want_rows)
+    assert store.device_status() == B.CCR_OK
+    store.free()

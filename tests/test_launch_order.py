@@ -41,3 +41,21 @@ def test_document_rows_are_fetched_behind_the_wait():
     role = body[body.index("if (role_rank >= n_res)"):]
     first = role.index("pdl_wait();")
     assert not re.search(r"\bemit_group\b|\bfetch_docs\(\)", role[:first])  # (the lambda is no call)
+
+
+def test_inputs_are_read_ahead_only_of_a_join_that_is_still_running():
+    """The end of a kernel is no point at which its writes are promised to be visible to a launch that has not waited, so a block looks
+    for the ticket of the join in front before it reads anything, and the ticket is there from before the trigger to the block's end."""
+    body = _kernel_body("ccr_ws.cuh", "join_ws_kernel")
+    settled = body.index("if (__syncthreads_or(in_front) == 0 && may_read_ahead(a)) {")
+    behind = body[settled:]
+    assert re.match(r"[^}]*\{\s*pdl_wait\(\);\s*if \(n_req_cached > 0\) mirror_offsets\(\);\s*__syncthreads\(\);\s*\}", behind)
+    early = body[:settled]
+    assert "if (!may_read_ahead(a)) pdl_wait();" in early and early.index("may_read_ahead") < early.index("mirror_offsets();  ".strip())
+    # in front of it only the offsets are read, past L1, and they are read again
+    assert not re.search(r"\bgload\(|\bstage_keys\b|\ba\.(cand_idx|edge_keys|sched)\s*[+\[]", early)
+    assert early.index("a.running + blockIdx.x) = a.ticket;") > 0
+    assert re.search(r"__threadfence\(\);\s*pdl_trigger\(\);", body) and body.count("pdl_trigger()") == 1
+    assert body.count("a.running + blockIdx.x) = 0;") == len(re.findall(r"\breturn;", body))
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "ccr_api.cu")).read())
+    assert "a.behind_pads = n_max > 0 ? 1 : 0;" in src and src.count("behind_pads") == 1
