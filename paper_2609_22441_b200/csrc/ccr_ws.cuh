@@ -26,13 +26,13 @@
 // were measured and lost 7-9 % on every configuration: all blocks walking one window of the candidate range
 // together is what the memory system likes.)
 //
-// PIPE (second-degree joins of the tuned widths): a streamer's document rows pass through shared memory.  What kept these
+// PIPE (second-degree joins of the tuned widths, where join_impl says so): a streamer's document rows pass through shared memory.  What kept these
 // joins from the memory's rate was the time a streamer spends on the edge2 section with no document row under way, and the
 // registers of its row loads.  Here a warp has a buffer of 32 rows: one bulk copy per row fetches the next group's while
 // the edge, edge2 and request sections of the group under way are written, so the warp needs no registers for them, both roles fit 96
 // (nothing spills, no setmaxnreg), and match indices of 16 bits make room in the ring.  50,000 x 256 with 128-byte edge
-// rows 2,423 -> 2,289 us, 30,000 x 64 with 128-byte edge rows 333-502 -> 315-343 us, with 64-byte ones 280 +- 4 us either way.  Measured and
-// slower: the same for first-degree joins (206 -> 222, 1,658 -> 1,906 us: their rows already fill the time) and with the cosine section
+// rows 2,423 -> 2,289 us, 30,000 x 64 with 128-byte edge rows 356-391 (16 warps) -> 315-347 us; 64-byte ones beside the rule in join_impl.
+// Measured and slower: the same for first-degree joins (206 -> 222, 1,658 -> 1,906 us: their rows already fill the time) and with the cosine section
 // (request flow 321 -> 396 us); 8 + 8, 8 + 12, 10 + 10, 12 + 10 and 12 + 12 warps; four candidates per resolver lane.
 #pragma once
 
@@ -136,7 +136,7 @@ struct WsLayout {
 // that was launched last on this stream is still running (some block of it shows its ticket), so nothing has run between the two; or
 // the launch in front writes the pads of this call's output, which has waited itself for what is in front of it.  The end of any other
 // kernel is no point at which its writes are promised to be visible to a launch that has not waited.  Reading ahead is worth 6 us of 207
-// (64 x 30,000) and 8 of 292 (second degree) to joins back to back, the look itself costs 0.5 us; where nothing is running in front, the wait costs nothing.
+// (64 x 30,000) and 8 of 292 (second degree) to joins back to back, the look itself costs up to 0.5 us; where nothing is running in front, the wait costs nothing.
 __device__ __forceinline__ bool may_read_ahead(const JoinArgs& a) { return a.front_running != nullptr || a.behind_pads != 0; }
 __device__ __forceinline__ bool join_in_front(const JoinArgs& a) {  // (this thread's share of the words)
   bool running = a.behind_pads != 0;
@@ -642,10 +642,8 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   }
 
   // no more work will be drawn by this block: a join queued behind this one may start to move in
-  if (gtid == 0) {
-    __threadfence();  // it will look for this block's ticket
-    pdl_trigger();
-  }
+  // (that it finds this block's ticket is not promised, only likely: without it, it waits)
+  if (gtid == 0) pdl_trigger();
 
   // stop slot: published by the warp whose turn it is
   if (static_cast<int>(it % n_resolvers) == rwarp && !dead) {

@@ -50,6 +50,18 @@ def test_sort_resolve_compaction_and_upsert_run_clean_under_the_bounds_checked_b
     assert " passed" in out.stdout
 
 
+def test_descent_regions_and_staged_rows_run_clean_under_the_bounds_checked_build(debug_lib):
+    """Resolution with levels below the top one and around the regions, in both forms of the buckets, and second-degree joins whose
+    document rows pass through shared memory."""
+    env = dict(os.environ, CCR_LIB_OVERRIDE=debug_lib)
+    out = subprocess.run(
+        [sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "tests/test_gpu_resolve_descent.py", "tests/test_gpu_resolve_regions.py",
+         "tests/test_gpu_staged_second.py", "-k", "not (added and 67)"],
+        cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)
+    assert out.returncode == 0, out.stdout[-3000:] + out.stderr[-2000:]
+    assert " passed" in out.stdout
+
+
 def test_a_sort_whose_output_rows_end_early_is_reported_and_skips_the_row(debug_lib):
     code = r"""
 import numpy as np, torch
