@@ -94,8 +94,9 @@ enum {
   CCR_FLAG_COSINE            = 1u << 8, /* append the derived cosine section (ccr_docstore_set_cosine,
                                            ccr_join_batch_ex); adds 32 bytes to the row                */
   CCR_FLAG_NO_REBALANCE      = 1u << 10, /* second-degree joins: keep the 16-warp form of the warp-specialised kernel
-                                           instead of its 20-warp form with registers moved from the search warps to
-                                           the row-streaming warps (comparison aid)                                  */
+                                           instead of a 20-warp form (document rows passing through shared memory, or
+                                           registers moved from the search warps to the row-streaming warps;
+                                           comparison aid)                                                           */
   CCR_FLAG_NO_OVERLAP        = 1u << 11, /* do not let this launch move in behind a join that is still draining on the same
                                            stream (see "Back-to-back joins" at ccr_join_batch)                       */
   CCR_FLAG_WARP_SEARCH       = 1u << 12, /* lists that are searched in global memory (CCR_FLAG_FORCE_GLOBAL, key capacity 0)

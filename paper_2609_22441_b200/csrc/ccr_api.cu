@@ -36,6 +36,7 @@ constexpr int kDefaultTileTwoPhase = 1024; // candidates per search/copy phase p
 constexpr int kSmemPerSm = 228 * 1024;
 constexpr int kDefaultKeyCap = 4096;
 constexpr long long kSmallLaunchCands = 131072;  // plain launches up to this size default to the two-phase kernel
+constexpr long long kStagedMinCands = 1 << 20;  // 64-byte edge rows: smallest launch with staged document rows (join_impl)
 constexpr int kAutoSmemBudget = 160 * 1024;  // shared memory the warp-specialised kernel takes by default
 constexpr long long kIdsInL2Bytes = 64LL << 20;  // an author-id array up to this size is taken to stay in the 126 MB L2
 constexpr int kMaxTile = ccr::kMaxTileCands;
@@ -1209,16 +1210,26 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     if (!use_ws) return CCR_ERR_UNSUPPORTED;  // the derived section is computed by the warp-specialised kernel only
     if (reinterpret_cast<uintptr_t>(member_emb) & 1u) return CCR_ERR_INVALID_ARG;
   }
-  // second-degree joins on the default warp split take the register-rebalanced form (12 + 8 warps); a configured
-  // split, a configured sub-tile and the cosine section keep the 16-warp kernel
+  // second-degree joins on the default warp split take a form of 12 + 8 warps; a configured split, a configured sub-tile and the cosine
+  // section keep the 16-warp kernel
   const bool cos_tuned = cos && (s->cos_dim + 7) / 8 == kTunedCosPieces;
   const Variant& v = (cos && !cos_tuned) ? kVariants[kNumVariants - 1] : pick_variant(s->doc_b / 16, s->edge_b / 16, s->req_b / 16);
   const bool rebalanced = use_ws && second && !cos && s->ws_streamers == 0 && s->tile == 0 && !(flags & CCR_FLAG_NO_REBALANCE);
-  // ... and, over rows of the tuned widths, its form with staged document rows, unless an explicit key capacity may need the shared
-  // memory that these take or a match index may not fit 16 bits.  (128-byte edge rows then take the 16-warp form: 387 us on 30,000 x 64
-  // with 64-byte request rows, 502 us rebalanced, 343 us staged; 64-byte ones 335, 284 and 287 us.)
+  // That is the one with staged document rows for 128-byte edge rows of the tuned widths (30,000 x 64 without / with 64-byte request rows 315 /
+  // 347 us, 16 warps 356 / 391, registers moved 367 / 415), unless an explicit key capacity may need the shared memory that the rows take or
+  // a match index may not fit 16 bits: then 16 warps.  With 64-byte edge rows it is ahead of the form with moved registers only where the
+  // launch is large and every list fits beside its table in what the rows leave.  Moved registers -> staged, without a request section:
+  // 240,000 candidates 49 -> 51 us, 480,000 81 -> 82, 960,000 145 -> 145, 1,290,000 191 -> 187, 1,590,000 234 -> 227, 1,920,000 281 -> 271;
+  // these against lists of 3,000 keys 296 -> 293, 5,000 296 -> 298, 6,000 329 -> 347, 20,000 366 -> 431.  With one: 240,000 candidates
+  // 49 -> 53, 1,920,000 289 -> 289, against lists of at most 500 keys 288 -> 280, 8,000 360 -> 384, 20,000 391 -> 450.
   const bool explicit_cap = (flags & CCR_FLAG_FORCE_SMEM) || s->key_cap > 0;
-  const bool staged = rebalanced && v.ws_second_staged != nullptr && !explicit_cap && max_edge_len < ccr::kNoPos16;
+  auto fits_staged = [&]() {
+    const int list_area = max_edge_len > 0 ? static_cast<int>(std::min<long long>(ccr::search_bytes(static_cast<int>(max_edge_len), true), kMaxSmemBytes)) : 0;
+    return ccr::WsLayout(kDefaultTileWsRebal, true, list_area, n_req <= ccr::kWsMaxCachedReq ? n_req : 0, 0, ccr::kRebalResolvers, ccr::kRebalSlots,
+                         ccr::kRebalInFlight * 128, ccr::kRebalStreamers * ccr::ws_docs_bytes(s->doc_b), 2).bytes <= kMaxSmemBytes;
+  };
+  const bool staged = rebalanced && v.ws_second_staged != nullptr && !explicit_cap && max_edge_len < ccr::kNoPos16 &&
+                      (s->edge_b >= 128 || (total_cands >= kStagedMinCands && fits_staged()));
   const bool rebal = staged || (rebalanced && v.ws_second_rebal != nullptr);
   // Default split of the 16-warp kernel: 12 streamers + 4 resolvers; over a store whose author ids do not stay in L2
   // (the id array, or the 64-byte id records of a store with engagers, beyond kIdsInL2Bytes) every candidate's id is a trip to HBM and a fifth resolver pays for the

@@ -107,3 +107,20 @@ def test_rows_and_ids_written_by_the_upsert_in_front(edge_dim):
         assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
     assert store.device_status() == B.CCR_OK
     store.free()
+
+
+@pytest.mark.parametrize("total,max_len", [((1 << 20) - 1, 700), (1 << 20, 700), ((1 << 20) + 77, 700), ((1 << 20) + 77, 5_000), ((1 << 20) + 77, 5_100)])
+def test_64_byte_edge_rows_on_both_sides_of_the_rule(total, max_len):
+    """Document rows of 64-byte edge rows are staged from 2^20 candidates on, while a list of the promised length fits beside its table."""
+    from paper_2609_22441_b200 import binding as B
+
+    lengths = [300_000, 33, 0, 200_001, 31, 1]
+    lengths.append(total - sum(lengths))
+    wl = _workload(total + max_len, 32, 0, lengths)
+    want_rows, want_mask = oracle.join_workload(wl, n_threads=8)
+    store, db = B.store_from_workload(wl), B.DeviceBatch(wl.batch)
+    db.max_edge_len = max(db.max_edge_len, max_len)
+    rows, mask = gpu_join(store, db, 0)
+    assert np.array_equal(mask, want_mask) and np.array_equal(rows, want_rows)
+    assert store.device_status() == B.CCR_OK
+    store.free()
