@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
         for (;;) {
           const int s = it % kSlots;
           if (!open) {
-            if (!block && !__all_sync(kFull, mbar_try_wait(full0 + 8 * s, (it / kSlots) & 1u))) return false;
+            if (!block && !__all_sync(kFull, mbar_test_wait(full0 + 8 * s, (it / kSlots) & 1u))) return false;
             if (block && !mbar_wait_bounded(full0 + 8 * s, (it / kSlots) & 1u)) {
               if (lane == 0) atomicExch(a.status, kDevWaitExpired);
               stop = true;

@@ -59,3 +59,9 @@ def test_inputs_are_read_ahead_only_of_a_join_that_is_still_running():
     assert body.count("a.running + blockIdx.x) = 0;") == len(re.findall(r"\breturn;", body))
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "ccr_api.cu")).read())
     assert "a.behind_pads = n_max > 0 ? 1 : 0;" in src and src.count("behind_pads") == 1
+
+
+def test_the_look_at_the_next_sub_tile_does_not_wait():
+    """A streamer that holds a group must not be held back by a sub-tile that is not there yet."""
+    body = _kernel_body("ccr_ws.cuh", "join_ws_kernel")
+    assert "if (!block && !__all_sync(kFull, mbar_test_wait(" in body and "mbar_try_wait(" not in body
