@@ -186,7 +186,7 @@ size_t ccr_out_row_bytes(const ccr_docstore* store, uint32_t flags);
  * Back-to-back joins.  Both join kernels are launched with programmatic stream serialization.  The two-phase kernel (the
  * default for ragged launches of at most 131,072 candidates without the cosine section) waits for everything in front of it
  * on `stream` before it reads its inputs: it is in stream order.  The warp-specialised kernel reads ahead: when the work in
- * front of it is another warp-specialised join of the same store, its blocks take over each SM as soon as that join's block
+ * front of it is another warp-specialised join, its blocks take over each SM as soon as that join's block
  * there has retired and read some of their own inputs (offsets, keys, positions, ids, member embeddings; in a padded call also beside
  * the pads of that call) while the earlier join drains; they read no feature rows and write nothing — rows, mask — before the
  * earlier join has completed, so reusing the output buffers of the previous call is safe.  A block finds out on the device

@@ -60,7 +60,6 @@ constexpr size_t kStageBytes = 16u << 20;  // staging block of second-degree sto
 constexpr size_t kKernelCopyBytes = 16u << 20;
 constexpr int kHostGroups = CCR_HOST_GROUPS;         // most request groups of a pipelined host-buffer join
 constexpr int kSchedRegions = 64;                    // launches of one store that may be in flight at once
-constexpr int kLastJoins = 8;                        // streams of a store whose last join is known
 constexpr int kStatusHead = 4;                       // [0] wait expiry, [1] validation code; then the scheduling words:
                                                      // kSchedRegions regions of sched_stride ints
 
@@ -103,16 +102,6 @@ struct ccr_docstore {
   int64_t dbg_shrink_rows;             // bounds-checked build: rows cut off the registered output extents
   std::atomic<int64_t> launches;  // kernels launched for this store; also hands out the scheduling-word pairs
   std::atomic<int64_t> sort_calls;  // chunked ccr_sort_edges calls; hands out their flag words
-  // the last warp-specialised join of each of a few streams (the oldest entry makes room), for the next one's look at what is in front
-  struct LastJoin {
-    cudaStream_t stream;
-    unsigned long long capture;  // the capture it became part of; 0: launched
-    int ticket;                  // 0: no entry
-  };
-  std::mutex last_joins_mutex;
-  LastJoin last_joins[kLastJoins];
-  int last_joins_next;
-  int* running;  // device: kSchedRegions x n_sms words (JoinArgs::running)
 };
 
 struct ccr_workspace {
@@ -377,43 +366,60 @@ ccr_status dbg_finish(int* word, cudaStream_t st) {
 }
 #endif
 
-// The capture that launches on `st` become part of (0: none; kNoCapture: cannot be told).  A ticket of a launch outside of it, or of
-// another capture, says nothing about what a replay finds in front.
-constexpr unsigned long long kNoCapture = ~0ull;
-unsigned long long capture_of(cudaStream_t st) {
-  if (st == cudaStreamPerThread) return kNoCapture;  // one handle, another stream for every thread
+// What a launch on a stream becomes part of: the stream and the capture, 0 if none.  A ticket of a launch outside of a capture, or of
+// another one, says nothing about what a replay finds in front.  (A handle is not handed out again before the work of the stream it stood
+// for is done.  cudaStreamPerThread is another stream for every thread: unknown.)
+struct StreamOrder {
+  int device;
+  cudaStream_t stream;
+  unsigned long long capture;
+  bool operator==(const StreamOrder& o) const { return device == o.device && stream == o.stream && capture == o.capture; }
+};
+bool stream_order(int device, cudaStream_t st, StreamOrder* out) {
+  if (st == cudaStreamPerThread) return false;
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-  unsigned long long id = 0;
-  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+  *out = {device, st, 0};
+  if (cudaStreamGetCaptureInfo(st, &status, &out->capture) != cudaSuccess) {
     cudaGetLastError();
-    return kNoCapture;
+    return false;
   }
-  return status == cudaStreamCaptureStatusNone ? 0 : id;
+  if (status == cudaStreamCaptureStatusNone) out->capture = 0;
+  return true;
 }
 
-int last_join(ccr_docstore* s, cudaStream_t st, unsigned long long capture) {
-  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
-  for (const auto& e : s->last_joins)
-    if (e.ticket != 0 && e.stream == st && e.capture == capture && capture != kNoCapture) return e.ticket;
-  return 0;
+// The last warp-specialised join of a stream, for the next one's look at what is in front of it, whichever stores the two belong to.  A
+// fixed number of streams is known; the oldest entry makes room, and a join on a stream without one waits.
+struct LastJoin {
+  StreamOrder at;
+  unsigned ticket;  // 0: none
+};
+constexpr int kLastJoins = 32;
+std::mutex g_last_joins_mutex;
+LastJoin g_last_joins[kLastJoins] = {};
+int g_last_joins_next = 0;
+std::atomic<uint32_t> g_tickets{0};
+
+LastJoin* find_last_join(const StreamOrder& at) {
+  for (auto& e : g_last_joins)
+    if (e.ticket != 0 && e.at == at) return &e;
+  return nullptr;
 }
 
-void forget_last_join(ccr_docstore* s, cudaStream_t st) {
-  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
-  for (auto& e : s->last_joins)
-    if (e.stream == st) e.ticket = 0;
+unsigned last_join(const StreamOrder& at) {
+  std::lock_guard<std::mutex> lock(g_last_joins_mutex);
+  const LastJoin* e = find_last_join(at);
+  return e != nullptr ? e->ticket : 0u;
 }
 
-void set_last_join(ccr_docstore* s, cudaStream_t st, unsigned long long capture, int ticket) {
-  std::lock_guard<std::mutex> lock(s->last_joins_mutex);
-  ccr_docstore::LastJoin* to = nullptr;
-  for (auto& e : s->last_joins)
-    if (e.stream == st) to = &e;
-  if (to == nullptr) {
-    to = &s->last_joins[s->last_joins_next];
-    s->last_joins_next = (s->last_joins_next + 1) % kLastJoins;
+void set_last_join(const StreamOrder& at, unsigned ticket) {  // 0: forget it
+  std::lock_guard<std::mutex> lock(g_last_joins_mutex);
+  LastJoin* e = find_last_join(at);
+  if (e == nullptr) {
+    if (ticket == 0) return;
+    e = &g_last_joins[g_last_joins_next];
+    g_last_joins_next = (g_last_joins_next + 1) % kLastJoins;
   }
-  *to = {st, capture, ticket};
+  *e = {at, ticket};
 }
 
 // Launch of a kernel that belongs to a chain of small launches (its first statement is chain_enter()): with
@@ -601,8 +607,6 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
   const size_t status_ints = kStatusHead + static_cast<size_t>(kSchedRegions) * s->sched_stride;
   ok = ok && cudaMalloc(&s->status, status_ints * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMemset(s->status, 0, status_ints * sizeof(int)) == cudaSuccess;
-  const size_t running_bytes = static_cast<size_t>(kSchedRegions) * s->n_sms * sizeof(int);
-  ok = ok && cudaMalloc(&s->running, running_bytes) == cudaSuccess && cudaMemset(s->running, 0, running_bytes) == cudaSuccess;
   ok = ok && cudaHostAlloc(&s->status_host, 4 * sizeof(int), cudaHostAllocDefault) == cudaSuccess;
   ccr_status st = ok ? allow_large_smem() : CCR_ERR_OOM;
   if (st != CCR_OK) {
@@ -612,7 +616,6 @@ ccr_status ccr_docstore_create(const ccr_docstore_desc* d, ccr_docstore** out) {
     cudaFree(s->id_recs);
     cudaFree(s->stage);
     cudaFree(s->status);
-    cudaFree(s->running);
     if (s->status_host) cudaFreeHost(s->status_host);
     delete s;
     return st;
@@ -632,7 +635,6 @@ ccr_status ccr_docstore_free(ccr_docstore* s) {
   cudaFree(s->id_recs);
   cudaFree(s->stage);
   cudaFree(s->status);
-  cudaFree(s->running);
   cudaFreeHost(s->status_host);
   delete s;
   return CCR_OK;
@@ -746,7 +748,8 @@ ccr_status ccr_docstore_upsert(ccr_docstore* s, int64_t n, const int32_t* positi
   long long blocks = (work + per_block - 1) / per_block;
   const long long cap = static_cast<long long>(s->n_sms) * 8;
   blocks = blocks < 1 ? 1 : (blocks > cap ? cap : blocks);
-  forget_last_join(s, static_cast<cudaStream_t>(stream));  // (it need not look for a join that has long completed)
+  StreamOrder at;
+  if (stream_order(s->desc.device, static_cast<cudaStream_t>(stream), &at)) set_last_join(at, 0);  // the next join need not look for one
   launch_chained(ccr::upsert_kernel, dim3(static_cast<unsigned>(blocks)), dim3(ccr::kUpsertThreads), 0, static_cast<cudaStream_t>(stream), a);
   s->launches++;
   if (cudaGetLastError() != cudaSuccess) return CCR_ERR_CUDA;
@@ -1408,12 +1411,10 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
     // (the pair is drawn from the atomic launch counter, so host threads that join against one store at the
     // same time never share a pair)
     const int64_t seq = s->launches.fetch_add(1);
-    a.n_words = s->n_sms;
-    a.running = s->running + (seq % kSchedRegions) * s->n_sms;
-    a.ticket = static_cast<int>(static_cast<uint32_t>(seq) | 0x80000000u);
-    const unsigned long long capture = capture_of(st);
-    a.front_ticket = last_join(s, st, capture);
-    a.front_running = a.front_ticket != 0 ? s->running + (static_cast<uint32_t>(a.front_ticket) % kSchedRegions) * s->n_sms : nullptr;
+    StreamOrder at;
+    const bool known = stream_order(s->desc.device, st, &at);
+    a.ticket = g_tickets.fetch_add(1) | 0x80000000u;
+    a.front_ticket = known ? last_join(at) : 0u;
     a.behind_pads = n_max > 0 ? 1 : 0;
     if (dynamic) a.sched = sched_override ? sched_override : s->status + kStatusHead + s->sched_stride * static_cast<int>(seq % kSchedRegions);
     // Launched with programmatic stream serialization: behind another join on the same stream the blocks become
@@ -1434,7 +1435,7 @@ ccr_status join_impl(const ccr_docstore* cs, int32_t n_req, int64_t total_cands,
       cudaGetLastError();
       return CCR_ERR_CUDA;
     }
-    set_last_join(s, st, capture, a.ticket);
+    if (known) set_last_join(at, a.ticket);
   } else {
     // persistent two-phase kernel: as many blocks as stay resident, each with at least 64 candidates (a single
     // small request is spread over many SMs: 21.6 against 23.4 us for 1,000 candidates with 256 per block)

@@ -73,11 +73,9 @@ struct JoinArgs {
   int warp_search;            // searches that run in global memory use the warp-cooperative 32-ary search (comparison aid)
   int* status;                // device status words
   int* sched;                 // two scheduling words (next tile, finished blocks), zero between launches; or null
-  // reading ahead (warp-specialised kernel): a word per block that holds the launch's ticket while the block runs
-  int* running;
-  const int* front_running;   // the same words of the last such launch on this stream; null: none
-  int ticket, front_ticket;   // never 0
-  int n_words;                // words of a launch
+  // reading ahead (warp-specialised kernel, g_running in ccr_ws.cuh)
+  unsigned ticket;            // of this launch, never 0
+  unsigned front_ticket;      // of the last such launch on this stream; 0: none
   int behind_pads;            // the launch in front writes the pads of this call's output
 };
 

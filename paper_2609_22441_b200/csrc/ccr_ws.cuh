@@ -136,12 +136,22 @@ struct WsLayout {
 // that was launched last on this stream is still running (some block of it shows its ticket), so nothing has run between the two; or
 // the launch in front writes the pads of this call's output, which has waited itself for what is in front of it.  The end of any other
 // kernel is no point at which its writes are promised to be visible to a launch that has not waited.  Reading ahead is worth 6 us of 207
-// (64 x 30,000) and 8 of 292 (second degree) to joins back to back, the look itself costs up to 0.5 us; where nothing is running in front, the wait costs nothing.
-__device__ __forceinline__ bool may_read_ahead(const JoinArgs& a) { return a.front_running != nullptr || a.behind_pads != 0; }
+// (64 x 30,000) and 8 of 292 (second degree) to joins back to back, of one store or of several, the look itself costs up to 0.5 us; where
+// nothing is running in front, the wait costs nothing.  The words are the device's, not a store's: the store of the join in front may be
+// another one.  A word is its launch's from the block's start to its end; a launch kRunLaunches later may take it over, and then the
+// ticket is not found.
+constexpr unsigned kRunLaunches = 256, kRunBlocks = 256;
+static __device__ unsigned g_running[kRunLaunches * kRunBlocks];
+
+__device__ __forceinline__ void show_ticket(const JoinArgs& a, unsigned v) {
+  if (blockIdx.x < kRunBlocks) *const_cast<volatile unsigned*>(g_running + (a.ticket % kRunLaunches) * kRunBlocks + blockIdx.x) = v;
+}
+__device__ __forceinline__ bool may_read_ahead(const JoinArgs& a) { return a.front_ticket != 0 || a.behind_pads != 0; }
 __device__ __forceinline__ bool join_in_front(const JoinArgs& a) {  // (this thread's share of the words)
   bool running = a.behind_pads != 0;
-  if (a.front_running != nullptr) {
-    for (int i = threadIdx.x; i < a.n_words; i += blockDim.x) running |= *reinterpret_cast<const volatile int*>(a.front_running + i) == a.front_ticket;
+  if (a.front_ticket != 0) {
+    for (unsigned i = threadIdx.x; i < kRunBlocks; i += blockDim.x)
+      running |= *const_cast<volatile unsigned*>(g_running + (a.front_ticket % kRunLaunches) * kRunBlocks + i) == a.front_ticket;
   }
   return running;
 }
@@ -195,7 +205,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   if (n_req_cached > 0) mirror_offsets();  // beside the look at the join in front; read once more if that turns out not to be running
   const bool in_front = join_in_front(a);
   if (tid == 0) {
-    *reinterpret_cast<volatile int*>(a.running + blockIdx.x) = a.ticket;
+    show_ticket(a, a.ticket);
     grab[2] = 0;  // streamers that have left
     mbar_init(bar, 1);
     for (int s = 0; s < kSlots; ++s) {
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
   const long long slice0 = min(a.total, static_cast<long long>(blockIdx.x) * per * 32);
   const long long slice1 = min(a.total, slice0 + per * 32);
   if (a.sched == nullptr && slice0 >= slice1) {  // block-uniform, before any named barrier
-    if (tid == 0) *reinterpret_cast<volatile int*>(a.running + blockIdx.x) = 0;
+    if (tid == 0) show_ticket(a, 0u);
     pdl_wait();  // (a launch never completes before the one in front of it)
     return;
   }
@@ -367,7 +377,7 @@ __global__ void __launch_bounds__(REBAL ? kRebalThreads : kWsMaxThreads, 1) join
     }
     // (the block counts as running up to here: joins that follow read ahead only while some block of this one does)
     __syncwarp();
-    if (lane == 0 && atomicAdd(grab + 2, 1) == n_streamers - 1) *reinterpret_cast<volatile int*>(a.running + blockIdx.x) = 0;
+    if (lane == 0 && atomicAdd(grab + 2, 1) == n_streamers - 1) show_ticket(a, 0u);
     pdl_wait();  // also of a block that had nothing to store or gave up: a launch never completes before the one in front of it
     return;
   }

@@ -159,3 +159,35 @@ def test_positions_written_between_two_joins_on_many_streams_and_in_graphs(secon
         assert np.array_equal(buf["mask"].cpu().numpy(), want_mask) and np.array_equal(buf["rows"].cpu().numpy(), want_rows)
     assert store.device_status() == B.CCR_OK
     store.free()
+
+
+def test_joins_of_two_stores_in_turn_with_an_upsert_into_one_of_them():
+    """The join in front may be another store's.  Rows and ids of the second store change between the joins of a round."""
+    from paper_2609_22441_b200 import binding as B
+
+    wls = [W.config1(seed=40 + i, n_docs=60_000, n_req=8, n_cand=20_000) for i in range(2)]
+    stores, dbs = [B.store_from_workload(wl) for wl in wls], [B.DeviceBatch(wl.batch) for wl in wls]
+    s, b = wls[1].store, wls[1].batch
+    rng = np.random.default_rng(2)
+    pos = rng.permutation(s.n_docs).astype(np.int32)
+    news = [(rng.standard_normal(s.doc_feats.shape).astype(s.doc_feats.dtype), rng.permutation(s.author_ids)) for _ in range(2)]
+    wants = []
+    for doc, auth in news:
+        st = oracle.upsert(s.doc_feats.copy(), s.author_ids.copy(), pos.astype(np.int64), doc, auth)
+        wants.append(oracle.join(st[0], st[1], b.edge_keys, b.edge_feats, b.edge_offsets, b.cand_idx, b.cand_offsets, req_feats=b.req_feats, n_threads=4))
+    want0 = oracle.join_workload(wls[0], n_threads=4)
+    dev = [tuple(torch.from_numpy(a).cuda() for a in (pos, *n)) for n in news]
+    outs = [[torch.zeros((db.total_cands, st.out_row_bytes()), dtype=torch.uint8, device="cuda"), torch.zeros(db.total_cands, dtype=torch.uint8, device="cuda")]
+            for st, db in ((stores[0], dbs[0]), (stores[1], dbs[1]), (stores[1], dbs[1]))]
+    torch.cuda.synchronize()
+    for i in range(30):
+        B.join_batch(stores[0], dbs[0], 0, *outs[0])
+        stores[1].upsert(*dev[i % 2])
+        B.join_batch(stores[1], dbs[1], 0, *outs[1 + i % 2])
+        B.join_batch(stores[0], dbs[0], 0, *outs[0])
+    torch.cuda.synchronize()
+    for (rows, mask), (want_rows, want_mask) in zip(outs, [want0] + wants):
+        assert np.array_equal(mask.cpu().numpy(), want_mask) and np.array_equal(rows.cpu().numpy(), want_rows)
+    for st in stores:
+        assert st.device_status() == B.CCR_OK
+        st.free()

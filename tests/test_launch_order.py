@@ -54,9 +54,9 @@ def test_inputs_are_read_ahead_only_of_a_join_that_is_still_running():
     assert "if (!may_read_ahead(a)) pdl_wait();" in early and early.index("may_read_ahead") < early.index("mirror_offsets();  ".strip())
     # in front of it only the offsets are read, past L1, and they are read again
     assert not re.search(r"\bgload\(|\bstage_keys\b|\ba\.(cand_idx|edge_keys|sched)\s*[+\[]", early)
-    assert early.index("a.running + blockIdx.x) = a.ticket;") > 0
+    assert early.index("show_ticket(a, a.ticket);") > 0
     assert body.count("pdl_trigger()") == 1 and "pdl_trigger()" in behind
-    assert body.count("a.running + blockIdx.x) = 0;") == len(re.findall(r"\breturn;", body))
+    assert body.count("show_ticket(a, 0u);") == len(re.findall(r"\breturn;", body))
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "ccr_api.cu")).read())
     assert "a.behind_pads = n_max > 0 ? 1 : 0;" in src and src.count("behind_pads") == 1
 
