@@ -1131,7 +1131,7 @@ def main():
                                          "elements 8..57 of the document row, 32 more bytes per output row; e2e and latency legs "
                                          "run without it")
         if args.padded:
-            line["config"]["layout"] = ("padded T[%d, %d]: a step is ccr_compact_valid (3 launches, %.1f us alone, L2-warm) + "
+            line["config"]["layout"] = ("padded T[%d, %d]: a step is ccr_compact_valid (2 launches, %.1f us alone, L2-warm) + "
                                         "pad fill + join; the roofline figure divides the join's bytes by the whole step"
                                         % (db.n_req, db.n_max_cands, compact_us))
         if world == 1 and not args.no_cpu_baseline and not args.timed_only:

@@ -66,7 +66,8 @@ struct ResolveArgs {
   int32_t* out_pos;
 };
 
-// Every bit of the id reaches the high bits, whatever regular pattern the ids follow (xor-shift and multiply, twice).
+// Every bit of the id reaches the high bits, whatever regular pattern the ids follow: xor-shift and multiply, twice, with the multiplier of
+// the public 64-bit mixer known as degski64 (in C. Wellons's hash-prospector collection).
 __device__ __forceinline__ unsigned id_bucket(int64_t id, unsigned n_buckets) {
   unsigned long long h = static_cast<unsigned long long>(id);
   h = (h ^ (h >> 32)) * 0xD6E8FEB86659FD93ull;
